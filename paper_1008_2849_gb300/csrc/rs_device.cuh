@@ -46,10 +46,15 @@ struct Ctrl {
     uint32_t tile_ctr[PLAN_SLOTS]; // dynamic tile ids, one counter per plan slot
     uint32_t dir[PLAN_SLOTS];      // pass plan
     uint32_t seg_tiles;            // segmented sorts: tiles of the large segments
-    uint32_t small_count;          // segmented sorts (and MSD buckets): one-CTA segments
-    uint32_t large_count;          // segmented sorts: number of large segments
-    uint32_t tiny_count;           // segmented sorts (and MSD buckets): one-warp segments
-    uint32_t pad[9];               // keep hist 64-byte aligned
+    // Segmented sorts (and MSD buckets): the segments listed for the one-CTA
+    // sorts by size (see list_small), for the one-warp sort, and the number of
+    // large ones.
+    uint32_t small_count;
+    uint32_t mid_count;
+    uint32_t big_count;
+    uint32_t large_count;
+    uint32_t tiny_count;
+    uint32_t pad[7];               // keep hist 64-byte aligned
     uint32_t hist[PASSES64][RADIX];  // digit histograms (H); 0..3 for 32-bit keys
     uint32_t gofs[PASSES64][RADIX];  // first output slot of every bucket (G)
 };

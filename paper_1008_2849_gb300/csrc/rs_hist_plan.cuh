@@ -191,15 +191,13 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
 // alternate buffers) and skips passes 0..3; every bucket is then sorted on
 // chip from the alternate buffers back into the caller's arrays (its digit 3
 // is constant, so that pass is trivial there).  msd_off[b] is bucket b's
-// first slot (msd_off[256] = n); non-empty buckets of at most warp_max keys
-// are listed in tiny_list (one-warp sort), larger ones in small_list
-// (one-CTA sort).
+// first slot (msd_off[256] = n), and small_count becomes the number of buckets
+// to sort (0 when the plan chooses the passes 0..3).
 // ---------------------------------------------------------------------------
 template <int NPASS>
 __global__ void __launch_bounds__(1024)
-k_plan(Ctrl* __restrict__ ctrl, uint32_t n, uint32_t msd_allowed, uint32_t warp_max,
-       uint32_t bucket_cap, uint32_t* __restrict__ msd_off, uint32_t* __restrict__ tiny_list,
-       uint32_t* __restrict__ small_list) {
+k_plan(Ctrl* __restrict__ ctrl, uint32_t n, uint32_t msd_allowed, uint32_t bucket_cap,
+       uint32_t* __restrict__ msd_off) {
     static_assert(NPASS == 4 || NPASS == 8, "32-bit or 64-bit keys");
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_trivial[NPASS];
@@ -211,7 +209,7 @@ k_plan(Ctrl* __restrict__ ctrl, uint32_t n, uint32_t msd_allowed, uint32_t warp_
     if (tid < NPASS) s_trivial[tid] = 0;
     if (tid == 0) s_big = 0;
     // Thread (p, b): p = tid / 256 (+ 4 in the second round for 64-bit keys).
-    uint32_t h3 = 0, first3 = 0;  // digit 3, for the MSD-first order
+    uint32_t first3 = 0;  // digit 3, for the MSD-first order
     for (uint32_t round = 0; round < NPASS / 4; ++round) {
         const uint32_t p = (tid >> 8) + 4 * round;
         const uint32_t h = ctrl->hist[p][b];
@@ -229,7 +227,6 @@ k_plan(Ctrl* __restrict__ ctrl, uint32_t n, uint32_t msd_allowed, uint32_t warp_
         ctrl->gofs[p][b] = first;
         if (h == n) s_trivial[p] = 1;
         if (p == PASSES - 1) {
-            h3 = h;
             first3 = first;
             if (h > bucket_cap) s_big = 1;
         }
@@ -239,16 +236,11 @@ k_plan(Ctrl* __restrict__ ctrl, uint32_t n, uint32_t msd_allowed, uint32_t warp_
     if (msd && (tid >> 8) == PASSES - 1) {
         msd_off[b] = first3;
         if (b == RADIX - 1) msd_off[RADIX] = n;
-        if (h3 > 0) {
-            if (h3 <= warp_max)
-                tiny_list[atomicAdd(&ctrl->tiny_count, 1u)] = b;
-            else
-                small_list[atomicAdd(&ctrl->small_count, 1u)] = b;
-        }
     }
     if (tid == 0 && msd) {
         for (uint32_t q = 0; q < PASSES; ++q) ctrl->dir[q] = DIR_SKIP;
         ctrl->dir[MSD_SLOT] = DIR_A_TO_B;
+        ctrl->small_count = RADIX;
     } else if (tid == 0) {
         ctrl->dir[MSD_SLOT] = DIR_SKIP;
         uint32_t trivial[NPASS], executed = 0;

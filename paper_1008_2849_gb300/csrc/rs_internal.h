@@ -119,7 +119,7 @@ rs_status device_info(DeviceInfo* out);
 
 // Workspace layout of an unsegmented sort of n items.
 struct Layout {
-    size_t ctrl, status0, status1, alt_keys, alt_vals, msd_off, msd_tiny, msd_small, total;
+    size_t ctrl, status0, status1, alt_keys, alt_vals, msd_off, total;
     uint32_t tiles;          // tiles of the smallest tile shape (status sizing)
     bool wide_status;        // 64-bit status words (n >= 2^30)
 };
@@ -201,16 +201,25 @@ rs_status launch_onesweep_pairs(int cfg, bool wide, uint32_t* ka, uint32_t* va, 
                                 Ctrl* ctrl, uint32_t* sticky, void* status, void* status_clear,
                                 const SegView* seg, uint32_t key_type, cudaStream_t stream);
 
-// One-CTA sort in shared memory: of every small segment listed by the
-// segmented planner (off != nullptr; none longer than max_items), or of the
-// single array [0, single_n) with single_n <= max_items <= small_sort_capacity().
-// bits: digit width, 4 or 8.
-// src_keys / src_vals (default: keys / vals, in place) is where items are read.
-rs_status launch_small_sort(uint32_t* keys, uint32_t* vals, const uint32_t* off,
-                            const uint32_t* small_list, const Ctrl* ctrl, uint32_t single_n,
-                            uint32_t max_items, int bits, uint32_t key_type, cudaStream_t stream,
-                            const uint32_t* src_keys = nullptr,
-                            const uint32_t* src_vals = nullptr);
+// One-CTA sorts on chip of those of the segments 0 .. *count - 1 that hold 1 to
+// small_sort_capacity() items (count on the device): a CTA of one size for those
+// of up to `usual` items, a larger one for the rest.  bits: 8, the bin sort
+// (rs_bin_sort.cuh); 4, eight counting passes of 4-bit digits.  Items are read
+// from src_keys / src_vals.
+rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
+                              const uint32_t* src_vals, const uint32_t* off,
+                              const uint32_t* count, const Ctrl* ctrl, uint32_t usual, int bits,
+                              uint32_t key_type, cudaStream_t stream);
+// The segments listed by size (rs_bin_sort.cuh list_small) in tiny_list and
+// small_list of `entries` entries each, in place: one launch per size up to
+// max_items.
+rs_status launch_small_lists(uint32_t* keys, uint32_t* vals, const uint32_t* off,
+                             const uint32_t* tiny_list, const uint32_t* small_list,
+                             uint32_t entries, const Ctrl* ctrl, uint32_t max_items, int bits,
+                             uint32_t key_type, cudaStream_t stream);
+// The same sort of the single array [0, n), n <= small_sort_capacity().
+rs_status launch_single_sort(uint32_t* keys, uint32_t* vals, uint32_t n, int bits,
+                             uint32_t key_type, cudaStream_t stream);
 uint32_t small_sort_capacity();
 
 // One-warp sort in shared memory: of every tiny segment listed by the

@@ -91,8 +91,8 @@ rs_status enqueue_sort_segmented(uint32_t* keys, uint32_t* vals, uint32_t n,
                               stream);
         if (st != RS_OK) return st;
     }
-    st = launch_small_sort(keys, vals, offsets, small_list, ctrl, 0, small_max, ck.small_bits,
-                           key_type, stream);
+    st = launch_small_lists(keys, vals, offsets, tiny_list, small_list, num_segments, ctrl,
+                            small_max, ck.small_bits, key_type, stream);
     if (st != RS_OK) return st;
 
     // Large segments: histograms, bucket bases, four scatter passes.

@@ -5,9 +5,9 @@
 // per segment).  Segments are routed by size (rs_small.cuh has the first two):
 //   tiny (2 <= size <= warp_max): k_warp_sort, one warp per segment, the whole
 //       segment in that warp's shared memory for every pass;
-//   small (warp_max < size <= small_max): k_small_sort, one CTA per segment,
-//       the whole segment in shared memory -- one read and one write of every
-//       item either way;
+//   small (warp_max < size <= small_max): k_bin_sort (rs_bin_sort.cuh), one CTA
+//       per segment, the whole segment on chip -- one read and one write of
+//       every item either way;
 //   large (size > small_max): the scatter passes of the unsegmented sort
 //       (k_onesweep<..., SEG>) over tiles that never straddle a segment, after
 //       k_seg_hist (per-segment digit histograms) and k_seg_scan (per-segment
@@ -15,6 +15,7 @@
 // k_seg_plan validates the table and lays the work out.
 #pragma once
 
+#include "rs_bin_sort.cuh"
 #include "rs_device.cuh"
 
 namespace rs {
@@ -27,8 +28,7 @@ namespace rs {
 //  - Large segments get consecutive tile ids (in segment order) and a dense
 //    ordinal; tile_geo[t] = (first item, item count, first tile of its
 //    segment, ordinal of its segment).
-//  - Tiny segments are listed in tiny_list, small ones in small_list (order
-//    irrelevant).
+//  - Tiny and small segments are listed by size (list_small; order irrelevant).
 //  - The pass plan runs all npass passes (four, or eight for 64-bit keys;
 //    caller -> alternate -> ... -> caller).
 // ---------------------------------------------------------------------------
@@ -69,12 +69,8 @@ k_seg_plan(const uint32_t* __restrict__ off, uint32_t num_segments, uint32_t n, 
         }
         const bool large = size > small_max;
         const uint32_t ntiles = large ? (size + tile - 1) / tile : 0u;
-        if (s < num_segments && !large && size >= 2) {
-            if (size <= warp_max)
-                tiny_list[atomicAdd(&ctrl->tiny_count, 1u)] = s;
-            else
-                small_list[atomicAdd(&ctrl->small_count, 1u)] = s;
-        }
+        if (s < num_segments && !large && size >= 2)
+            list_small(ctrl, s, size, warp_max, num_segments - 1, tiny_list, small_list);
         // Block-wide exclusive scans of (tiles, large flag), packed as two
         // 32-bit halves of one 64-bit sum.
         unsigned long long v = ((unsigned long long)ntiles << 32) | (large ? 1u : 0u);

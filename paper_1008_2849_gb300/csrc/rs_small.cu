@@ -1,44 +1,92 @@
 // rs_small.cu -- host launchers of the on-chip sorts (rs_small.cuh): the
 // one-warp sort and the one-CTA sort, each at digit width 4 or 8.
+#include <type_traits>
+
 #include "rs_internal.h"
+#include "rs_bin_sort.cuh"
 #include "rs_small.cuh"
 
 namespace rs {
 
 namespace {
 
-// One-CTA sort shapes: 256 threads x 16 items (4096) and 512 x 16 (8192).
-template <int THREADS, int ITEMS, int BITS, bool PAIRS>
-rs_status launch_small_shape(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
-                             const uint32_t* src_vals, const uint32_t* off,
-                             const uint32_t* list, const Ctrl* ctrl, uint32_t single_n,
-                             uint32_t grid, uint32_t key_type, cudaStream_t stream) {
-    constexpr uint32_t CAP = THREADS * ITEMS;
-    constexpr size_t SMEM =
-        ((PAIRS ? 4u : 2u) * CAP + (THREADS / 32) * (1u << BITS)) * sizeof(uint32_t);
-    auto kern = k_small_sort<THREADS, ITEMS, BITS, PAIRS>;
-    static DeviceOnce smem_set;
-    rs_status st = allow_smem_once(kern, SMEM, smem_set);
-    if (st != RS_OK) return st;
+// What a one-CTA sort works on: arrays listed on the device, or a single one.
+struct SmallWork {
+    uint32_t *keys, *vals;
+    const uint32_t *src_keys, *src_vals, *off, *list;
+    int32_t step;
+    const uint32_t* list_count;
+    const Ctrl* ctrl;
+    uint32_t single_n;  // off == nullptr: the array's items; list == nullptr: see k_bin_sort
+    uint32_t key_type;
+};
+
+// A single array takes one CTA, a list as many as fit the GPU `per_sm` to an SM.
+rs_status grid_of(const SmallWork& w, uint32_t per_sm, uint32_t* grid) {
+    DeviceInfo di;
+    const rs_status st = device_info(&di);
+    if (st == RS_OK) *grid = w.off == nullptr ? 1u : (uint32_t)di.sm_count * per_sm;
+    return st;
+}
+
+template <typename Kern>
+rs_status launch_small_kernel(Kern kern, uint32_t grid, uint32_t threads, size_t smem,
+                              const SmallWork& w, cudaStream_t stream) {
     note_launch_begin(KK_SMALL, stream);
-    const cudaError_t e = launch_after_previous(kern, dim3(grid), dim3(THREADS), SMEM, stream, keys,
-                                                vals, src_keys, src_vals, off, list, ctrl,
-                                                single_n, key_type);
+    const cudaError_t e = launch_after_previous(kern, dim3(grid), dim3(threads), smem, stream,
+                                                w.keys, w.vals, w.src_keys, w.src_vals, w.off,
+                                                w.list, w.step, w.list_count, w.ctrl, w.single_n,
+                                                w.key_type);
     note_launch_end(KK_SMALL, stream);
     return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
 
-template <int BITS, bool PAIRS>
-rs_status launch_small_bits(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
-                            const uint32_t* src_vals, const uint32_t* off,
-                            const uint32_t* list, const Ctrl* ctrl, uint32_t single_n,
-                            uint32_t max_items, uint32_t grid, uint32_t key_type,
+template <bool PAIRS, int THREADS, int ITEMS, int MIN_BLOCKS>
+rs_status launch_bin_shape(const SmallWork& w, cudaStream_t stream) {
+    using L = BinSortSmem<uint32_t, uint32_t, PAIRS, THREADS, ITEMS>;
+    auto kern = k_bin_sort<uint32_t, uint32_t, PAIRS, THREADS, ITEMS, MIN_BLOCKS>;
+    static DeviceOnce smem_set;
+    rs_status st = allow_smem_once(kern, L::BYTES, smem_set);
+    if (st != RS_OK) return st;
+    uint32_t grid = 0;
+    st = grid_of(w, MIN_BLOCKS, &grid);
+    if (st != RS_OK) return st;
+    return launch_small_kernel(kern, grid, THREADS, L::BYTES, w, stream);
+}
+
+template <int THREADS, int ITEMS, bool PAIRS>
+rs_status launch_small_shape4(const SmallWork& w, cudaStream_t stream) {
+    constexpr uint32_t CAP = THREADS * ITEMS;
+    constexpr size_t SMEM = ((PAIRS ? 4u : 2u) * CAP + (THREADS / 32) * 16u) * sizeof(uint32_t);
+    auto kern = k_small_sort<THREADS, ITEMS, 4, PAIRS>;
+    static DeviceOnce smem_set;
+    rs_status st = allow_smem_once(kern, SMEM, smem_set);
+    if (st != RS_OK) return st;
+    uint32_t grid = 0;
+    st = grid_of(w, 4, &grid);
+    if (st != RS_OK) return st;
+    return launch_small_kernel(kern, grid, THREADS, SMEM, w, stream);
+}
+
+// The CTA for arrays of at most max_items items: 128 threads up to 1024, 512 up
+// to 4096, 1024 up to 8192 (eight items a thread).  A single array of up to 1024
+// takes 512 threads: fewer items a thread, a shorter chain.
+template <bool PAIRS>
+rs_status launch_small_size(uint32_t max_items, int bits, const SmallWork& w,
                             cudaStream_t stream) {
-    if (max_items <= 4096)
-        return launch_small_shape<256, 16, BITS, PAIRS>(keys, vals, src_keys, src_vals, off, list,
-                                                        ctrl, single_n, grid, key_type, stream);
-    return launch_small_shape<512, 16, BITS, PAIRS>(keys, vals, src_keys, src_vals, off, list, ctrl,
-                                                    single_n, grid, key_type, stream);
+    if (bits == 4)
+        return max_items <= SMALL_MID_MAX ? launch_small_shape4<256, 16, PAIRS>(w, stream)
+                                          : launch_small_shape4<512, 16, PAIRS>(w, stream);
+    if (max_items <= SMALL_SHORT_MAX && w.off != nullptr)
+        return launch_bin_shape<PAIRS, 128, 8, 10>(w, stream);
+    if (max_items <= SMALL_MID_MAX) return launch_bin_shape<PAIRS, 512, 8, 3>(w, stream);
+    return launch_bin_shape<PAIRS, 1024, 8, 1>(w, stream);
+}
+
+rs_status launch_small_any(uint32_t max_items, int bits, const SmallWork& w,
+                           cudaStream_t stream) {
+    return w.vals != nullptr ? launch_small_size<true>(max_items, bits, w, stream)
+                             : launch_small_size<false>(max_items, bits, w, stream);
 }
 
 template <int BITS, bool PAIRS>
@@ -64,28 +112,53 @@ rs_status launch_warp_bits(uint32_t* keys, uint32_t* vals, const uint32_t* src_k
 uint32_t small_sort_capacity() { return 8192; }
 uint32_t warp_sort_capacity() { return 32 * WARP_SORT_ITEMS; }
 
-rs_status launch_small_sort(uint32_t* keys, uint32_t* vals, const uint32_t* off,
-                            const uint32_t* small_list, const Ctrl* ctrl, uint32_t single_n,
-                            uint32_t max_items, int bits, uint32_t key_type, cudaStream_t stream,
-                            const uint32_t* src_keys, const uint32_t* src_vals) {
-    if (max_items > small_sort_capacity()) return RS_ERR_INVALID_ARG;
-    DeviceInfo di;
-    rs_status st = device_info(&di);
-    if (st != RS_OK) return st;
-    // Single array: one CTA.  Segment list: a grid-stride loop over it.
-    const uint32_t grid = off == nullptr ? 1u : (uint32_t)di.sm_count * 4u;
-    const bool pairs = vals != nullptr;
-    const uint32_t* sk = src_keys ? src_keys : keys;
-    const uint32_t* sv = src_keys ? src_vals : vals;
-    if (bits == 4)
-        return pairs ? launch_small_bits<4, true>(keys, vals, sk, sv, off, small_list, ctrl,
-                                                  single_n, max_items, grid, key_type, stream)
-                     : launch_small_bits<4, false>(keys, vals, sk, sv, off, small_list, ctrl,
-                                                   single_n, max_items, grid, key_type, stream);
-    return pairs ? launch_small_bits<8, true>(keys, vals, sk, sv, off, small_list, ctrl, single_n,
-                                              max_items, grid, key_type, stream)
-                 : launch_small_bits<8, false>(keys, vals, sk, sv, off, small_list, ctrl, single_n,
-                                               max_items, grid, key_type, stream);
+rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
+                              const uint32_t* src_vals, const uint32_t* off,
+                              const uint32_t* count, const Ctrl* ctrl, uint32_t usual, int bits,
+                              uint32_t key_type, cudaStream_t stream) {
+    SmallWork w{keys, vals, src_keys, src_vals, off, nullptr, 1, count, ctrl, 0, key_type};
+    // (The 4-bit sorts have no CTA for up to SMALL_SHORT_MAX items: one launch.)
+    const uint32_t sizes[] = {bits == 4 || usual > SMALL_MID_MAX ? small_sort_capacity()
+                              : usual > SMALL_SHORT_MAX          ? SMALL_MID_MAX
+                                                                 : SMALL_SHORT_MAX,
+                              small_sort_capacity()};
+    for (const uint32_t size : sizes) {
+        const rs_status st = launch_small_any(size, bits, w, stream);
+        if (st != RS_OK || size == small_sort_capacity()) return st;
+        w.single_n = size;  // the larger CTA takes the buckets above
+    }
+    return RS_OK;
+}
+
+rs_status launch_small_lists(uint32_t* keys, uint32_t* vals, const uint32_t* off,
+                             const uint32_t* tiny_list, const uint32_t* small_list,
+                             uint32_t entries, const Ctrl* ctrl, uint32_t max_items, int bits,
+                             uint32_t key_type, cudaStream_t stream) {
+    const struct {
+        const uint32_t* list;
+        int step;
+        const uint32_t* count;
+        uint32_t below, max;
+    } sizes[] = {
+        {small_list, 1, &ctrl->small_count, 0, SMALL_SHORT_MAX},
+        {small_list + entries - 1, -1, &ctrl->mid_count, SMALL_SHORT_MAX, SMALL_MID_MAX},
+        {tiny_list + entries - 1, -1, &ctrl->big_count, SMALL_MID_MAX, small_sort_capacity()},
+    };
+    for (const auto& c : sizes) {
+        if (max_items <= c.below) break;
+        const SmallWork w{keys, vals, keys, vals, off, c.list, c.step, c.count, ctrl, 0,
+                          key_type};
+        const rs_status st = launch_small_any(c.max, bits, w, stream);
+        if (st != RS_OK) return st;
+    }
+    return RS_OK;
+}
+
+rs_status launch_single_sort(uint32_t* keys, uint32_t* vals, uint32_t n, int bits,
+                             uint32_t key_type, cudaStream_t stream) {
+    if (n > small_sort_capacity()) return RS_ERR_INVALID_ARG;
+    const SmallWork w{keys, vals, keys, vals, nullptr, nullptr, 1, nullptr, nullptr, n, key_type};
+    return launch_small_any(n, bits, w, stream);
 }
 
 rs_status launch_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* off,

@@ -1,5 +1,6 @@
-// rs_small.cuh -- sorts of arrays that fit in on-chip memory: the one-warp
-// sort (k_warp_sort) and the one-CTA sort (k_small_sort).  Both run the
+// rs_small.cuh -- sorts of arrays that fit in on-chip memory by counting passes:
+// the one-warp sort (k_warp_sort) and the one-CTA sort with 4-bit digits
+// (k_small_sort; the default one-CTA sort is k_bin_sort).  Both run the
 // stable counting-sort passes of Sec. 3 between two shared-memory buffers, so
 // every item is read from and written to global memory once.  The digit width
 // BITS is a template parameter: 8 bits (four passes, 256 buckets, as in the
@@ -157,8 +158,10 @@ k_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uint
 // ---------------------------------------------------------------------------
 // k_small_sort: one CTA sorts a whole array of at most CAP = THREADS * ITEMS
 // items in shared memory: 32 / BITS stable counting-sort passes between two
-// shared buffers.  Arrays are the segments listed in small_list (count in
-// ctrl->small_count), or with off == nullptr the single array [0, single_n).
+// shared buffers.  Arrays are the segments listed from `list` on (every
+// `step`-th entry; count in *list_count), with list == nullptr those of
+// the segments 0, 1, ... that hold more than single_n items and at most CAP, or with off == nullptr the single
+// array [0, single_n).  The 4-bit form only; 8-bit digits take k_bin_sort.
 // Per pass: per-warp digit counts, their prefix over (digit, warp), then every
 // warp ranks its items slot by slot (peers from one ballot per digit bit,
 // positions from the warp's counters) and moves them to the other buffer.  A
@@ -167,8 +170,9 @@ k_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uint
 template <int THREADS, int ITEMS, int BITS, bool PAIRS>
 __global__ void __launch_bounds__(THREADS)
 k_small_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uint32_t* src_vals,
-             const uint32_t* __restrict__ off, const uint32_t* __restrict__ small_list,
-             const Ctrl* __restrict__ ctrl, uint32_t single_n, uint32_t key_type) {
+             const uint32_t* __restrict__ off, const uint32_t* __restrict__ list, int32_t step,
+             const uint32_t* __restrict__ list_count, const Ctrl* __restrict__ ctrl,
+             uint32_t single_n, uint32_t key_type) {
     constexpr uint32_t NB = 1u << BITS;
     constexpr uint32_t NPASS = 32 / BITS;
     constexpr uint32_t NW = (NB + 31) / 32;  // warps holding digit totals
@@ -191,15 +195,16 @@ k_small_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uin
     uint32_t count = 1;
     if (off != nullptr) {
         if (ctrl->err != 0) return;
-        count = ctrl->small_count;
+        count = *list_count;
     }
     for (uint32_t w = tid; w < WARPS * NB; w += THREADS) s_w[w] = 0;
     for (uint32_t idx = blockIdx.x; idx < count; idx += gridDim.x) {
         uint32_t lo = 0, m = single_n;
         if (off != nullptr) {
-            const uint32_t s = small_list[idx];
+            const uint32_t s = list != nullptr ? list[(ptrdiff_t)idx * step] : idx;
             lo = off[s];
             m = off[s + 1] - lo;
+            if (list == nullptr && (m <= single_n || m > CAP)) continue;
         }
         for (uint32_t i = tid; i < m; i += THREADS) {
             s_k[i] = key_to_ordered(src_keys[lo + i], key_type);

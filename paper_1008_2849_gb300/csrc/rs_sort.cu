@@ -37,12 +37,8 @@ Layout layout_for(size_t n, bool pairs) {
     off = align_up(off + n * sizeof(uint32_t), 256);
     L.alt_vals = off;
     if (pairs) off = align_up(off + n * sizeof(uint32_t), 256);
-    L.msd_off = off;  // MSD-first order: bucket offsets and bucket lists
+    L.msd_off = off;  // MSD-first order: bucket offsets
     off = align_up(off + (RADIX + 1) * sizeof(uint32_t), 256);
-    L.msd_tiny = off;
-    off = align_up(off + RADIX * sizeof(uint32_t), 256);
-    L.msd_small = off;
-    off = align_up(off + RADIX * sizeof(uint32_t), 256);
     L.total = off;
     return L;
 }
@@ -149,8 +145,7 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     // A single small array takes one CTA (one warp alone measured slower);
     // the one-warp sort serves batches of short segments and MSD buckets.
     if (n <= (uint32_t)ck.small_max && n <= small_sort_capacity())
-        return launch_small_sort(keys, vals, nullptr, nullptr, nullptr, n, n, ck.small_bits,
-                                 key_type, stream);
+        return launch_single_sort(keys, vals, n, ck.small_bits, key_type, stream);
     // Three passes of 11/11/10-bit digits, where the size class takes them
     // and the caller's workspace holds their buffers.
     if (ck.digits == 11 && key_type == KEY_U32 && workspace_bytes >= layout11(n, pairs).total)
@@ -167,19 +162,14 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     // from the digit-3 histogram, so the launch sequence stays fixed.
     const bool msd = ck.msd != 0 && key_type == KEY_U32 && n <= kMsdMaxItems;
     uint32_t* msd_off = reinterpret_cast<uint32_t*>(ws + L.msd_off);
-    uint32_t* msd_tiny = reinterpret_cast<uint32_t*>(ws + L.msd_tiny);
-    uint32_t* msd_small = reinterpret_cast<uint32_t*>(ws + L.msd_small);
-    const uint32_t warp_max =
-        (uint32_t)ck.warp_max < warp_sort_capacity() ? (uint32_t)ck.warp_max : warp_sort_capacity();
 
     if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
     st = enqueue_hist4(keys, n, &ctrl->hist[0][0], status[0], status_bytes, key_type, stream);
     if (st != RS_OK) return st;
     note_launch_begin(KK_PLAN, stream);
     const cudaError_t pe = launch_after_previous(k_plan<PASSES>, dim3(1), dim3(1024), 0, stream,
-                                                 ctrl, n, msd ? 1u : 0u, warp_max,
-                                                 small_sort_capacity(), msd_off, msd_tiny,
-                                                 msd_small);
+                                                 ctrl, n, msd ? 1u : 0u, small_sort_capacity(),
+                                                 msd_off);
     note_launch_end(KK_PLAN, stream);
     if (pe != cudaSuccess) return RS_ERR_CUDA;
 
@@ -194,13 +184,9 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
                    : launch_onesweep_keys(cfg, false, keys, alt_k, n, PASSES - 1, MSD_SLOT, ctrl,
                                           di.sticky, status[0], nullptr, nullptr, KEY_U32, stream);
         if (st != RS_OK) return st;
-        if (warp_max > 0) {
-            st = launch_warp_sort(keys, vals, msd_off, msd_tiny, ctrl, 0, ck.small_bits, KEY_U32,
-                                  stream, alt_k, alt_v);
-            if (st != RS_OK) return st;
-        }
-        st = launch_small_sort(keys, vals, msd_off, msd_small, ctrl, 0, small_sort_capacity(),
-                               ck.small_bits, KEY_U32, stream, alt_k, alt_v);
+        // (Usual buckets of evenly spread keys hold less than twice the average.)
+        st = launch_bucket_sorts(keys, vals, alt_k, alt_v, msd_off, &ctrl->small_count, ctrl,
+                                 n / RADIX * 2, ck.small_bits, KEY_U32, stream);
         if (st != RS_OK) return st;
     }
     for (uint32_t p = 0; p < PASSES; ++p) {

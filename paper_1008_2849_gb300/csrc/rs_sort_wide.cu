@@ -78,7 +78,7 @@ Layout layout_wide(size_t n, bool key64, uint32_t val_bytes) {
     off = align_up(off + n * (key64 ? 8 : 4), 256);
     L.alt_vals = off;
     off = align_up(off + n * val_bytes, 256);
-    L.msd_off = L.msd_tiny = L.msd_small = off;  // no MSD-first order for wide items
+    L.msd_off = off;  // no MSD-first order for wide items
     L.total = off;
     return L;
 }
@@ -124,12 +124,12 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
         if (st != RS_OK) return st;
     }
     note_launch_begin(KK_PLAN, stream);
-    uint32_t* const no_list = nullptr;
+    uint32_t* const no_buckets = nullptr;
     const cudaError_t pe =
         key64 ? launch_after_previous(k_plan<PASSES64>, dim3(1), dim3(1024), 0, stream, ctrl, n,
-                                      0u, 0u, 0u, no_list, no_list, no_list)
+                                      0u, 0u, no_buckets)
               : launch_after_previous(k_plan<PASSES>, dim3(1), dim3(1024), 0, stream, ctrl, n, 0u,
-                                      0u, 0u, no_list, no_list, no_list);
+                                      0u, no_buckets);
     note_launch_end(KK_PLAN, stream);
     if (pe != cudaSuccess) return RS_ERR_CUDA;
 
