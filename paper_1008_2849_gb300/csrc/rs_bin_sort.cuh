@@ -254,6 +254,7 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 keys[lo + i] = key_from_ordered(s_w[i], key_type);
                 if (PAIRS) vals[lo + i] = s_v[i];
             }
+            __syncthreads();  // shared memory is free for the next array
         } else {
             // ---- digit passes ------------------------------------------------
             // Items stay in registers; a pass moves them to their new slots
