@@ -452,9 +452,13 @@ def main():
     elapsed_ms = max_over_ranks(elapsed_ms, world, dev)
     value = job_throughput(world, args.steps, n, elapsed_ms / 1e3)
 
-    # Roofline of the dominant kernel: the scatter pass.
+    # Roofline of the dominant kernel: the scatter pass.  A launch whose pass the
+    # plan left out returns at once; the passes that ran took tiles (the
+    # workspace's control block: the error word, then tiles taken by passes 0..3).
     peaks, peak_src = measured_peaks()
     os_launches, os_ms = per_kind.get("onesweep", (0, 0.0))
+    passes = int((ws[4:20].cpu().numpy().view(np.uint32) > 0).sum())
+    os_launches = passes * args.steps if os_launches else 0
     hist_launches, hist_ms = per_kind.get("hist4", (0, 0.0))
     algo_bytes = roofline.scatter_bytes_per_item(True) * n   # per scatter launch
     achieved = algo_bytes / (os_ms / os_launches / 1e3) / 1e9 if os_launches else None
@@ -466,11 +470,17 @@ def main():
             "nominal_peak": NOMINAL_HBM_GBS,
             "frac_of_nominal": achieved / NOMINAL_HBM_GBS if achieved else None,
             "avg_launch_ms": os_ms / os_launches if os_launches else None,
+            "scatter_passes": passes,
             "algorithmic_bytes_per_launch": algo_bytes,
             "hist_avg_launch_ms": hist_ms / hist_launches if hist_launches else None,
             "hist_achieved_gbs": (roofline.histogram_bytes_per_item() * n / (hist_ms / hist_launches / 1e3) / 1e9)
             if hist_launches else None,
-            "whole_sort_gbs": roofline.sort_bytes_per_item(True) * n * args.steps / (elapsed_ms / 1e3) / 1e9,
+            # Items read once by the histogram, moved by every pass that ran and, after
+            # two passes of the top-digits order, once more by the on-chip sorts.
+            "whole_sort_gbs": (roofline.histogram_bytes_per_item()
+                               + roofline.scatter_bytes_per_item(True)
+                               * (passes + (1 if "chunk_bounds" in per_kind and passes == 2 else 0)))
+            * n * args.steps / (elapsed_ms / 1e3) / 1e9,
             "per_kind_ms": {k: v[1] / max(v[0], 1) for k, v in per_kind.items() if v[0]}}
 
     # Release the step buffers before the end-to-end and CPU legs.

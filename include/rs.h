@@ -372,14 +372,17 @@ typedef enum rs_tune_knob {
                                      one-CTA shared-memory sort; segments up to 4096 always
                                      take an on-chip sort */
     RS_TUNE_TILE_SEG = 5,         /* tile shape index of the segmented scatter passes */
-    RS_TUNE_WARP_MAX = 6,         /* segments (and MSD-first buckets) up to this size (<= 512)
+    RS_TUNE_WARP_MAX = 6,         /* segments up to this size (<= 512)
                                      take the one-warp shared-memory sort; 0 turns it off */
-    RS_TUNE_SMALL_BITS = 7,       /* digit width of the one-warp and one-CTA sorts: 8 (four
-                                     passes, the default) or 4 (eight passes) */
-    RS_TUNE_MSD = 8,              /* 1: unsigned whole arrays of up to 2^21 items may take the
-                                     MSD-first order of Alg. 2 (one pass by the top digit, then
-                                     every bucket sorted on chip) when no top-digit bucket holds
-                                     more than 8192 keys; 0: always the four LSD passes */
+    RS_TUNE_SMALL_BITS = 7,       /* on-chip sorts: 8 (the default), the one-warp sort in four
+                                     8-bit passes and the one-CTA bin sort; 4, both in eight
+                                     4-bit passes */
+    RS_TUNE_MSD = 8,              /* 1 (the default): whole arrays may take the MSD-first order
+                                     of Alg. 2 (one pass by the top digit, then every bucket
+                                     sorted on chip) where the buckets fit a CTA, or from 2^25
+                                     items the top-digits order (two passes by the two highest
+                                     digits, then chunks sorted on chip) where the keys spread
+                                     evenly; 0: always the LSD passes */
     RS_TUNE_TYPED_SPLIT = 9       /* signed and float keys: sorts of at least this many items
                                      launch two instances of every scatter pass (the passes that
                                      need no key map run without it, at the unsigned speed);

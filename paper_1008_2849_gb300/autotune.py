@@ -6,9 +6,9 @@ captured CUDA graphs (rs_graph_*) of a representative synthetic workload
 under every candidate setting and keeps the fastest:
 
 * whole arrays: the tile shape of the scatter passes, for key-value and for
-  keys-only sorts; up to 2^21 items, the MSD-first order of Alg. 2 (one pass
-  by the top digit, then on-chip bucket sorts) or the four LSD passes; from
-  2^24 items, four passes of 8-bit digits or three of 11/11/10 bits; for
+  keys-only sorts; the MSD-first order of Alg. 2 (one pass by the top digit,
+  then on-chip bucket sorts; from 2^25 items two passes and on-chip chunks) or
+  the four LSD passes; from 2^24 items, four passes of 8-bit digits or three of 11/11/10 bits; for
   arrays up to 8192 items, which take the one-CTA sort, and at which digit
   width;
 * segmented batches: the tile shape of the segmented scatter passes and the
@@ -33,7 +33,8 @@ import numpy as np
 
 # Representative item counts per size class (whole arrays).
 CLASS_SIZES = {1: 1 << 16, 2: 1 << 20, 3: 1 << 24, 4: 1 << 27}
-MSD_MAX_ITEMS = 256 * 8192  # largest whole array the MSD-first order is tried for
+# Whole arrays the orders by the top digits first are tried for.
+MSD_MAX_ITEMS, TOP_MIN_ITEMS = 256 * 7400, 1 << 25
 DIGITS11_MIN_ITEMS = 1 << 24  # smallest whole array the 11-bit-digit order is tried for
 
 
@@ -86,9 +87,9 @@ def tune_whole(rs, torch, inputs, reps=3, quick=False):
             best[knob] = min(res, key=res.get)
             best[knob + "_ms"] = res
             rs.tune_set_class(cls, knob, best[knob])
-        if n <= MSD_MAX_ITEMS:
-            # MSD-first order (one top-digit pass + on-chip bucket sorts) or
-            # the four LSD passes, with the chosen shapes; pairs + keys time.
+        if n <= MSD_MAX_ITEMS or n >= TOP_MIN_ITEMS:
+            # Top digits first (one or two passes + on-chip sorts) or the four
+            # LSD passes, with the chosen shapes; pairs + keys time.
             old_msd = rs.tune_get_class(cls, "msd")
             res = {}
             for msd in (0, 1):

@@ -35,9 +35,8 @@ constexpr uint32_t DIR_B_TO_A = 2; // alternate buffers -> caller's arrays
 // Per-call control block, zeroed by one cudaMemsetAsync at the start of a
 // call.  Lives at the start of the workspace.
 // Plan slots: the LSD passes 0..7 (0..3 for 32-bit keys), and MSD_SLOT for
-// the most-significant-digit pass of the MSD-first order (Alg. 2), which runs
-// before the passes 0..3 are reached and, when the plan chooses it, makes them
-// all DIR_SKIP.
+// the most-significant-digit pass of the MSD-first order (Alg. 2): when the plan
+// chooses it, the passes 0..3 are all DIR_SKIP, and the launch of pass 3 runs it.
 constexpr uint32_t MSD_SLOT = PASSES64;
 constexpr uint32_t PLAN_SLOTS = PASSES64 + 1;
 
@@ -54,7 +53,8 @@ struct Ctrl {
     uint32_t big_count;
     uint32_t large_count;
     uint32_t tiny_count;
-    uint32_t pad[7];               // keep hist 64-byte aligned
+    uint32_t chunk_count;          // top-digits order: chunks sorted on chip (0: another order)
+    uint32_t pad[6];               // keep hist 64-byte aligned
     uint32_t hist[PASSES64][RADIX];  // digit histograms (H); 0..3 for 32-bit keys
     uint32_t gofs[PASSES64][RADIX];  // first output slot of every bucket (G)
 };
@@ -85,6 +85,8 @@ constexpr uint32_t KEY_F64 = 5;
 constexpr uint32_t ROLE_PLAIN_PASSES = 1u << 8;
 constexpr uint32_t ROLE_MAP_PASSES = 1u << 9;
 constexpr uint32_t KEY_TYPE_MASK = 0xffu;
+// A launch of pass 3 that is the MSD-first order's pass when the plan chose it.
+constexpr uint32_t ROLE_MSD_TOO = 1u << 10;
 
 __device__ __forceinline__ uint32_t key_to_ordered(uint32_t k, uint32_t type) {
     const uint32_t neg = type == KEY_F32 ? (uint32_t)((int32_t)k >> 31) : 0u;

@@ -5,6 +5,8 @@
 //            sum"; Alg. 2 PrefixSum) and the pass plan.
 #pragma once
 
+#include <type_traits>
+
 #include "rs_device.cuh"
 
 namespace rs {
@@ -106,16 +108,18 @@ k_hist4(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict__ hi
 }
 
 // ---------------------------------------------------------------------------
-// k_hist4_cols: the same histograms with one private column per lane: bin b
-// of digit p, as seen by lane l, lives at word (p*256 + b)*32 + l of a
-// 128 KiB shared array, so the 32 lanes of a warp always add into 32
+// k_hist4_cols: the same histograms with private columns: bin b of digit p, as
+// seen by lane l, lives at word (p*256 + b)*COLS + l % COLS.  With 32 columns
+// (128 KiB, one CTA per SM) the 32 lanes of a warp always add into 32
 // different banks (one shared-memory wavefront per warp-wide add, whatever
-// the keys).  Columns are summed (in rotated order, again conflict-free) at
-// the end.  One CTA per SM.
+// the keys).  Eight columns (32 KiB) take up to four, but a quarter of the time
+// to clear and to sum, which is what small arrays pay for.  Columns are
+// summed (in rotated order, conflict-free) at the end.
 // ---------------------------------------------------------------------------
-constexpr uint32_t HIST_COL_WORDS = PASSES * RADIX * 32;
+template <int COLS>
+constexpr uint32_t HIST_COL_WORDS = PASSES * RADIX * COLS;
 
-template <int THREADS, bool TYPED>
+template <int THREADS, int COLS, bool TYPED>
 __global__ void __launch_bounds__(THREADS, 1)
 k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict__ hist,
              uint4* __restrict__ clear, uint32_t clear_vec4, uint32_t key_type) {
@@ -124,7 +128,8 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
     const uint32_t tid = threadIdx.x;
     const uint32_t lane = tid & 31;
     pdl_launch_next();  // the plan kernel may launch; it waits for this one
-    for (uint32_t i = tid; i < HIST_COL_WORDS / 4; i += THREADS) s_cols4[i] = make_uint4(0, 0, 0, 0);
+    for (uint32_t i = tid; i < HIST_COL_WORDS<COLS> / 4; i += THREADS)
+        s_cols4[i] = make_uint4(0, 0, 0, 0);
     const uint32_t gtid = blockIdx.x * THREADS + tid;
     const uint32_t gsize = gridDim.x * THREADS;
     for (uint32_t i = gtid; i < clear_vec4; i += gsize) clear[i] = make_uint4(0, 0, 0, 0);
@@ -135,12 +140,12 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
     const uint32_t body4 = (n - head) >> 2;
     const uint32_t tail = head + body4 * 4;
     const uint4* __restrict__ body = reinterpret_cast<const uint4*>(keys + head);
-    uint32_t* const mycol = s_col + lane;
+    uint32_t* const mycol = s_col + lane % COLS;
     auto count_key = [&](uint32_t key) {
         if (TYPED) key = key_to_ordered(key, key_type);
 #pragma unroll
         for (uint32_t p = 0; p < PASSES; ++p)
-            atomicAdd(mycol + ((p * RADIX + ((key >> (p * RADIX_BITS)) & (RADIX - 1))) << 5), 1u);
+            atomicAdd(mycol + (p * RADIX + ((key >> (p * RADIX_BITS)) & (RADIX - 1))) * COLS, 1u);
     };
     // HIST_LOADS independent 16-byte loads in flight per thread and
     // iteration (64 KiB per SM): enough bytes in flight to cover the HBM
@@ -169,15 +174,18 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
     __syncthreads();
     for (uint32_t bin = tid; bin < PASSES * RADIX; bin += THREADS) {
         uint32_t c = 0;
+        const uint32_t turn = bin * COLS / 32 + bin;  // 32 lanes, 32 banks
 #pragma unroll 8
-        for (uint32_t j = 0; j < 32; ++j) c += s_col[(bin << 5) + ((j + bin) & 31)];
+        for (uint32_t j = 0; j < COLS; ++j) c += s_col[bin * COLS + (j + turn) % COLS];
         if (c) atomicAdd(hist + bin, c);
     }
 }
 
 // ---------------------------------------------------------------------------
 // k_plan: G[p][b] = sum_{b' < b} H[p][b'] and the pass plan.  One CTA of
-// 1024 threads, thread (p, b) = (tid / 256, tid % 256).
+// 1024 threads, thread (p, b) = (tid / 256, tid % 256).  (Made by the histogram
+// kernel's last CTA instead, it takes 4 us longer: as a kernel of its own it is
+// resident when the counts are complete.)
 //
 // A pass whose digit takes one value for every key is the identity (a stable
 // partition into one bucket).  Such passes are skipped, except that the
@@ -193,21 +201,48 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
 // is constant, so that pass is trivial there).  msd_off[b] is bucket b's
 // first slot (msd_off[256] = n), and small_count becomes the number of buckets
 // to sort (0 when the plan chooses the passes 0..3).
+//
+// Top-digits order, when top_bits > 0: if the keys spread evenly, only the
+// passes by the two highest digits run.  The array is then stably sorted by
+// its top 16 bits, and every chunk of keys with the same top_bits highest
+// bits (about n >> top_bits of them) is sorted on chip by the rest.  "Evenly":
+// no bucket of either digit holds over twice its share, at least three passes
+// would run otherwise, and of TOP_SAMPLES keys no chunk holds far more than its
+// share (the digits may be even one by one and not together).  Chunks that are
+// too long all the same are sorted in global memory by one CTA each, so a
+// sample that misses them costs time, not correctness.
 // ---------------------------------------------------------------------------
+constexpr uint32_t TOP_SAMPLES = 4096;
+constexpr uint32_t TOP_MAX_BITS = 16;
+constexpr size_t TOP_PLAN_SMEM = (size_t(1) << TOP_MAX_BITS) * sizeof(uint16_t);
+
+// What the plan works on; bucket_cap and msd_off for the MSD-first order
+// (msd_off == nullptr: not allowed), top_bits for the top-digits order.
+struct PlanArgs {
+    Ctrl* ctrl;
+    const void* keys;
+    uint32_t n, key_type, bucket_cap;
+    uint32_t* msd_off;
+    uint32_t top_bits;
+};
+
+// Dynamic shared memory: 2 << top_bits bytes when top_bits is set.
 template <int NPASS>
-__global__ void __launch_bounds__(1024)
-k_plan(Ctrl* __restrict__ ctrl, uint32_t n, uint32_t msd_allowed, uint32_t bucket_cap,
-       uint32_t* __restrict__ msd_off) {
+__global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
+    extern __shared__ uint4 s_dyn[];
     static_assert(NPASS == 4 || NPASS == 8, "32-bit or 64-bit keys");
+    using K = std::conditional_t<NPASS == 8, unsigned long long, uint32_t>;
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_trivial[NPASS];
-    __shared__ uint32_t s_big;
+    __shared__ uint32_t s_big, s_uneven;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t b = tid & (RADIX - 1);
+    Ctrl* const ctrl = plan.ctrl;
+    const uint32_t n = plan.n, top_bits = plan.top_bits;
     pdl_launch_next();
     pdl_wait();  // the histograms are complete
     if (tid < NPASS) s_trivial[tid] = 0;
-    if (tid == 0) s_big = 0;
+    if (tid == 0) s_big = s_uneven = 0;
     // Thread (p, b): p = tid / 256 (+ 4 in the second round for 64-bit keys).
     uint32_t first3 = 0;  // digit 3, for the MSD-first order
     for (uint32_t round = 0; round < NPASS / 4; ++round) {
@@ -228,40 +263,109 @@ k_plan(Ctrl* __restrict__ ctrl, uint32_t n, uint32_t msd_allowed, uint32_t bucke
         if (h == n) s_trivial[p] = 1;
         if (p == PASSES - 1) {
             first3 = first;
-            if (h > bucket_cap) s_big = 1;
+            if (h > plan.bucket_cap) s_big = 1;
         }
+        if (p >= NPASS - 2 && h > n / RADIX * 2) s_uneven = 1;
         __syncthreads();  // s_warp is reused by the next round
     }
-    const bool msd = NPASS == 4 && msd_allowed && !s_trivial[PASSES - 1] && !s_big;
+    const bool msd =
+        NPASS == 4 && plan.msd_off != nullptr && !s_trivial[PASSES - 1] && !s_big;
+    uint32_t executed = 0;
+    for (uint32_t q = 0; q < NPASS; ++q) executed += s_trivial[q] ? 0 : 1;
+    bool top = !msd && top_bits != 0 && !s_uneven && executed >= 3;
+    if (top) {  // the same for every thread
+        uint32_t* const s_pair = reinterpret_cast<uint32_t*>(s_dyn);  // two 16-bit counts a word
+        const uint32_t chunks = 1u << top_bits;
+        for (uint32_t i = tid; i < (chunks + 7) / 8; i += 1024) s_dyn[i] = make_uint4(0, 0, 0, 0);
+        const K* const keys = static_cast<const K*>(plan.keys);
+        constexpr uint32_t PER = TOP_SAMPLES / 1024;
+        const uint32_t stride = n / TOP_SAMPLES;
+        K k[PER];
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q) {  // one key of each of TOP_SAMPLES parts
+            const uint32_t i = q * 1024 + tid;
+            uint32_t r = i * 0x9E3779B1u;
+            r ^= r >> 15;
+            r *= 0x85EBCA6Bu;
+            const uint32_t at = (uint32_t)(((uint64_t)i * n) / TOP_SAMPLES) + __umulhi(r, stride);
+            k[q] = keys[at];
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t q = 0; q < PER; ++q) {
+            const uint32_t c =
+                (uint32_t)(key_to_ordered(k[q], plan.key_type) >> (8 * sizeof(K) - top_bits));
+            const uint32_t was = atomicAdd(&s_pair[c >> 1], 1u << (16 * (c & 1)));
+            if (((was >> (16 * (c & 1))) & 0xffffu) >= 2 * (TOP_SAMPLES >> top_bits) + 12)
+                s_uneven = 1;
+        }
+        __syncthreads();
+        top = !s_uneven;
+    }
     if (msd && (tid >> 8) == PASSES - 1) {
-        msd_off[b] = first3;
-        if (b == RADIX - 1) msd_off[RADIX] = n;
+        plan.msd_off[b] = first3;
+        if (b == RADIX - 1) plan.msd_off[RADIX] = n;
     }
-    if (tid == 0 && msd) {
-        for (uint32_t q = 0; q < PASSES; ++q) ctrl->dir[q] = DIR_SKIP;
-        ctrl->dir[MSD_SLOT] = DIR_A_TO_B;
-        ctrl->small_count = RADIX;
-    } else if (tid == 0) {
-        ctrl->dir[MSD_SLOT] = DIR_SKIP;
-        uint32_t trivial[NPASS], executed = 0;
-        for (uint32_t q = 0; q < NPASS; ++q) {
-            trivial[q] = s_trivial[q];
-            executed += trivial[q] ? 0 : 1;
-        }
-        if (executed & 1) {
-            for (uint32_t q = 0; q < NPASS; ++q)
-                if (trivial[q]) { trivial[q] = 0; break; }
-        }
-        uint32_t parity = 0;
-        for (uint32_t q = 0; q < NPASS; ++q) {
-            if (trivial[q]) {
-                ctrl->dir[q] = DIR_SKIP;
-            } else {
-                ctrl->dir[q] = parity ? DIR_B_TO_A : DIR_A_TO_B;
-                parity ^= 1;
-            }
+    if (tid != 0) return;
+    ctrl->dir[MSD_SLOT] = msd ? DIR_A_TO_B : DIR_SKIP;
+    ctrl->small_count = msd ? RADIX : 0u;
+    ctrl->chunk_count = top ? 1u << top_bits : 0u;
+    bool skip[NPASS];
+    for (uint32_t q = 0; q < NPASS; ++q) skip[q] = msd || s_trivial[q] || (top && q < NPASS - 2);
+    if (!msd && !top && (executed & 1)) {
+        for (uint32_t q = 0; q < NPASS; ++q)
+            if (skip[q]) { skip[q] = false; break; }
+    }
+    uint32_t parity = 0;
+    for (uint32_t q = 0; q < NPASS; ++q) {
+        if (skip[q]) {
+            ctrl->dir[q] = DIR_SKIP;
+        } else {
+            ctrl->dir[q] = parity ? DIR_B_TO_A : DIR_A_TO_B;
+            parity ^= 1;
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// k_chunk_bounds: the chunks of the top-digits order, once the array is sorted
+// by its top 16 bits: off[c] = the first key with its top_bits highest bits
+// equal to c or more, off[1 << top_bits] = n.  WAYS lanes search together for
+// each bound in the bucket of its highest digit (G of that digit says where it
+// lies), reading WAYS keys at a time that cut what is left into WAYS + 1 parts:
+// dependent reads are what takes the time, and 32 ways need 3 to 4 of them where
+// halving needs 13 to 16 (14 us for 8192 chunks of 2^24 keys).  Many chunks take
+// fewer ways, for the keys read.
+// ---------------------------------------------------------------------------
+template <typename K, int WAYS>
+__global__ void __launch_bounds__(256)
+k_chunk_bounds(const K* __restrict__ keys, uint32_t n, const Ctrl* __restrict__ ctrl,
+               uint32_t top_bits, uint32_t key_type, uint32_t* __restrict__ off) {
+    pdl_launch_next();
+    pdl_wait();  // the scatter passes are complete
+    if (ctrl->chunk_count == 0) return;
+    const uint32_t chunks = 1u << top_bits;
+    const uint32_t way = threadIdx.x % WAYS;
+    const uint32_t first_lane = (threadIdx.x & 31) / WAYS * WAYS;
+    // (chunks is a multiple of the bounds per CTA: the grid is exact.)
+    const uint32_t c = (blockIdx.x * 256 + threadIdx.x) / WAYS;
+    if (c == 0 && way == 0) off[chunks] = n;
+    const uint32_t* const g = ctrl->gofs[sizeof(K) - 1];
+    const uint32_t b = c >> (top_bits - RADIX_BITS);
+    uint32_t lo = g[b], hi = b + 1 < RADIX ? g[b + 1] : n;  // the answer is in [lo, hi]
+    const K want = (K)c << (8 * sizeof(K) - top_bits);
+    while (__any_sync(0xffffffffu, lo < hi)) {
+        const uint32_t part = (hi - lo) / (WAYS + 1) + 1;  // keys left of the first cut, at most
+        const uint32_t at = lo + (way + 1) * part - 1;
+        const bool below = at < hi && key_to_ordered(keys[at], key_type) < want;
+        const uint32_t votes =
+            __ballot_sync(0xffffffffu, below) >> first_lane & (0xffffffffu >> (32 - WAYS));
+        const uint32_t cuts = __popc(votes);  // the first `cuts` cuts are below
+        const uint32_t next = lo + cuts * part;
+        hi = min(hi, next + part - 1);
+        lo = min(next, hi);
+    }
+    if (way == 0) off[c] = lo;
 }
 
 // ---------------------------------------------------------------------------

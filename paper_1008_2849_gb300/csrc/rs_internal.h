@@ -29,6 +29,7 @@ enum KernelKind : int {
     KK_D11_UP = 9,
     KK_D11_SCAN = 10,
     KK_D11_DOWN = 11,
+    KK_CHUNK_BOUNDS = 12,
     KK_COUNT
 };
 const char* kernel_kind_name(int kind);
@@ -75,13 +76,24 @@ struct ClassKnobs {
     int small_max;
     int warp_max;
     int small_bits;
-    int msd;        // 1: whole arrays up to kMsdMaxItems may take the MSD-first order
+    int msd;        // 1: whole arrays may take the MSD-first or the top-digits order
     int digits;     // 8: four 8-bit passes; 11: three 11/11/10-bit passes (rs_digits11.cu)
                     // for unsigned keys, when the caller's workspace holds their buffers
 };
-// Largest whole array the MSD-first order is tried for: 256 buckets of at
-// most the one-CTA sort's capacity.
-constexpr uint32_t kMsdMaxItems = 256u * 8192u;
+// The MSD-first order sorts the buckets of the highest digit on chip: by a CTA of
+// 5120 items for arrays of up to 256 * 4600 items, of 8192 up to 256 * 7400 items
+// (the largest bucket of evenly spread keys stays seven or more standard deviations below).
+constexpr uint32_t kMsdShortItems = 256u * 4600u;
+constexpr uint32_t kMsdMaxItems = 256u * 7400u;
+// Arrays of kTopMinItems and more may take the top-digits order: two scatter passes,
+// then chunks of the keys' `bits` highest bits sorted on chip, by a CTA of 4608 items,
+// or 8192 for long_chunks.  bits = 0: not tried.
+constexpr uint32_t kTopMinItems = 1u << 25;
+struct TopOrder {
+    uint32_t bits;
+    bool long_chunks;
+};
+TopOrder top_order(size_t n);
 // Size classes by item count (whole array; for a segmented sort the average
 // segment): <= 2^13, <= 2^16, <= 2^20, <= 2^24, <= 2^28, larger.
 constexpr int NUM_SIZE_CLASSES = 6;
@@ -179,6 +191,9 @@ rs_status enqueue_histograms(const uint32_t* keys, uint32_t n, uint32_t* hist,
 // the ordered words of typed keys, and clearing clear_bytes at `clear`.
 rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* clear,
                         size_t clear_bytes, uint32_t key_type, cudaStream_t stream);
+// The plan kernel (rs_hist_plan.cuh), for keys of NPASS digits.
+struct PlanArgs;
+template <int NPASS> rs_status enqueue_plan(const PlanArgs& plan, cudaStream_t stream);
 
 // Segmented scatter passes: per-tile geometry and per-segment bucket bases
 // built on the device, and an upper bound of the tile count for the launch.
@@ -201,15 +216,21 @@ rs_status launch_onesweep_pairs(int cfg, bool wide, uint32_t* ka, uint32_t* va, 
                                 Ctrl* ctrl, uint32_t* sticky, void* status, void* status_clear,
                                 const SegView* seg, uint32_t key_type, cudaStream_t stream);
 
-// One-CTA sorts on chip of those of the segments 0 .. *count - 1 that hold 1 to
-// small_sort_capacity() items (count on the device): a CTA of one size for those
-// of up to `usual` items, a larger one for the rest.  bits: 8, the bin sort
-// (rs_bin_sort.cuh); 4, eight counting passes of 4-bit digits.  Items are read
-// from src_keys / src_vals.
+// One-CTA sorts on chip of the segments 0 .. *count - 1 (count on the device) of at
+// most bucket_capacity(long_buckets) items each, read from src_keys / src_vals.
+// bits: 8, the bin sort (rs_bin_sort.cuh); 4, eight counting passes of 4-bit digits.
+uint32_t bucket_capacity(bool long_buckets);
 rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
                               const uint32_t* src_vals, const uint32_t* off,
-                              const uint32_t* count, const Ctrl* ctrl, uint32_t usual, int bits,
-                              uint32_t key_type, cudaStream_t stream);
+                              const uint32_t* count, const Ctrl* ctrl, bool long_buckets,
+                              int bits, uint32_t key_type, cudaStream_t stream);
+// On-chip sorts, in place, of the chunks 0 .. *count - 1 of the top-digits order
+// (off[c] .. off[c + 1]); longer ones than the chip takes are sorted in global
+// memory through the spare arrays (of the same size as keys / vals).
+rs_status launch_chunk_sorts(uint32_t* keys, uint32_t* vals, uint32_t* spare_keys,
+                             uint32_t* spare_vals, const uint32_t* off, const uint32_t* count,
+                             const Ctrl* ctrl, TopOrder top, uint32_t key_type,
+                             cudaStream_t stream);
 // The segments listed by size (rs_bin_sort.cuh list_small) in tiny_list and
 // small_list of `entries` entries each, in place: one launch per size up to
 // max_items.

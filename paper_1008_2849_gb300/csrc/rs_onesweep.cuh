@@ -188,6 +188,10 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
     // one are all complete from here on.
     pdl_launch_next();
     pdl_wait();
+    if (key_type & ROLE_MSD_TOO) {
+        if (ctrl->dir[MSD_SLOT] != DIR_SKIP) slot = MSD_SLOT;
+        key_type &= ~ROLE_MSD_TOO;
+    }
     if (key_type & (ROLE_PLAIN_PASSES | ROLE_MAP_PASSES)) {
         // One of the two instances of a typed sort's pass: keep the pass if
         // it is this instance's (an executed first or last pass needs the
@@ -208,8 +212,11 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
     }
     const uint32_t dir = ctrl->dir[slot];
     if (dir == DIR_SKIP) {
-        // No tiles in this pass: clear the whole next status array here.
-        if (status_clear != nullptr)
+        // No tiles in this pass: clear the whole next status array here, if
+        // the next launch has tiles.
+        if (status_clear != nullptr &&
+            (ctrl->dir[slot + 1] != DIR_SKIP ||
+             (slot + 1 == PASSES - 1 && ctrl->dir[MSD_SLOT] != DIR_SKIP)))
             for (uint32_t i = blockIdx.x * THREADS + tid; i < clear_words; i += gridDim.x * THREADS)
                 status_clear[i] = 0;
         return;

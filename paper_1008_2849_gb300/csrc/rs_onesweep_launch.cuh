@@ -64,7 +64,7 @@ static rs_status launch_onesweep_variant(int cfg, uint32_t* ka, uint32_t* va, ui
                                          uint32_t* sticky, void* status, void* status_clear,
                                          const SegView& seg, uint32_t key_type,
                                          cudaStream_t stream) {
-    if (key_type != KEY_U32) {
+    if ((key_type & KEY_TYPE_MASK) != KEY_U32) {
         // Typed keys: from typed_split_min items on, the passes that need no
         // maps run without them (see ROLE_PLAIN_PASSES) and both instances
         // are launched for every pass; below it the mapping instance alone
@@ -87,7 +87,7 @@ static rs_status launch_onesweep_variant(int cfg, uint32_t* ka, uint32_t* va, ui
 #define RS_CASE(I, T, J, B, W)                                                                    \
     case I:                                                                                       \
         return launch_onesweep_shape<T, J, B, W, PAIRS, S, SEG, false>(                           \
-            ka, va, kb, vb, n, pass, slot, ctrl, sticky, status, status_clear, seg, KEY_U32, stream);
+            ka, va, kb, vb, n, pass, slot, ctrl, sticky, status, status_clear, seg, key_type, stream);
         RS_TILE_SHAPES(RS_CASE)
 #undef RS_CASE
     default: return RS_ERR_INVALID_ARG;

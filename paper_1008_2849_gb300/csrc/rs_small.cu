@@ -29,29 +29,27 @@ rs_status grid_of(const SmallWork& w, uint32_t per_sm, uint32_t* grid) {
     return st;
 }
 
-template <typename Kern>
-rs_status launch_small_kernel(Kern kern, uint32_t grid, uint32_t threads, size_t smem,
-                              const SmallWork& w, cudaStream_t stream) {
-    note_launch_begin(KK_SMALL, stream);
-    const cudaError_t e = launch_after_previous(kern, dim3(grid), dim3(threads), smem, stream,
-                                                w.keys, w.vals, w.src_keys, w.src_vals, w.off,
-                                                w.list, w.step, w.list_count, w.ctrl, w.single_n,
-                                                w.key_type);
-    note_launch_end(KK_SMALL, stream);
-    return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
-}
-
-template <bool PAIRS, int THREADS, int ITEMS, int MIN_BLOCKS>
-rs_status launch_bin_shape(const SmallWork& w, cudaStream_t stream) {
-    using L = BinSortSmem<uint32_t, uint32_t, PAIRS, THREADS, ITEMS>;
-    auto kern = k_bin_sort<uint32_t, uint32_t, PAIRS, THREADS, ITEMS, MIN_BLOCKS>;
+// The word of the bin sort: the key alone; for pairs 64 bits, or in chunks, whose
+// keys have few bits left, 32.
+template <bool PAIRS, int THREADS, int MIN_BLOCKS, bool CHUNKS = false>
+rs_status launch_bin_shape(const SmallWork& w, cudaStream_t stream, uint32_t* spare_keys = nullptr,
+                           uint32_t* spare_vals = nullptr) {
+    using W = std::conditional_t<PAIRS && !CHUNKS, unsigned long long, uint32_t>;
+    using L = BinSortSmem<uint32_t, uint32_t, W, PAIRS, THREADS, CHUNKS>;
+    auto kern = k_bin_sort<uint32_t, uint32_t, W, PAIRS, THREADS, MIN_BLOCKS, CHUNKS>;
     static DeviceOnce smem_set;
     rs_status st = allow_smem_once(kern, L::BYTES, smem_set);
     if (st != RS_OK) return st;
     uint32_t grid = 0;
     st = grid_of(w, MIN_BLOCKS, &grid);
     if (st != RS_OK) return st;
-    return launch_small_kernel(kern, grid, THREADS, L::BYTES, w, stream);
+    note_launch_begin(KK_SMALL, stream);
+    const cudaError_t e = launch_after_previous(
+        kern, dim3(grid), dim3(THREADS), L::BYTES, stream, w.keys, w.vals, w.src_keys, w.src_vals,
+        w.off, w.list, w.step, w.list_count, w.ctrl, w.single_n, w.key_type, spare_keys,
+        spare_vals);
+    note_launch_end(KK_SMALL, stream);
+    return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
 
 template <int THREADS, int ITEMS, bool PAIRS>
@@ -65,7 +63,13 @@ rs_status launch_small_shape4(const SmallWork& w, cudaStream_t stream) {
     uint32_t grid = 0;
     st = grid_of(w, 4, &grid);
     if (st != RS_OK) return st;
-    return launch_small_kernel(kern, grid, THREADS, SMEM, w, stream);
+    note_launch_begin(KK_SMALL, stream);
+    const cudaError_t e = launch_after_previous(kern, dim3(grid), dim3(THREADS), SMEM, stream,
+                                                w.keys, w.vals, w.src_keys, w.src_vals, w.off,
+                                                w.list, w.step, w.list_count, w.ctrl, w.single_n,
+                                                w.key_type);
+    note_launch_end(KK_SMALL, stream);
+    return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
 
 // The CTA for arrays of at most max_items items: 128 threads up to 1024, 512 up
@@ -78,9 +82,9 @@ rs_status launch_small_size(uint32_t max_items, int bits, const SmallWork& w,
         return max_items <= SMALL_MID_MAX ? launch_small_shape4<256, 16, PAIRS>(w, stream)
                                           : launch_small_shape4<512, 16, PAIRS>(w, stream);
     if (max_items <= SMALL_SHORT_MAX && w.off != nullptr)
-        return launch_bin_shape<PAIRS, 128, 8, 10>(w, stream);
-    if (max_items <= SMALL_MID_MAX) return launch_bin_shape<PAIRS, 512, 8, 3>(w, stream);
-    return launch_bin_shape<PAIRS, 1024, 8, 1>(w, stream);
+        return launch_bin_shape<PAIRS, 128, 8>(w, stream);
+    if (max_items <= SMALL_MID_MAX) return launch_bin_shape<PAIRS, 512, 2>(w, stream);
+    return launch_bin_shape<PAIRS, 1024, 1>(w, stream);
 }
 
 rs_status launch_small_any(uint32_t max_items, int bits, const SmallWork& w,
@@ -112,22 +116,30 @@ rs_status launch_warp_bits(uint32_t* keys, uint32_t* vals, const uint32_t* src_k
 uint32_t small_sort_capacity() { return 8192; }
 uint32_t warp_sort_capacity() { return 32 * WARP_SORT_ITEMS; }
 
+uint32_t bucket_capacity(bool long_buckets) { return long_buckets ? 8192 : 5120; }
+
 rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
                               const uint32_t* src_vals, const uint32_t* off,
-                              const uint32_t* count, const Ctrl* ctrl, uint32_t usual, int bits,
-                              uint32_t key_type, cudaStream_t stream) {
-    SmallWork w{keys, vals, src_keys, src_vals, off, nullptr, 1, count, ctrl, 0, key_type};
-    // (The 4-bit sorts have no CTA for up to SMALL_SHORT_MAX items: one launch.)
-    const uint32_t sizes[] = {bits == 4 || usual > SMALL_MID_MAX ? small_sort_capacity()
-                              : usual > SMALL_SHORT_MAX          ? SMALL_MID_MAX
-                                                                 : SMALL_SHORT_MAX,
-                              small_sort_capacity()};
-    for (const uint32_t size : sizes) {
-        const rs_status st = launch_small_any(size, bits, w, stream);
-        if (st != RS_OK || size == small_sort_capacity()) return st;
-        w.single_n = size;  // the larger CTA takes the buckets above
-    }
-    return RS_OK;
+                              const uint32_t* count, const Ctrl* ctrl, bool long_buckets,
+                              int bits, uint32_t key_type, cudaStream_t stream) {
+    const SmallWork w{keys, vals, src_keys, src_vals, off, nullptr, 1, count, ctrl, 0, key_type};
+    if (long_buckets || bits == 4) return launch_small_any(small_sort_capacity(), bits, w, stream);
+    return vals != nullptr ? launch_bin_shape<true, 640, 2>(w, stream)
+                           : launch_bin_shape<false, 640, 2>(w, stream);
+}
+
+rs_status launch_chunk_sorts(uint32_t* keys, uint32_t* vals, uint32_t* spare_keys,
+                             uint32_t* spare_vals, const uint32_t* off, const uint32_t* count,
+                             const Ctrl* ctrl, TopOrder top, uint32_t key_type,
+                             cudaStream_t stream) {
+    const SmallWork w{keys, vals, keys, vals, off, nullptr, 1, count, ctrl, top.bits, key_type};
+    // (Index bits <= top.bits: a word holds the index and the bits that differ.)
+    const bool pairs = vals != nullptr;
+    if (top.long_chunks)
+        return pairs ? launch_bin_shape<true, 1024, 1, true>(w, stream, spare_keys, spare_vals)
+                     : launch_bin_shape<false, 1024, 1, true>(w, stream, spare_keys, nullptr);
+    return pairs ? launch_bin_shape<true, 576, 2, true>(w, stream, spare_keys, spare_vals)
+                 : launch_bin_shape<false, 576, 2, true>(w, stream, spare_keys, nullptr);
 }
 
 rs_status launch_small_lists(uint32_t* keys, uint32_t* vals, const uint32_t* off,

@@ -43,6 +43,18 @@ Layout layout_for(size_t n, bool pairs) {
     return L;
 }
 
+// The fewest chunks whose average is at most 4096 items, or 7400 for the largest
+// arrays: eight standard deviations or more below what the CTA takes, for evenly
+// spread keys.  (32-bit words hold an index of 13 bits and the 32 - bits low bits
+// of a key: bits >= 13.)
+TopOrder top_order(size_t n) {
+    if (n < kTopMinItems) return {0, false};
+    for (uint32_t bits = 13; bits <= TOP_MAX_BITS; ++bits)
+        if ((n >> bits) <= 4096) return {bits, false};
+    if ((n >> TOP_MAX_BITS) <= 7400) return {TOP_MAX_BITS, true};
+    return {0, false};
+}
+
 rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* clear,
                         size_t clear_bytes, uint32_t key_type, cudaStream_t stream) {
     DeviceInfo di;
@@ -54,17 +66,22 @@ rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* 
     if (blocks > needed) blocks = needed;
     if (blocks < 1) blocks = 1;
     if (knobs().hist_mode == HIST_COLUMNS) {
-        constexpr int T = 1024;
-        constexpr size_t SMEM = HIST_COL_WORDS * sizeof(uint32_t);
-        auto kern = key_type != KEY_U32 ? k_hist4_cols<T, true> : k_hist4_cols<T, false>;
-        static DeviceOnce smem_set[2];  // per instance
-        st = allow_smem_once(kern, SMEM, smem_set[key_type != KEY_U32 ? 1 : 0]);
+        // Eight columns (two CTAs per SM, two 16-byte loads a thread) up to 2^21
+        // keys, then 32: 2^20 uniform keys sort in 37.1 us instead of 38.9, 2^18 in
+        // 31.4 instead of 32.1; from 2^22 on the 32-column reads are faster.
+        const bool few = n <= (1u << 21), typed = key_type != KEY_U32;
+        constexpr int T8 = 512, T32 = 1024;
+        const size_t smem = (few ? HIST_COL_WORDS<8> : HIST_COL_WORDS<32>) * sizeof(uint32_t);
+        auto kern = few ? (typed ? k_hist4_cols<T8, 8, true> : k_hist4_cols<T8, 8, false>)
+                        : (typed ? k_hist4_cols<T32, 32, true> : k_hist4_cols<T32, 32, false>);
+        static DeviceOnce smem_set[4];  // per instance
+        st = allow_smem_once(kern, smem, smem_set[(few ? 2 : 0) + (typed ? 1 : 0)]);
         if (st != RS_OK) return st;
-        uint32_t grid = (uint32_t)di.sm_count;
-        const uint32_t need = (vec4 + T - 1) / T;
+        uint32_t grid = (uint32_t)di.sm_count * (few ? 2u : 1u);
+        const uint32_t need = few ? (vec4 + 2 * T8 - 1) / (2 * T8) : (vec4 + T32 - 1) / T32;
         if (grid > need) grid = need > 0 ? need : 1;
         note_launch_begin(KK_HIST, stream);
-        kern<<<grid, T, SMEM, stream>>>(keys, n, hist, static_cast<uint4*>(clear),
+        kern<<<grid, few ? T8 : T32, smem, stream>>>(keys, n, hist, static_cast<uint4*>(clear),
                                          (uint32_t)(clear_bytes / sizeof(uint4)), key_type);
         note_launch_end(KK_HIST, stream);
         return cudaPeekAtLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
@@ -89,6 +106,21 @@ rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* 
     note_launch_end(KK_HIST, stream);
     return cudaPeekAtLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
+
+template <int NPASS>
+rs_status enqueue_plan(const PlanArgs& plan, cudaStream_t stream) {
+    static DeviceOnce smem_set;
+    const rs_status st = allow_smem_once(k_plan<NPASS>, TOP_PLAN_SMEM, smem_set);
+    if (st != RS_OK) return st;
+    note_launch_begin(KK_PLAN, stream);
+    const cudaError_t e = launch_after_previous(
+        k_plan<NPASS>, dim3(1), dim3(1024), plan.top_bits ? sizeof(uint16_t) << plan.top_bits : 0,
+        stream, plan);
+    note_launch_end(KK_PLAN, stream);
+    return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
+}
+template rs_status enqueue_plan<PASSES>(const PlanArgs&, cudaStream_t);
+template rs_status enqueue_plan<PASSES64>(const PlanArgs&, cudaStream_t);
 
 rs_status enqueue_histograms(const uint32_t* keys, uint32_t n, uint32_t* hist,
                              cudaStream_t stream) {
@@ -157,46 +189,53 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     uint32_t* alt_k = reinterpret_cast<uint32_t*>(ws + L.alt_keys);
     uint32_t* alt_v = pairs ? reinterpret_cast<uint32_t*>(ws + L.alt_vals) : nullptr;
 
-    // MSD-first order (Alg. 2): tried for unsigned arrays that can split into
-    // 256 buckets the one-CTA sort takes; the plan decides on the device
-    // from the digit-3 histogram, so the launch sequence stays fixed.
-    const bool msd = ck.msd != 0 && key_type == KEY_U32 && n <= kMsdMaxItems;
+    // MSD-first order (Alg. 2): tried for arrays that can split into 256
+    // buckets the one-CTA sort takes; the plan decides on the device from the
+    // digit-3 histogram, so the launch sequence stays fixed.  Large arrays: the
+    // top-digits order likewise.
+    const bool msd = ck.msd != 0 && n <= kMsdMaxItems;
+    const bool long_buckets = n > kMsdShortItems;
+    const TopOrder top = ck.msd != 0 ? top_order(n) : TopOrder{0, false};
     uint32_t* msd_off = reinterpret_cast<uint32_t*>(ws + L.msd_off);
+    const PlanArgs plan{ctrl, keys, n, key_type, bucket_capacity(long_buckets),
+                        msd ? msd_off : nullptr, top.bits};
 
     if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
     st = enqueue_hist4(keys, n, &ctrl->hist[0][0], status[0], status_bytes, key_type, stream);
     if (st != RS_OK) return st;
-    note_launch_begin(KK_PLAN, stream);
-    const cudaError_t pe = launch_after_previous(k_plan<PASSES>, dim3(1), dim3(1024), 0, stream,
-                                                 ctrl, n, msd ? 1u : 0u, small_sort_capacity(),
-                                                 msd_off);
-    note_launch_end(KK_PLAN, stream);
-    if (pe != cudaSuccess) return RS_ERR_CUDA;
+    st = enqueue_plan<PASSES>(plan, stream);
+    if (st != RS_OK) return st;
 
     const int cfg = pairs ? ck.tile_pairs : ck.tile_keys;
-    if (msd) {
-        // One pass by digit 3 into the alternate buffers (skipped unless the
-        // plan chose this order), then every bucket on chip back into the
-        // caller's arrays.
-        st = pairs ? launch_onesweep_pairs(cfg, false, keys, vals, alt_k, alt_v, n, PASSES - 1,
-                                           MSD_SLOT, ctrl, di.sticky, status[0], nullptr, nullptr,
-                                           KEY_U32, stream)
-                   : launch_onesweep_keys(cfg, false, keys, alt_k, n, PASSES - 1, MSD_SLOT, ctrl,
-                                          di.sticky, status[0], nullptr, nullptr, KEY_U32, stream);
-        if (st != RS_OK) return st;
-        // (Usual buckets of evenly spread keys hold less than twice the average.)
-        st = launch_bucket_sorts(keys, vals, alt_k, alt_v, msd_off, &ctrl->small_count, ctrl,
-                                 n / RADIX * 2, ck.small_bits, KEY_U32, stream);
-        if (st != RS_OK) return st;
-    }
     for (uint32_t p = 0; p < PASSES; ++p) {
         void* cur = status[p & 1];
         void* next = p + 1 < PASSES ? status[(p + 1) & 1] : nullptr;
+        // Pass 3 is the MSD-first order's only pass (into the alternate
+        // buffers) when the plan chose it.
+        const uint32_t kt = key_type | (msd && p == PASSES - 1 ? ROLE_MSD_TOO : 0u);
         st = pairs ? launch_onesweep_pairs(cfg, L.wide_status, keys, vals, alt_k, alt_v, n, p, p,
-                                           ctrl, di.sticky, cur, next, nullptr, key_type, stream)
+                                           ctrl, di.sticky, cur, next, nullptr, kt, stream)
                    : launch_onesweep_keys(cfg, L.wide_status, keys, alt_k, n, p, p, ctrl, di.sticky,
-                                          cur, next, nullptr, key_type, stream);
+                                          cur, next, nullptr, kt, stream);
         if (st != RS_OK) return st;
+    }
+    if (msd)  // every bucket on chip, back into the caller's arrays
+        return launch_bucket_sorts(keys, vals, alt_k, alt_v, msd_off, &ctrl->small_count, ctrl,
+                                   long_buckets, ck.small_bits, key_type, stream);
+    if (top.bits != 0) {
+        // The array is sorted by its top 16 bits (or finished, if the plan
+        // chose the four passes); the status words are free for the table.
+        uint32_t* const off = static_cast<uint32_t*>(status[0]);
+        note_launch_begin(KK_CHUNK_BOUNDS, stream);
+        const uint32_t ways = top.bits <= 14 ? 32 : 8;
+        const cudaError_t be = launch_after_previous(
+            ways == 32 ? k_chunk_bounds<uint32_t, 32> : k_chunk_bounds<uint32_t, 8>,
+            dim3((ways << top.bits) / 256), dim3(256), 0, stream, (const uint32_t*)keys, n,
+            (const Ctrl*)ctrl, top.bits, key_type, off);
+        note_launch_end(KK_CHUNK_BOUNDS, stream);
+        if (be != cudaSuccess) return RS_ERR_CUDA;
+        return launch_chunk_sorts(keys, vals, alt_k, alt_v, off, &ctrl->chunk_count, ctrl,
+                                  top, key_type, stream);
     }
     return RS_OK;
 }

@@ -123,15 +123,9 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
                            status_bytes, key_type, stream);
         if (st != RS_OK) return st;
     }
-    note_launch_begin(KK_PLAN, stream);
-    uint32_t* const no_buckets = nullptr;
-    const cudaError_t pe =
-        key64 ? launch_after_previous(k_plan<PASSES64>, dim3(1), dim3(1024), 0, stream, ctrl, n,
-                                      0u, 0u, no_buckets)
-              : launch_after_previous(k_plan<PASSES>, dim3(1), dim3(1024), 0, stream, ctrl, n, 0u,
-                                      0u, no_buckets);
-    note_launch_end(KK_PLAN, stream);
-    if (pe != cudaSuccess) return RS_ERR_CUDA;
+    const PlanArgs plan{ctrl, keys, n, key_type, 0u, nullptr, 0u};
+    st = key64 ? enqueue_plan<PASSES64>(plan, stream) : enqueue_plan<PASSES>(plan, stream);
+    if (st != RS_OK) return st;
 
     for (uint32_t p = 0; p < npass; ++p) {
         void* cur = status[p & 1];
