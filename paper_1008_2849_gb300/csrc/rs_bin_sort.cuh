@@ -108,7 +108,6 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
                                             uint32_t key_type, uint32_t* s_cnt, uint32_t* s_base,
                                             uint32_t* s_hist) {
     constexpr uint32_t WARPS = THREADS / 32, SLOTS = 4, TILE = THREADS * SLOTS;
-    static_assert(THREADS >= (int)RADIX, "one thread per digit");
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = lanemask_lt();
     bool in_a = true;
@@ -120,16 +119,16 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
         auto digit = [&](K k) {
             return (uint32_t)(key_to_ordered(k, key_type) >> (8 * p)) & (RADIX - 1);
         };
-        if (tid < RADIX) s_hist[tid] = 0;
+        for (uint32_t d = tid; d < RADIX; d += THREADS) s_hist[d] = 0;
         __syncthreads();
         for (uint32_t i = tid; i < m; i += THREADS) atomicAdd(&s_hist[digit(sk[i])], 1u);
         __syncthreads();
         bool trivial = false;
-        if (tid < RADIX) {
+        for (uint32_t d = tid; d < RADIX; d += THREADS) {
             uint32_t before = 0;
-            for (uint32_t d = 0; d < tid; ++d) before += s_hist[d];
-            s_base[tid] = before;
-            trivial = s_hist[tid] == m;
+            for (uint32_t q = 0; q < d; ++q) before += s_hist[q];
+            s_base[d] = before;
+            trivial |= s_hist[d] == m;
         }
         if (__syncthreads_or(trivial)) continue;  // one digit only: the identity
         for (uint32_t t0 = 0; t0 < m; t0 += TILE) {
@@ -154,14 +153,14 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
                 at[j] = before + __popc(peers & lt);
             }
             __syncthreads();
-            if (tid < RADIX) {
-                uint32_t run = s_base[tid];
+            for (uint32_t d = tid; d < RADIX; d += THREADS) {
+                uint32_t run = s_base[d];
                 for (uint32_t w = 0; w < WARPS; ++w) {
-                    const uint32_t c = s_cnt[w * RADIX + tid];
-                    s_cnt[w * RADIX + tid] = run;
+                    const uint32_t c = s_cnt[w * RADIX + d];
+                    s_cnt[w * RADIX + d] = run;
                     run += c;
                 }
-                s_base[tid] = run;
+                s_base[d] = run;
             }
             __syncthreads();
 #pragma unroll

@@ -85,15 +85,23 @@ struct ClassKnobs {
 // (the largest bucket of evenly spread keys stays seven or more standard deviations below).
 constexpr uint32_t kMsdShortItems = 256u * 4600u;
 constexpr uint32_t kMsdMaxItems = 256u * 7400u;
-// Arrays of kTopMinItems and more may take the top-digits order: two scatter passes,
-// then chunks of the keys' `bits` highest bits sorted on chip, by a CTA of 4608 items,
-// or 8192 for long_chunks.  bits = 0: not tried.
+// Large arrays may take the top-digits order: two scatter passes, then chunks of the
+// keys' `bits` highest bits sorted on chip by a CTA of `capacity` items (rs_chunks.cu).
+// bits = 0: not tried.  32-bit keys from kTopMinItems on (where the saved passes outweigh
+// what keys that do not spread pay for the launches: 18 us, 3 % of 2^25 keys), 64-bit
+// keys, which save six passes of eight, from kTopMinItems64.
 constexpr uint32_t kTopMinItems = 1u << 25;
+constexpr uint32_t kTopMinItems64 = 1u << 14;
 struct TopOrder {
-    uint32_t bits;
-    bool long_chunks;
+    uint32_t bits, capacity;
 };
 TopOrder top_order(size_t n);
+TopOrder top_order_wide(size_t n, bool key64);
+// The end of that order, once the passes are enqueued: off is a table of 2^bits + 1 words
+// in the workspace; the spare arrays are the other buffers of the passes.
+rs_status enqueue_chunks(void* keys, void* vals, void* spare_keys, void* spare_vals, uint32_t n,
+                         uint32_t key_type, uint32_t val_bytes, const Ctrl* ctrl, uint32_t* off,
+                         TopOrder top, cudaStream_t stream);
 // Size classes by item count (whole array; for a segmented sort the average
 // segment): <= 2^13, <= 2^16, <= 2^20, <= 2^24, <= 2^28, larger.
 constexpr int NUM_SIZE_CLASSES = 6;
@@ -224,13 +232,6 @@ rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* sr
                               const uint32_t* src_vals, const uint32_t* off,
                               const uint32_t* count, const Ctrl* ctrl, bool long_buckets,
                               int bits, uint32_t key_type, cudaStream_t stream);
-// On-chip sorts, in place, of the chunks 0 .. *count - 1 of the top-digits order
-// (off[c] .. off[c + 1]); longer ones than the chip takes are sorted in global
-// memory through the spare arrays (of the same size as keys / vals).
-rs_status launch_chunk_sorts(uint32_t* keys, uint32_t* vals, uint32_t* spare_keys,
-                             uint32_t* spare_vals, const uint32_t* off, const uint32_t* count,
-                             const Ctrl* ctrl, TopOrder top, uint32_t key_type,
-                             cudaStream_t stream);
 // The segments listed by size (rs_bin_sort.cuh list_small) in tiny_list and
 // small_list of `entries` entries each, in place: one launch per size up to
 // max_items.

@@ -29,14 +29,12 @@ rs_status grid_of(const SmallWork& w, uint32_t per_sm, uint32_t* grid) {
     return st;
 }
 
-// The word of the bin sort: the key alone; for pairs 64 bits, or in chunks, whose
-// keys have few bits left, 32.
-template <bool PAIRS, int THREADS, int MIN_BLOCKS, bool CHUNKS = false>
-rs_status launch_bin_shape(const SmallWork& w, cudaStream_t stream, uint32_t* spare_keys = nullptr,
-                           uint32_t* spare_vals = nullptr) {
-    using W = std::conditional_t<PAIRS && !CHUNKS, unsigned long long, uint32_t>;
-    using L = BinSortSmem<uint32_t, uint32_t, W, PAIRS, THREADS, CHUNKS>;
-    auto kern = k_bin_sort<uint32_t, uint32_t, W, PAIRS, THREADS, MIN_BLOCKS, CHUNKS>;
+// The word of the bin sort: the key alone; for pairs 64 bits.
+template <bool PAIRS, int THREADS, int MIN_BLOCKS>
+rs_status launch_bin_shape(const SmallWork& w, cudaStream_t stream) {
+    using W = std::conditional_t<PAIRS, unsigned long long, uint32_t>;
+    using L = BinSortSmem<uint32_t, uint32_t, W, PAIRS, THREADS, false>;
+    auto kern = k_bin_sort<uint32_t, uint32_t, W, PAIRS, THREADS, MIN_BLOCKS, false>;
     static DeviceOnce smem_set;
     rs_status st = allow_smem_once(kern, L::BYTES, smem_set);
     if (st != RS_OK) return st;
@@ -46,8 +44,8 @@ rs_status launch_bin_shape(const SmallWork& w, cudaStream_t stream, uint32_t* sp
     note_launch_begin(KK_SMALL, stream);
     const cudaError_t e = launch_after_previous(
         kern, dim3(grid), dim3(THREADS), L::BYTES, stream, w.keys, w.vals, w.src_keys, w.src_vals,
-        w.off, w.list, w.step, w.list_count, w.ctrl, w.single_n, w.key_type, spare_keys,
-        spare_vals);
+        w.off, w.list, w.step, w.list_count, w.ctrl, w.single_n, w.key_type,
+        (uint32_t*)nullptr, (uint32_t*)nullptr);
     note_launch_end(KK_SMALL, stream);
     return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
@@ -126,20 +124,6 @@ rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* sr
     if (long_buckets || bits == 4) return launch_small_any(small_sort_capacity(), bits, w, stream);
     return vals != nullptr ? launch_bin_shape<true, 640, 2>(w, stream)
                            : launch_bin_shape<false, 640, 2>(w, stream);
-}
-
-rs_status launch_chunk_sorts(uint32_t* keys, uint32_t* vals, uint32_t* spare_keys,
-                             uint32_t* spare_vals, const uint32_t* off, const uint32_t* count,
-                             const Ctrl* ctrl, TopOrder top, uint32_t key_type,
-                             cudaStream_t stream) {
-    const SmallWork w{keys, vals, keys, vals, off, nullptr, 1, count, ctrl, top.bits, key_type};
-    // (Index bits <= top.bits: a word holds the index and the bits that differ.)
-    const bool pairs = vals != nullptr;
-    if (top.long_chunks)
-        return pairs ? launch_bin_shape<true, 1024, 1, true>(w, stream, spare_keys, spare_vals)
-                     : launch_bin_shape<false, 1024, 1, true>(w, stream, spare_keys, nullptr);
-    return pairs ? launch_bin_shape<true, 576, 2, true>(w, stream, spare_keys, spare_vals)
-                 : launch_bin_shape<false, 576, 2, true>(w, stream, spare_keys, nullptr);
 }
 
 rs_status launch_small_lists(uint32_t* keys, uint32_t* vals, const uint32_t* off,

@@ -43,18 +43,6 @@ Layout layout_for(size_t n, bool pairs) {
     return L;
 }
 
-// The fewest chunks whose average is at most 4096 items, or 7400 for the largest
-// arrays: eight standard deviations or more below what the CTA takes, for evenly
-// spread keys.  (32-bit words hold an index of 13 bits and the 32 - bits low bits
-// of a key: bits >= 13.)
-TopOrder top_order(size_t n) {
-    if (n < kTopMinItems) return {0, false};
-    for (uint32_t bits = 13; bits <= TOP_MAX_BITS; ++bits)
-        if ((n >> bits) <= 4096) return {bits, false};
-    if ((n >> TOP_MAX_BITS) <= 7400) return {TOP_MAX_BITS, true};
-    return {0, false};
-}
-
 rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* clear,
                         size_t clear_bytes, uint32_t key_type, cudaStream_t stream) {
     DeviceInfo di;
@@ -195,7 +183,7 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     // top-digits order likewise.
     const bool msd = ck.msd != 0 && n <= kMsdMaxItems;
     const bool long_buckets = n > kMsdShortItems;
-    const TopOrder top = ck.msd != 0 ? top_order(n) : TopOrder{0, false};
+    const TopOrder top = ck.msd != 0 ? top_order(n) : TopOrder{0, 0};
     uint32_t* msd_off = reinterpret_cast<uint32_t*>(ws + L.msd_off);
     const PlanArgs plan{ctrl, keys, n, key_type, bucket_capacity(long_buckets),
                         msd ? msd_off : nullptr, top.bits};
@@ -222,21 +210,11 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     if (msd)  // every bucket on chip, back into the caller's arrays
         return launch_bucket_sorts(keys, vals, alt_k, alt_v, msd_off, &ctrl->small_count, ctrl,
                                    long_buckets, ck.small_bits, key_type, stream);
-    if (top.bits != 0) {
-        // The array is sorted by its top 16 bits (or finished, if the plan
-        // chose the four passes); the status words are free for the table.
-        uint32_t* const off = static_cast<uint32_t*>(status[0]);
-        note_launch_begin(KK_CHUNK_BOUNDS, stream);
-        const uint32_t ways = top.bits <= 14 ? 32 : 8;
-        const cudaError_t be = launch_after_previous(
-            ways == 32 ? k_chunk_bounds<uint32_t, 32> : k_chunk_bounds<uint32_t, 8>,
-            dim3((ways << top.bits) / 256), dim3(256), 0, stream, (const uint32_t*)keys, n,
-            (const Ctrl*)ctrl, top.bits, key_type, off);
-        note_launch_end(KK_CHUNK_BOUNDS, stream);
-        if (be != cudaSuccess) return RS_ERR_CUDA;
-        return launch_chunk_sorts(keys, vals, alt_k, alt_v, off, &ctrl->chunk_count, ctrl,
-                                  top, key_type, stream);
-    }
+    // The array is sorted by its top 16 bits (or finished, if the plan chose the
+    // four passes); the status words are free for the table of chunks.
+    if (top.bits != 0)
+        return enqueue_chunks(keys, vals, alt_k, alt_v, n, key_type, pairs ? 4u : 0u, ctrl,
+                              static_cast<uint32_t*>(status[0]), top, stream);
     return RS_OK;
 }
 

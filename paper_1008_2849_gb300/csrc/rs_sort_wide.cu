@@ -123,7 +123,10 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
                            status_bytes, key_type, stream);
         if (st != RS_OK) return st;
     }
-    const PlanArgs plan{ctrl, keys, n, key_type, 0u, nullptr, 0u};
+    // Keys that spread evenly: two passes, then chunks on chip (see enqueue_sort).
+    const TopOrder top = knobs().cls[size_class(n)].msd != 0 ? top_order_wide(n, key64)
+                                                             : TopOrder{0, 0};
+    const PlanArgs plan{ctrl, keys, n, key_type, 0u, nullptr, top.bits};
     st = key64 ? enqueue_plan<PASSES64>(plan, stream) : enqueue_plan<PASSES>(plan, stream);
     if (st != RS_OK) return st;
 
@@ -143,6 +146,9 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
                                     di.sticky, cur, next, stream);
         if (st != RS_OK) return st;
     }
+    if (top.bits != 0)
+        return enqueue_chunks(keys, vals, alt_k, alt_v, n, key_type, val_bytes, ctrl,
+                              static_cast<uint32_t*>(status[0]), top, stream);
     return RS_OK;
 }
 

@@ -94,3 +94,49 @@ def test_chunk_sizes(rs, n):
     kd.copy_(k0)
     rs.sort_keys(kd)
     assert np.array_equal(to_host(kd), ko)
+
+
+def _wide_keys(kind, n, seed, bits):
+    k = inputs.splitmix32(seed, n, 0).astype(np.uint64)
+    if bits == 32:
+        return k.astype(np.uint32)
+    k = (k << np.uint64(32)) | inputs.splitmix32(seed, n, 1).astype(np.uint64)
+    if kind == "long chunks":  # one prefix with 1500 keys more, their low words nearly equal
+        k[7:3007:2] = (k[7:3007:2] & np.uint64(0x3)) | np.uint64(0x1234000000000000)
+    elif kind == "equal low":  # chunks of few distinct keys
+        k &= np.uint64(0xFFFFFF0000000000)
+    return k
+
+
+@pytest.mark.parametrize("n", [(1 << 14) - 1, 1 << 14, 100_003, (1 << 20) + 5, 3_000_001])
+@pytest.mark.parametrize("key_type,value_bits", [("u64", 0), ("u64", 32), ("i64", 64), ("f64", 32),
+                                                 ("f64", 64)])
+def test_wide_keys(rs, n, key_type, value_bits):
+    for kind in ("uniform", "long chunks", "equal low"):
+        if kind != "uniform" and n < (1 << 20):
+            continue
+        k = _wide_keys(kind, n, 80 + n % 17, 64)
+        v = None
+        if value_bits:
+            v = np.arange(n, dtype=np.uint64 if value_bits == 64 else np.uint32)
+        import torch
+        signed = np.int64 if value_bits == 64 else np.int32
+        kd = torch.from_numpy(k.view(np.int64)).cuda()
+        vd = None if v is None else torch.from_numpy(v.view(signed)).cuda()
+        rs.sort_kv(kd, vd, key_type)
+        ko, vo = oracle.sort_kv(k, v, key_type)
+        assert np.array_equal(kd.cpu().numpy().view(np.uint64), ko), kind
+        if v is not None:
+            assert np.array_equal(vd.cpu().numpy().view(v.dtype), vo), kind
+
+
+def test_32_bit_keys_with_64_bit_values(rs):
+    import torch
+    n = FIRST + 3
+    k = inputs.keys("uniform", n, 91)
+    v = np.arange(n, dtype=np.uint64) << np.uint64(20)
+    kd, vd = to_dev(k), torch.from_numpy(v.view(np.int64)).cuda()
+    rs.sort_kv(kd, vd, "i32")
+    place = np.argsort(k.view(np.int32), kind="stable")
+    assert np.array_equal(to_host(kd), k[place])
+    assert np.array_equal(vd.cpu().numpy().view(np.uint64), v[place])
