@@ -319,7 +319,7 @@ static rs_status plain_segmented(uint32_t* keys, uint32_t* vals, size_t n,
     st = device_info_for(dev, &di);
     if (st != RS_OK) return st;
     DevState& d = g_dev[dev];
-    st = ensure_workspace_locked(d, seg_layout_for(n, vals != nullptr, num_segments).total);
+    st = ensure_workspace_locked(d, seg_layout_for(n, vals != nullptr, num_segments).routed_total);
     if (st != RS_OK) return st;
     st = enqueue_sort_segmented(keys, vals, (uint32_t)n, offsets, num_segments, cudaStreamLegacy,
                                 d.ws, d.ws_bytes);
@@ -382,7 +382,7 @@ rs_status rs_sort_pairs_segmented_ex(uint32_t* d_keys, uint32_t* d_vals, size_t 
 
 size_t rs_workspace_bytes(size_t n, int with_values, uint32_t num_segments) {
     if (n == 0) return 0;
-    if (num_segments > 0) return seg_layout_for(n, with_values != 0, num_segments).total;
+    if (num_segments > 0) return seg_layout_for(n, with_values != 0, num_segments).routed_total;
     return sort_workspace_bytes(n, with_values != 0);
 }
 
@@ -449,7 +449,7 @@ size_t rs_workspace_bytes_kv_segmented(size_t n, int key_type, int value_bits,
                                        uint32_t num_segments) {
     if (n == 0 || num_segments == 0 || !valid_kv_types(key_type, value_bits)) return 0;
     if (kv_is_narrow(key_type, value_bits))
-        return seg_layout_for(n, value_bits != 0, num_segments).total;
+        return seg_layout_for(n, value_bits != 0, num_segments).routed_total;
     return seg_layout_wide(n, key_type >= RS_KEY_U64, (uint32_t)value_bits / 8, num_segments)
         .total;
 }

@@ -17,21 +17,39 @@ namespace rs {
 constexpr uint32_t SMALL_SHORT_MAX = 1024;
 constexpr uint32_t SMALL_MID_MAX = 4096;
 
-// Lists segment s of `size` items (more than warp_max, or tiny); `last` is the
-// last entry of either array.
+// Lists segment s of `size` items where it holds two or more (called by whole warps;
+// one atomic per warp and list); `last` is the last entry of either array.
 __device__ __forceinline__ void list_small(Ctrl* ctrl, uint32_t s, uint32_t size,
                                            uint32_t warp_max, uint32_t last, uint32_t* tiny,
                                            uint32_t* small) {
-    if (size <= warp_max) tiny[atomicAdd(&ctrl->tiny_count, 1u)] = s;
-    else if (size <= SMALL_SHORT_MAX) small[atomicAdd(&ctrl->small_count, 1u)] = s;
-    else if (size <= SMALL_MID_MAX) small[last - atomicAdd(&ctrl->mid_count, 1u)] = s;
-    else tiny[last - atomicAdd(&ctrl->big_count, 1u)] = s;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t kind = size < 2                  ? 4u
+                          : size <= warp_max        ? 0u
+                          : size <= SMALL_SHORT_MAX ? 1u
+                          : size <= SMALL_MID_MAX   ? 2u
+                                                    : 3u;
+    uint32_t* const counts[4] = {&ctrl->tiny_count, &ctrl->small_count, &ctrl->mid_count,
+                                 &ctrl->big_count};
+#pragma unroll
+    for (uint32_t c = 0; c < 4; ++c) {
+        const uint32_t of_kind = __ballot_sync(0xffffffffu, kind == c);
+        if (of_kind == 0) continue;
+        uint32_t first = 0;
+        if (lane == 0) first = atomicAdd(counts[c], (uint32_t)__popc(of_kind));
+        first = __shfl_sync(0xffffffffu, first, 0) + __popc(of_kind & lanemask_lt());
+        if (kind != c) continue;
+        if (c == 0) tiny[first] = s;
+        if (c == 1) small[first] = s;
+        if (c == 2) small[last - first] = s;
+        if (c == 3) tiny[last - first] = s;
+    }
 }
 
 // Shared-memory plan of k_bin_sort: bin words (or the counters of the digit
-// passes), binned words with room for the last windows' padding, values in input
-// order, and the list of bins that the windows do not cover.
-template <typename K, typename V, typename W, bool PAIRS, int THREADS, bool CHUNKS>
+// passes), binned words with room for the last windows' padding, keys (unless words
+// hold them whole) and values in input order, and the list of bins that the windows
+// do not cover.
+template <typename K, typename V, bool PAIRS, int THREADS, bool CHUNKS>
 struct BinSortSmem {
     static constexpr uint32_t ITEMS = 8;  // a thread's items, and the width of a window
     static constexpr uint32_t CAP = THREADS * ITEMS;
@@ -44,24 +62,29 @@ struct BinSortSmem {
                                          : THREADS >= 256 ? 256 : 128;
     static constexpr uint32_t COUNTERS = (THREADS / 32) * RADIX * 4;
     static constexpr uint32_t BINS = MAX_BINS * 4 > COUNTERS ? MAX_BINS * 4 : COUNTERS;
-    static constexpr uint32_t WORDS = (CAP + 2 * ITEMS) * (uint32_t)sizeof(W);
+    static constexpr uint32_t WORDS = (CAP + 2 * ITEMS) * (uint32_t)sizeof(K);
+    static constexpr uint32_t KEYS = PAIRS && !CHUNKS ? CAP * (uint32_t)sizeof(K) : 0;
     static constexpr uint32_t VALS = PAIRS ? CAP * (uint32_t)sizeof(V) : 0;
     static constexpr uint32_t BIG = (CAP / 6 + 1) * 4;
-    static constexpr size_t BYTES = BINS + WORDS + VALS + BIG;
+    static constexpr size_t BYTES = BINS + WORDS + KEYS + VALS + BIG;
     static_assert(BINS % 16 == 0 && WORDS % 16 == 0 && VALS % 16 == 0, "aligned parts");
 };
 
-__device__ __forceinline__ uint32_t warp_or(uint32_t x) {
-    return __reduce_or_sync(0xffffffffu, x);
+__device__ __forceinline__ uint32_t warp_min(uint32_t x) {
+    return __reduce_min_sync(0xffffffffu, x);
 }
-__device__ __forceinline__ unsigned long long warp_or(unsigned long long x) {
-    return ((unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)(x >> 32)) << 32) |
-           __reduce_or_sync(0xffffffffu, (uint32_t)x);
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long x) {
+    const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(x >> 32));
+    const uint32_t lo =
+        __reduce_min_sync(0xffffffffu, (uint32_t)(x >> 32) == hi ? (uint32_t)x : 0xffffffffu);
+    return ((unsigned long long)hi << 32) | lo;
 }
-__device__ __forceinline__ uint32_t significant_bits(uint32_t x) { return 32u - __clz(x); }
-__device__ __forceinline__ uint32_t significant_bits(unsigned long long x) {
-    return 64u - __clzll((long long)x);
+__device__ __forceinline__ uint32_t leading_zeros(uint32_t x) { return __clz(x); }
+__device__ __forceinline__ uint32_t leading_zeros(unsigned long long x) {
+    return __clzll((long long)x);
 }
+__device__ __forceinline__ uint32_t high_word(uint32_t x) { return x; }
+__device__ __forceinline__ uint32_t high_word(unsigned long long x) { return (uint32_t)(x >> 32); }
 
 // Batcher's odd-even merge sort of eight words in registers.
 template <typename W>
@@ -188,18 +211,17 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
 // k_bin_sort: sorts arrays of 2 to CAP = 8 * THREADS items, one CTA per array,
 // each item read from and written to global memory once.  Arrays are the segments
 // listed in `list` (every `step`-th entry from it; count in *list_count), or with
-// list == nullptr those of the segments 0, 1, ... that hold more than single_n
-// items and at most CAP; or with off == nullptr the single array [0, single_n).
+// list == nullptr the segments 0, 1, ..., or with step == 0 the ranges (first item,
+// items) in `list`; or with off == nullptr the single array [0, single_n).
 // CHUNKS: the segments 0, 1, ... (list == nullptr), sorted in place; longer ones
 // than CAP in global memory, with the other buffer at spare_keys / spare_vals
 // (sort_in_global); their keys share the single_n highest bits.
 //
 // For an array of m items, with nb = 2^bb bins (m <= nb < 2m; chunks at most
 // MAX_BINS):
-//  1. The keys' bits that differ (an OR over the array) say where the bb
-//     highest of them lie; those are the item's bin.  Every item adds one to
-//     its bin and keeps the count before it: its place among the bin's items,
-//     in no particular order.
+//  1. The smallest and the largest key cut the range between them into nb bins of
+//     the same width.  Every item adds one to its bin and keeps the count before
+//     it: its place among the bin's items, in no particular order.
 //  2. The exclusive prefix over bins gives every bin's first position.  Every
 //     item writes its word to its bin's next position: the key, and for
 //     key-value items its index below it, so that the words of a whole array
@@ -216,9 +238,11 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
 // stable counting pass per 8-bit digit that differs instead: ranks from ballots
 // and per-warp counters, items exchanged through shared memory.
 //
-// The word: W = K without values; 64-bit words hold any 32-bit key and its index;
-// 32-bit words (64-bit for 64-bit keys) hold the index and the low bits of the
-// key where the others are the same in the whole array, as in chunks.
+// The word has the width of the key: the key itself without values; else the key's
+// distance from the smallest, moved up until the largest has its highest bit set, with
+// the index in the lowest bits.  In chunks, whose keys share as many bits as an index
+// takes, that is the whole key.  Elsewhere its lowest bits may be lost: words that differ in their index only are put in order by their
+// keys in step 4 (for 4096 keys that spread evenly, eight such pairs).
 //
 // What bounds it: instruction issue (135 warp instructions per 32 pairs, 61 % of the
 // issue slots) and shared-memory wavefronts (28 per 32 pairs: counting atomic, bin
@@ -258,28 +282,30 @@ __device__ __forceinline__ void sort_bin(W* bin, uint32_t c, uint32_t lane) {
         if (r * 32 + lane < c) bin[pos[r]] = w[r];
 }
 
-template <typename K, typename V, typename W, bool PAIRS, int THREADS, int MIN_BLOCKS,
+template <typename K, typename V, bool PAIRS, int THREADS, int MIN_BLOCKS,
           bool CHUNKS = false>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
 k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
            const uint32_t* __restrict__ off, const uint32_t* __restrict__ list, int32_t step,
            const uint32_t* __restrict__ list_count, const Ctrl* __restrict__ ctrl,
            uint32_t single_n, uint32_t key_type, K* spare_keys, V* spare_vals) {
-    using L = BinSortSmem<K, V, W, PAIRS, THREADS, CHUNKS>;
+    using L = BinSortSmem<K, V, PAIRS, THREADS, CHUNKS>;
+    constexpr bool WHOLE = !PAIRS || CHUNKS;  // words hold whole keys
     constexpr int ITEMS = L::ITEMS;
     constexpr uint32_t WARPS = THREADS / 32;
     constexpr uint32_t SCANNERS = L::SCANNERS;
     static_assert(WARPS <= 32 && L::CAP <= 65535, "one lane per warp total; 16-bit counts");
-    static_assert(sizeof(W) >= sizeof(K), "a word holds a key");
     pdl_launch_next();
     pdl_wait();  // the kernel before this one (planner, scatter pass) is complete
     extern __shared__ uint4 s_dyn[];
     uint32_t* const s_bin = reinterpret_cast<uint32_t*>(s_dyn);
-    W* const s_w = reinterpret_cast<W*>(reinterpret_cast<char*>(s_dyn) + L::BINS);
-    V* const s_v = reinterpret_cast<V*>(reinterpret_cast<char*>(s_dyn) + L::BINS + L::WORDS);
-    uint32_t* const s_big = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(s_dyn) + L::BINS +
-                                                        L::WORDS + L::VALS);
-    __shared__ K s_or;
+    char* const parts = reinterpret_cast<char*>(s_dyn) + L::BINS;
+    K* const s_w = reinterpret_cast<K*>(parts);
+    K* const s_k = reinterpret_cast<K*>(parts + L::WORDS);
+    V* const s_v = reinterpret_cast<V*>(parts + L::WORDS + L::KEYS);
+    uint32_t* const s_big =
+        reinterpret_cast<uint32_t*>(parts + L::WORDS + L::KEYS + L::VALS);
+    __shared__ K s_min, s_max;
     __shared__ uint32_t s_sum[32], s_work[32];
     __shared__ uint32_t s_bigs;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -290,14 +316,19 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         count = *list_count;
     }
     const bool typed = key_type != KEY_U32 && key_type != KEY_U64;
-    if (tid == 0) s_or = 0, s_bigs = 0;
+    if (tid == 0) s_min = ~K(0), s_max = 0, s_bigs = 0;
     for (uint32_t idx = blockIdx.x; idx < count; idx += gridDim.x) {
         uint32_t lo = 0, m = single_n;
         if (off != nullptr) {
-            const uint32_t s = !CHUNKS && list != nullptr ? list[(ptrdiff_t)idx * step] : idx;
-            lo = off[s];
-            m = off[s + 1] - lo;
-            if (!CHUNKS && list == nullptr && (m <= single_n || m > L::CAP)) continue;
+            if (!CHUNKS && step == 0) {
+                lo = list[2 * idx];
+                m = list[2 * idx + 1];
+            } else {
+                const uint32_t s = !CHUNKS && list != nullptr ? list[(ptrdiff_t)idx * step] : idx;
+                lo = off[s];
+                m = off[s + 1] - lo;
+            }
+            if (!CHUNKS && (m == 0 || m > L::CAP)) continue;
             if (CHUNKS && m < 2) continue;
             if constexpr (CHUNKS) {
                 if (m > L::CAP) {
@@ -322,39 +353,57 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         const uint32_t nb = 1u << bb;
         for (uint32_t b = tid; b < (nb + 3) / 4; b += THREADS)
             reinterpret_cast<uint4*>(s_bin)[b] = make_uint4(0, 0, 0, 0);
-        const K first = key_to_ordered(from[0], key_type);
-        K varying = ~K(0) >> (CHUNKS ? single_n : 0u), diff = 0;
         if (typed) {
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) k[j] = key_to_ordered(k[j], key_type);
         }
-        if (!CHUNKS) {
+        // Chunks: their keys share the single_n highest bits.
+        K least, most, range = ~K(0) >> (CHUNKS ? single_n : 0u);
+        if constexpr (CHUNKS) {
+            least = key_to_ordered(from[0], key_type) & ~range;
+            most = least | range;
+            __syncthreads();  // the bins are zero; the array before is done with the rest
+        } else {
+            K lo_k = ~K(0), not_hi = ~K(0);
 #pragma unroll
-            for (int j = 0; j < ITEMS; ++j)
-                if (tid + j * THREADS < m) diff |= k[j] ^ first;
+            for (int j = 0; j < ITEMS; ++j) {
+                if (tid + j * THREADS < m) {
+                    lo_k = min(lo_k, k[j]);
+                    not_hi = min(not_hi, ~k[j]);
+                }
+            }
+            lo_k = warp_min(lo_k);
+            not_hi = warp_min(not_hi);
+            __syncthreads();  // s_min, s_max and the bins are set; as above
+            if (lane == 0) {
+                atomicMin(&s_min, lo_k);
+                atomicMax(&s_max, ~not_hi);
+            }
+            __syncthreads();
+            least = s_min;
+            most = s_max;
+            range = (most - least) | 1;
         }
-        __syncthreads();  // the bins are zero; the array before is done with the words and values
         if (PAIRS) {
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
                 if (tid + j * THREADS < m)
                     cp_async_elem(s_v + tid + j * THREADS, src_vals + lo + tid + j * THREADS);
         }
-        if (!CHUNKS) {
-            diff = warp_or(diff);
-            if (lane == 0 && diff != 0) atomicOr(&s_or, diff);
-            __syncthreads();
-            varying = s_or;
-        }
-        const uint32_t sig = significant_bits(varying);
-        const uint32_t shift = sig > bb ? sig - bb : 0u;
+        const uint32_t top = CHUNKS ? single_n : leading_zeros(range);  // zero bits of a distance
+        // Bins: distance * scale / 2^32, of the (high words of the) distances moved up
+        // by `top`; scale = nb * 2^32 / (range + 1), rounded down.
+        const uint32_t scale =
+            CHUNKS ? nb
+                   : (uint32_t)(((unsigned long long)nb << 32) /
+                                ((unsigned long long)high_word((K)(range << top)) + 1));
         // Scanning thread t scans the `per` consecutive bins from t * per on,
         // four at a time; their groups of four are swizzled so that the eight
         // lanes of a 16-byte access fall into 32 different banks.
         const uint32_t per = nb > SCANNERS ? nb / SCANNERS : 1u;  // 1, 2, 4, 8 or 16
         const uint32_t swizzle = per > 4 ? (per / 4 - 1) << 2 : 0u;
         auto bin_of = [&](K x) {
-            const uint32_t b = (uint32_t)(x >> shift) & (nb - 1);
+            const uint32_t b = __umulhi(high_word((K)((CHUNKS ? x : x - least) << top)), scale);
             return b ^ ((b >> 3) & swizzle);
         };
 
@@ -448,26 +497,31 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         else if (per == 4 || MAX_PER == 4) work = scan_bins(std::integral_constant<uint32_t, 4>{});
         else if (per == 8 || MAX_PER == 8) work = scan_bins(std::integral_constant<uint32_t, 8>{});
         else work = scan_bins(std::integral_constant<uint32_t, MAX_PER>{});
-        if (tid == 0) s_or = 0;  // for the next array
+        if (tid == 0) s_min = ~K(0), s_max = 0;  // for the next array
         __syncthreads();
         const uint32_t bigs = s_bigs;
 
-        // Words that the word type cannot hold in order (see above) take the
-        // digit passes too; the callers' choices of W leave none.
-        if (work <= m && sig + ib <= 8 * sizeof(W)) {
+        // (Chunks whose words would not hold whole keys take the digit passes too;
+        // the choice of chunks leaves none.)
+        if (work <= m && (!CHUNKS || ib <= top)) {
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
-                if (tid + j * THREADS < m)
-                    s_w[s_bin[bin_of(k[j])] + at[j]] =
-                        ((W)k[j] << ib) | (PAIRS ? (W)(tid + j * THREADS) : W(0));
+                if (tid + j * THREADS < m) {
+                    const uint32_t i = tid + j * THREADS;
+                    K w = k[j];
+                    if (PAIRS && CHUNKS) w = (w << top) | (K)i;  // (least << top is 0)
+                    if (PAIRS && !CHUNKS) w = ((w - least) << top >> ib << ib) | (K)i;
+                    s_w[s_bin[bin_of(k[j])] + at[j]] = w;
+                    if (!WHOLE) s_k[i] = k[j];
+                }
             // Padding above every word, to the end of the last window.
             const uint32_t windows = (m + 7) / 8;
-            if (tid < 8 * windows + 8 - m) s_w[m + tid] = ~W(0);
+            if (tid < 8 * windows + 8 - m) s_w[m + tid] = ~K(0);
             __syncthreads();
             // ---- 3. the order inside bins ----------------------------------
             if (bigs != 0) {
                 for (uint32_t g = warp; g < bigs; g += WARPS) {
-                    sort_bin<W, !PAIRS>(s_w + (s_big[g] & 0xffffu), s_big[g] >> 16, lane);
+                    sort_bin<K, !PAIRS>(s_w + (s_big[g] & 0xffffu), s_big[g] >> 16, lane);
                 }
                 if (tid == 0) s_bigs = 0;  // for the next array (read above, before a barrier)
                 __syncthreads();
@@ -478,16 +532,39 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
             if (PAIRS) cp_async_wait_all();
             __syncthreads();
             // ---- 4. stored in order -----------------------------------------
-            const K high = PAIRS && sizeof(W) == sizeof(K) ? first & ~(~K(0) >> ib) : K(0);
+            const uint32_t imask = (1u << bits) - 1;
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) {
-                const uint32_t i = tid + j * THREADS;
-                if (i < m) {
-                    const W w = s_w[i];
-                    K key = (K)(w >> ib) | high;
+                uint32_t at_ = tid + j * THREADS;
+                if (at_ < m) {
+                    const K w = s_w[at_];
+                    const uint32_t i = (uint32_t)w & imask;
+                    K key;
+                    if constexpr (WHOLE) {
+                        key = PAIRS ? (K)(w >> top) | least : w;
+                    } else {
+                        // Words next to each other may differ in their index only
+                        // because the key's last bits did not fit: those few
+                        // items find their places among each other by the keys.
+                        key = s_k[i];
+                        const K t = w >> ib;
+                        const bool below = at_ > 0 && s_w[at_ - 1] >> ib == t;
+                        const bool above = at_ + 1 < m && s_w[at_ + 1] >> ib == t;
+                        if (below || above) {
+                            uint32_t lo_ = at_, hi_ = at_ + 1;
+                            while (lo_ > 0 && s_w[lo_ - 1] >> ib == t) --lo_;
+                            while (hi_ < m && s_w[hi_] >> ib == t) ++hi_;
+                            at_ = lo_;
+                            for (uint32_t q = lo_; q < hi_; ++q) {
+                                const uint32_t o = (uint32_t)s_w[q] & imask;
+                                const K ok = s_k[o];
+                                at_ += ok < key || (ok == key && o < i) ? 1u : 0u;
+                            }
+                        }
+                    }
                     if (typed) key = key_from_ordered(key, key_type);
-                    keys[lo + i] = key;
-                    if (PAIRS) vals[lo + i] = s_v[(uint32_t)w & ((1u << bits) - 1)];
+                    keys[lo + at_] = key;
+                    if (PAIRS) vals[lo + at_] = s_v[i];
                 }
             }
         } else {
@@ -502,7 +579,6 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
             const uint32_t mine = left < ipt ? left : ipt;
             const uint32_t lt = lanemask_lt();
             uint32_t* const row = s_bin + warp * RADIX;
-            K* const s_k = reinterpret_cast<K*>(s_w);
             V v[PAIRS ? ITEMS : 1];
             if (PAIRS) cp_async_wait_all();
             __syncthreads();
@@ -515,7 +591,7 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 }
             }
             for (uint32_t p = 0; p < sizeof(K); ++p) {
-                if (((varying >> (8 * p)) & (RADIX - 1)) == 0) continue;
+                if (least >> (8 * p) == most >> (8 * p)) break;  // the rest is the same in all
                 for (uint32_t b = lane; b < RADIX; b += 32) row[b] = 0;
                 __syncwarp();
 #pragma unroll
@@ -536,14 +612,17 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 // every warp's first position of the digit.
                 constexpr uint32_t PER = RADIX > THREADS ? RADIX / THREADS : 1;
                 uint32_t c[PER], sum = 0;
+                bool trivial = false;
 #pragma unroll
                 for (uint32_t q = 0; q < PER; ++q) {
                     c[q] = 0;
                     const uint32_t d = tid * PER + q;
                     if (d < RADIX)
                         for (uint32_t w = 0; w < WARPS; ++w) c[q] += s_bin[w * RADIX + d];
+                    trivial |= c[q] == m;
                     sum += c[q];
                 }
+                if (__syncthreads_or(trivial)) continue;  // one digit only: the identity
                 uint32_t x = sum;
 #pragma unroll
                 for (uint32_t o = 1; o < 32; o <<= 1) {
@@ -572,7 +651,7 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 for (int j = 0; j < ITEMS; ++j) {
                     if (j < mine) {
                         at[j] += row[(uint32_t)(k[j] >> (8 * p)) & (RADIX - 1)];
-                        s_k[at[j]] = k[j];
+                        s_w[at[j]] = k[j];
                         if (PAIRS) s_v[at[j]] = v[j];
                     }
                 }
@@ -580,7 +659,7 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
 #pragma unroll
                 for (int j = 0; j < ITEMS; ++j) {
                     if (j < mine) {
-                        k[j] = s_k[me + j * 32];
+                        k[j] = s_w[me + j * 32];
                         if (PAIRS) v[j] = s_v[me + j * 32];
                     }
                 }

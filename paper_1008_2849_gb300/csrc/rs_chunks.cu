@@ -12,10 +12,10 @@ template <typename K, typename V, bool PAIRS, int THREADS, int MIN_BLOCKS>
 rs_status launch_chunks(K* keys, V* vals, K* spare_keys, V* spare_vals, const uint32_t* off,
                         const Ctrl* ctrl, uint32_t top_bits, uint32_t key_type, int sm_count,
                         cudaStream_t stream) {
-    // A word as wide as the key: the index takes the place of the bits that the
-    // chunk's keys have in common (TopOrder).
-    using L = BinSortSmem<K, V, K, PAIRS, THREADS, true>;
-    auto kern = k_bin_sort<K, V, K, PAIRS, THREADS, MIN_BLOCKS, true>;
+    // (The index of an item takes the place of the bits that its chunk's keys have in
+    // common, see TopOrder.)
+    using L = BinSortSmem<K, V, PAIRS, THREADS, true>;
+    auto kern = k_bin_sort<K, V, PAIRS, THREADS, MIN_BLOCKS, true>;
     static DeviceOnce smem_set;
     const rs_status st = allow_smem_once(kern, L::BYTES, smem_set);
     if (st != RS_OK) return st;

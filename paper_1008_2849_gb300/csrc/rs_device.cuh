@@ -54,7 +54,11 @@ struct Ctrl {
     uint32_t large_count;
     uint32_t tiny_count;
     uint32_t chunk_count;          // top-digits order: chunks sorted on chip (0: another order)
-    uint32_t pad[6];               // keep hist 64-byte aligned
+    // Segmented sorts: tiles of the large segments that take the MSD-first order
+    // (chunk_count counts their runs) and of those that take all passes.
+    uint32_t msd_tiles;
+    uint32_t lsd_tiles;
+    uint32_t pad[4];               // keep hist 64-byte aligned
     uint32_t hist[PASSES64][RADIX];  // digit histograms (H); 0..3 for 32-bit keys
     uint32_t gofs[PASSES64][RADIX];  // first output slot of every bucket (G)
 };
@@ -87,6 +91,9 @@ constexpr uint32_t ROLE_MAP_PASSES = 1u << 9;
 constexpr uint32_t KEY_TYPE_MASK = 0xffu;
 // A launch of pass 3 that is the MSD-first order's pass when the plan chose it.
 constexpr uint32_t ROLE_MSD_TOO = 1u << 10;
+// Segmented sorts whose tiles k_seg_scan has placed: the MSD pass takes the first
+// msd_tiles tiles, the others the lsd_tiles last ones.
+constexpr uint32_t ROLE_ROUTED = 1u << 11;
 
 __device__ __forceinline__ uint32_t key_to_ordered(uint32_t k, uint32_t type) {
     const uint32_t neg = type == KEY_F32 ? (uint32_t)((int32_t)k >> 31) : 0u;

@@ -209,6 +209,7 @@ struct SegView {
     const uint4* tile_geo = nullptr;
     const uint32_t* gofs = nullptr;
     uint32_t max_tiles = 0;
+    bool routed = false;  // tiles placed by each segment's order (k_seg_scan)
 };
 
 // Scatter-pass launchers, one per value flavour (separate translation units);
@@ -232,6 +233,11 @@ rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* sr
                               const uint32_t* src_vals, const uint32_t* off,
                               const uint32_t* count, const Ctrl* ctrl, bool long_buckets,
                               int bits, uint32_t key_type, cudaStream_t stream);
+// One-CTA sorts on chip of *count ranges (first item, items) at `runs`, of at most 4096
+// items each.
+rs_status launch_run_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
+                           const uint32_t* src_vals, const uint32_t* runs, const uint32_t* count,
+                           const Ctrl* ctrl, int bits, uint32_t key_type, cudaStream_t stream);
 // The segments listed by size (rs_bin_sort.cuh list_small) in tiny_list and
 // small_list of `entries` entries each, in place: one launch per size up to
 // max_items.
@@ -257,6 +263,9 @@ uint32_t warp_sort_capacity();
 struct SegLayout {
     size_t ctrl, status0, status1, alt_keys, alt_vals, tile_geo, tiny_list, small_list, large_first,
         gofs, total;
+    // The 32-bit sorts' parts for segments that take the MSD-first order; a
+    // workspace of `total` bytes, without them, has all take the LSD passes.
+    size_t route_geo, runs, routed_total;
     uint32_t max_tiles, max_large;
 };
 SegLayout seg_layout_for(size_t n, bool pairs, uint32_t num_segments);

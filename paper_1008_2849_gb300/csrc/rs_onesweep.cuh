@@ -121,7 +121,8 @@ struct OnesweepSmem {
 // (first item, item count, first tile of its segment, segment) for every tile
 // of the large segments; seg_gofs[s][pass][b] (pass < 4, or < 8 for 64-bit
 // keys) is the absolute first output
-// slot of bucket b of segment s; the number of tiles is ctrl->seg_tiles.
+// slot of bucket b of segment s; the number of tiles is ctrl->seg_tiles, or with
+// ROLE_ROUTED those of the segments that take this launch's order.
 template <int THREADS, int ITEMS, int MIN_BLOCKS, bool PAIRS, typename S, int WINDOW, bool SEG,
           bool TYPED, typename K = uint32_t, typename V = uint32_t>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
@@ -192,6 +193,20 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
         if (ctrl->dir[MSD_SLOT] != DIR_SKIP) slot = MSD_SLOT;
         key_type &= ~ROLE_MSD_TOO;
     }
+    uint32_t tile0 = 0;  // the first tile of this launch
+    if (SEG) {
+        if (ld_relaxed(&ctrl->err) != 0) return;  // malformed segment table: no work
+        if (key_type & ROLE_ROUTED) {
+            if (slot == MSD_SLOT) num_tiles = ctrl->msd_tiles;
+            else tile0 = num_tiles - ctrl->lsd_tiles;  // of max_tiles
+            key_type &= ~ROLE_ROUTED;
+        } else {
+            num_tiles = ctrl->seg_tiles;
+        }
+        if (tile0 >= num_tiles) return;
+    }
+    // The MSD-first order's only pass is the first and the last.
+    const bool only_pass = slot == MSD_SLOT;
     if (key_type & (ROLE_PLAIN_PASSES | ROLE_MAP_PASSES)) {
         // One of the two instances of a typed sort's pass: keep the pass if
         // it is this instance's (an executed first or last pass needs the
@@ -202,13 +217,9 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
             if (q < pass) first = false;
             if (q > pass) last = false;
         }
-        const bool maps = ctrl->dir[slot] != DIR_SKIP && (first || last);
+        const bool maps = ctrl->dir[slot] != DIR_SKIP && (first || last || only_pass);
         if (maps != ((key_type & ROLE_MAP_PASSES) != 0)) return;
         key_type &= KEY_TYPE_MASK;
-    }
-    if (SEG) {
-        if (ld_relaxed(&ctrl->err) != 0) return;  // malformed segment table: no work
-        num_tiles = ctrl->seg_tiles;
     }
     const uint32_t dir = ctrl->dir[slot];
     if (dir == DIR_SKIP) {
@@ -231,8 +242,8 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
             if (q < pass) first = false;
             if (q > pass) last = false;
         }
-        map_in = first ? key_type : KEY_U32;
-        map_out = last ? key_type : KEY_U32;
+        map_in = first || only_pass ? key_type : KEY_U32;
+        map_out = last || only_pass ? key_type : KEY_U32;
     }
     auto read_key = [map_in](K k) -> K {
         if constexpr (TYPED) return key_to_ordered(k, map_in);
@@ -256,7 +267,7 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
     if (tid == 0) {
         for (int b = 0; b < 3; ++b) mbar_init(&s_bar[b], 1);
         fence_mbar_init();
-        s_ids[0] = atomicAdd(&ctrl->tile_ctr[slot], 1u);
+        s_ids[0] = tile0 + atomicAdd(&ctrl->tile_ctr[slot], 1u);
         s_geo[0] = load_geo(s_ids[0]);
         s_flag = 0;
         s_err_seen = 0;
@@ -380,7 +391,7 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
             c += v;
         }
         s_cnt[tid] = c;
-        const bool withhold = (debug & DBG_WITHHOLD_FIRST_TILE) && t == 0;
+        const bool withhold = (debug & DBG_WITHHOLD_FIRST_TILE) && t == tile0;
         if (!withhold)
             st_relaxed(status + (size_t)t * RADIX + tid, (t == first ? SW::INC : SW::AGG) | (S)c);
         uint32_t x = c;
@@ -415,7 +426,7 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
     __syncthreads();
     if (tid < RADIX) prep_tile(s_ids[0], s_geo[0].z);
     if (tid == 0) {
-        s_ids[1] = atomicAdd(&ctrl->tile_ctr[slot], 1u);
+        s_ids[1] = tile0 + atomicAdd(&ctrl->tile_ctr[slot], 1u);
         s_geo[1] = load_geo(s_ids[1]);
     }
     __syncthreads();
@@ -589,7 +600,7 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
                 // This CTA waits on no other CTA from here until the counts of
                 // the tile taken now are published: taking it cannot stall
                 // anyone.
-                next_id = atomicAdd(&ctrl->tile_ctr[slot], 1u);
+                next_id = tile0 + atomicAdd(&ctrl->tile_ctr[slot], 1u);
                 next_geo = load_geo(next_id);
                 // 32-bit pairs copy a tile in only once the tile before it is
                 // ranked: start pulling it into L2 an iteration earlier.

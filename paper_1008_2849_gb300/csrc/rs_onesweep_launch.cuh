@@ -52,7 +52,8 @@ static rs_status launch_onesweep_shape(K* ka, V* va, K* kb, V* vb,
     const cudaError_t e = launch_after_previous(
         kern, dim3(grid), dim3(THREADS), L::BYTES, stream, ka, va, kb, vb, n, pass, slot, tiles,
         ctrl, sticky, static_cast<S*>(status), static_cast<S*>(status_clear), tiles * RADIX,
-        knobs().spin_limit, knobs().debug, seg.tile_geo, seg.gofs, key_type);
+        knobs().spin_limit, knobs().debug, seg.tile_geo, seg.gofs,
+        key_type | (SEG && seg.routed ? ROLE_ROUTED : 0u));
     note_launch_end(SEG ? KK_SEG_ONESWEEP : KK_ONESWEEP, stream);
     return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }

@@ -40,6 +40,11 @@ SegLayout seg_layout_for(size_t n, bool pairs, uint32_t num_segments) {
     L.gofs = off;
     off = align_up(off + large * PASSES * RADIX * 4, 256);
     L.total = off;
+    L.route_geo = off;
+    off = align_up(off + (size_t)L.max_tiles * 16, 256);
+    L.runs = off;  // a run per 512 items, and up to two more per segment
+    off = align_up(off + (n / 512 + 2 * large + 2) * 8, 256);
+    L.routed_total = off;
     return L;
 }
 
@@ -80,8 +85,9 @@ rs_status enqueue_sort_segmented(uint32_t* keys, uint32_t* vals, uint32_t n,
         cudaMemsetAsync(gofs, 0, (size_t)L.max_large * PASSES * RADIX * 4, stream) != cudaSuccess)
         return RS_ERR_CUDA;
     note_launch_begin(KK_SEG_PLAN, stream);
-    k_seg_plan<<<1, 1024, 0, stream>>>(offsets, num_segments, n, tile, warp_max, small_max, ctrl,
-                                       di.sticky, tile_geo, tiny_list, small_list, large_first);
+    k_seg_plan<<<(num_segments + 1023) / 1024, 1024, 0, stream>>>(
+        offsets, num_segments, n, tile, warp_max, small_max, ctrl, di.sticky, tile_geo,
+        L.max_tiles, tiny_list, small_list, large_first, L.max_large);
     note_launch_end(KK_SEG_PLAN, stream);
     if (cudaPeekAtLastError() != cudaSuccess) return RS_ERR_CUDA;
 
@@ -112,25 +118,38 @@ rs_status enqueue_sort_segmented(uint32_t* keys, uint32_t* vals, uint32_t n,
     }
     note_launch_end(KK_SEG_HIST, stream);
     note_launch_begin(KK_SEG_SCAN, stream);
+    // Each large segment takes the MSD-first order or the four passes.
+    const bool routed = ck.msd != 0 && workspace_bytes >= L.routed_total;
+    const SegRoute route{routed ? reinterpret_cast<uint4*>(ws + L.route_geo) : nullptr,
+                         reinterpret_cast<uint2*>(ws + L.runs), L.max_tiles, tile};
     const cudaError_t se = launch_after_previous(k_seg_scan<PASSES>, dim3(di.sm_count * 2),
-                                                 dim3(1024), 0, stream, (const Ctrl*)ctrl, gofs,
-                                                 (const uint32_t*)large_first);
+                                                 dim3(1024), 0, stream, ctrl, gofs,
+                                                 (const uint32_t*)large_first, route);
     note_launch_end(KK_SEG_SCAN, stream);
     if (se != cudaSuccess) return RS_ERR_CUDA;
 
     SegView view;
-    view.tile_geo = tile_geo;
+    view.tile_geo = routed ? route.geo : tile_geo;
     view.max_tiles = L.max_tiles;
-    for (uint32_t p = 0; p < PASSES; ++p) {
-        view.gofs = gofs;
-        void* cur = status[p & 1];
-        void* next = p + 1 < PASSES ? status[(p + 1) & 1] : nullptr;
-        st = pairs ? launch_onesweep_pairs(cfg, false, keys, vals, alt_k, alt_v, n, p, p, ctrl,
-                                           di.sticky, cur, next, &view, key_type, stream)
-                   : launch_onesweep_keys(cfg, false, keys, alt_k, n, p, p, ctrl, di.sticky, cur,
-                                          next, &view, key_type, stream);
+    view.gofs = gofs;
+    view.routed = routed;
+    auto pass = [&](uint32_t p, uint32_t slot, void* cur, void* next) {
+        return pairs ? launch_onesweep_pairs(cfg, false, keys, vals, alt_k, alt_v, n, p, slot, ctrl,
+                                             di.sticky, cur, next, &view, key_type, stream)
+                     : launch_onesweep_keys(cfg, false, keys, alt_k, n, p, slot, ctrl, di.sticky,
+                                            cur, next, &view, key_type, stream);
+    };
+    if (routed) {
+        st = pass(PASSES - 1, MSD_SLOT, status[0], nullptr);
         if (st != RS_OK) return st;
     }
+    for (uint32_t p = 0; p < PASSES; ++p) {
+        st = pass(p, p, status[p & 1], p + 1 < PASSES ? status[(p + 1) & 1] : nullptr);
+        if (st != RS_OK) return st;
+    }
+    if (routed)
+        return launch_run_sorts(keys, vals, alt_k, alt_v, reinterpret_cast<uint32_t*>(ws + L.runs),
+                                &ctrl->chunk_count, ctrl, ck.small_bits, key_type, stream);
     return RS_OK;
 }
 

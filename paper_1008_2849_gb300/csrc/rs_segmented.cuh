@@ -8,10 +8,11 @@
 //   small (warp_max < size <= small_max): k_bin_sort (rs_bin_sort.cuh), one CTA
 //       per segment, the whole segment on chip -- one read and one write of
 //       every item either way;
-//   large (size > small_max): the scatter passes of the unsegmented sort
+//   large (size > small_max): scatter passes as of the unsegmented sort
 //       (k_onesweep<..., SEG>) over tiles that never straddle a segment, after
 //       k_seg_hist (per-segment digit histograms) and k_seg_scan (per-segment
-//       bucket bases).
+//       bucket bases, and each segment's order: one pass by digit 3 and its
+//       buckets sorted on chip, or all passes).
 // k_seg_plan validates the table and lays the work out.
 #pragma once
 
@@ -20,91 +21,99 @@
 
 namespace rs {
 
+// `count` threads write the tile geometries of one segment of `size` items from
+// item `lo` on, tiles t0, t0 + 1, ...
+__device__ __forceinline__ void write_tiles(uint4* tile_geo, uint32_t lo, uint32_t size,
+                                            uint32_t t0, uint32_t ordinal, uint32_t tile,
+                                            uint32_t thread, uint32_t count) {
+    for (uint32_t k = thread; (unsigned long long)k * tile < size; k += count) {
+        const uint32_t left = size - k * tile;
+        tile_geo[t0 + k] = make_uint4(lo + k * tile, left < tile ? left : tile, t0, ordinal);
+    }
+}
+
 // ---------------------------------------------------------------------------
-// k_seg_plan: one CTA of 1024 threads.
+// k_seg_plan: CTAs of 1024 threads, a segment per thread.
 //  - Validates the table: nondecreasing, off[S] <= n, every segment < 2^30
 //    items.  A bad table sets ERR_SEGMENTS; every later kernel then exits
 //    without writing anything.
-//  - Large segments get consecutive tile ids (in segment order) and a dense
-//    ordinal; tile_geo[t] = (first item, item count, first tile of its
-//    segment, ordinal of its segment).
+//  - Large segments get consecutive tile ids and a dense ordinal, in any order;
+//    tile_geo[t] = (first item, item count, first tile of its segment, ordinal
+//    of its segment).  Nothing is written past max_tiles or max_large, which a
+//    bad table could ask for.
 //  - Tiny and small segments are listed by size (list_small; order irrelevant).
 //  - The pass plan runs all npass passes (four, or eight for 64-bit keys;
-//    caller -> alternate -> ... -> caller).
+//    caller -> alternate -> ... -> caller), and the MSD-first pass of the segments
+//    that take it.
+// The order of segments does not matter to any later kernel, so CTAs take their
+// places with one atomic each: 2^15 segments in 4 us, where one CTA that scanned
+// over them in turn took 53.
 // ---------------------------------------------------------------------------
 static __global__ void __launch_bounds__(1024)
 k_seg_plan(const uint32_t* __restrict__ off, uint32_t num_segments, uint32_t n, uint32_t tile,
            uint32_t warp_max, uint32_t small_max, Ctrl* __restrict__ ctrl,
-           uint32_t* __restrict__ sticky, uint4* __restrict__ tile_geo,
+           uint32_t* __restrict__ sticky, uint4* __restrict__ tile_geo, uint32_t max_tiles,
            uint32_t* __restrict__ tiny_list, uint32_t* __restrict__ small_list,
            uint32_t* __restrict__ large_first /* [S] first item of large ordinal */,
-           uint32_t npass = PASSES) {
-    __shared__ uint32_t s_carry[2];  // tiles and large segments before this chunk
+           uint32_t max_large, uint32_t npass = PASSES) {
+    __shared__ unsigned long long s_w64[32];
+    __shared__ uint32_t s_base[2];  // this CTA's first tile and first ordinal
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_launch_next();
     pdl_wait();
 
+    const uint32_t s = blockIdx.x * 1024 + tid;
+    uint32_t size = 0, lo = 0;
     bool bad = false;
-    for (uint32_t s = tid; s < num_segments; s += 1024) {
-        const uint32_t a = off[s], b = off[s + 1];
-        if (b < a || b - a >= (1u << 30)) bad = true;
+    if (s < num_segments) {
+        lo = off[s];
+        const uint32_t hi = off[s + 1];
+        bad = hi < lo || hi > n || hi - lo >= (1u << 30);
+        size = bad ? 0u : hi - lo;
     }
-    if (tid == 0 && off[num_segments] > n) bad = true;
-    if (__syncthreads_or(bad)) {
-        if (tid == 0) record_error(ctrl, sticky, ERR_SEGMENTS);
-        return;
+    const bool large = size > small_max;
+    const uint32_t ntiles = large ? (size + tile - 1) / tile : 0u;
+    list_small(ctrl, s, large ? 0u : size, warp_max, num_segments - 1, tiny_list, small_list);
+    // CTA-wide exclusive scan of (tiles, large flag), two 32-bit halves.
+    const unsigned long long v = ((unsigned long long)ntiles << 32) | (large ? 1u : 0u);
+    unsigned long long x = v;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w64[warp] = x;
+    __syncthreads();
+    unsigned long long before = 0, all = 0;
+    for (uint32_t w = 0; w < 32; ++w) {
+        if (w < warp) before += s_w64[w];
+        all += s_w64[w];
     }
     if (tid == 0) {
-        s_carry[0] = 0;
-        s_carry[1] = 0;
-        for (uint32_t p = 0; p < npass; ++p) ctrl->dir[p] = (p & 1) ? DIR_B_TO_A : DIR_A_TO_B;
+        s_base[0] = atomicAdd(&ctrl->seg_tiles, (uint32_t)(all >> 32));
+        s_base[1] = atomicAdd(&ctrl->large_count, (uint32_t)all);
+        if (blockIdx.x == 0) {
+            for (uint32_t p = 0; p < npass; ++p) ctrl->dir[p] = (p & 1) ? DIR_B_TO_A : DIR_A_TO_B;
+            ctrl->dir[MSD_SLOT] = DIR_A_TO_B;
+        }
     }
     __syncthreads();
-    for (uint32_t c = 0; c < num_segments; c += 1024) {
-        const uint32_t s = c + tid;
-        uint32_t size = 0, lo = 0;
-        if (s < num_segments) {
-            lo = off[s];
-            size = off[s + 1] - lo;
-        }
-        const bool large = size > small_max;
-        const uint32_t ntiles = large ? (size + tile - 1) / tile : 0u;
-        if (s < num_segments && !large && size >= 2)
-            list_small(ctrl, s, size, warp_max, num_segments - 1, tiny_list, small_list);
-        // Block-wide exclusive scans of (tiles, large flag), packed as two
-        // 32-bit halves of one 64-bit sum.
-        unsigned long long v = ((unsigned long long)ntiles << 32) | (large ? 1u : 0u);
-        unsigned long long x = v;
-#pragma unroll
-        for (uint32_t o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        __shared__ unsigned long long s_w64[32];
-        if (lane == 31) s_w64[warp] = x;
-        __syncthreads();
-        unsigned long long off64 = 0;
-        for (uint32_t w = 0; w < warp; ++w) off64 += s_w64[w];
-        const unsigned long long excl = off64 + x - v;
-        const uint32_t t0 = s_carry[0] + (uint32_t)(excl >> 32);
-        const uint32_t ordinal = s_carry[1] + (uint32_t)(excl & 0xffffffffu);
-        if (large) {
-            large_first[ordinal] = lo;
-            for (uint32_t k = 0; k < ntiles; ++k) {
-                const uint32_t left = size - k * tile;
-                tile_geo[t0 + k] = make_uint4(lo + k * tile, left < tile ? left : tile, t0, ordinal);
-            }
-        }
-        __syncthreads();
-        if (tid == 1023) {
-            s_carry[0] = t0 + ntiles;
-            s_carry[1] = ordinal + (large ? 1u : 0u);
-        }
-        __syncthreads();
-    }
-    if (tid == 0) {
-        ctrl->seg_tiles = s_carry[0];
-        ctrl->large_count = s_carry[1];
+    const unsigned long long excl = before + x - v;
+    const uint32_t t0 = s_base[0] + (uint32_t)(excl >> 32);
+    const uint32_t ordinal = s_base[1] + (uint32_t)excl;
+    const bool fits = !large || (t0 + ntiles <= max_tiles && t0 + ntiles >= t0 &&
+                                 ordinal < max_large);
+    if (__any_sync(0xffffffffu, bad || !fits) && lane == 0)
+        record_error(ctrl, sticky, ERR_SEGMENTS);
+    if (large && fits) large_first[ordinal] = lo;
+    // The warp writes the tiles of its large segments together.
+    for (uint32_t todo = __ballot_sync(0xffffffffu, large && fits); todo != 0; todo &= todo - 1) {
+        const uint32_t l = __ffs(todo) - 1;
+        const uint32_t l_lo = __shfl_sync(0xffffffffu, lo, l);
+        const uint32_t l_size = __shfl_sync(0xffffffffu, size, l);
+        const uint32_t l_t0 = __shfl_sync(0xffffffffu, t0, l);
+        const uint32_t l_ord = __shfl_sync(0xffffffffu, ordinal, l);
+        write_tiles(tile_geo, l_lo, l_size, l_t0, l_ord, tile, lane, 32);
     }
 }
 
@@ -220,13 +229,35 @@ k_seg_hist(const uint32_t* __restrict__ keys, const Ctrl* __restrict__ ctrl,
 // buckets, twice for the eight digits of 64-bit keys), the exclusive prefix
 // over buckets plus the segment's first item: the absolute first output slot
 // of every bucket, written over the histogram hist[segment][NP][256].
+//
+// With route.geo set (32-bit keys), it also decides each segment's order: where
+// digit 3 takes more than one value and no bucket of it holds more than
+// MSD_SEG_BUCKET items, one pass by digit 3 into the alternate buffers, then runs
+// of its buckets sorted on chip back into the caller's arrays; else the four
+// passes.  Segments of the first kind get tiles 0 .. msd_tiles - 1 of route.geo,
+// the others the lsd_tiles last ones; route.chunks lists (first item, items) of
+// the runs: the buckets that start in the same stretch of CAPACITY - (largest
+// bucket) items, CAPACITY in all at most.
 // ---------------------------------------------------------------------------
+constexpr uint32_t MSD_SEG_CAPACITY = SMALL_MID_MAX;  // of the on-chip sort
+constexpr uint32_t MSD_SEG_BUCKET = MSD_SEG_CAPACITY - 512;  // so a stretch is 512 items or more
+
+struct SegRoute {
+    uint4* geo;
+    uint2* chunks;
+    uint32_t max_tiles, tile;
+};
+
 template <int NP = PASSES>
 __global__ void __launch_bounds__(1024)
-k_seg_scan(const Ctrl* __restrict__ ctrl, uint32_t* __restrict__ hist,
-           const uint32_t* __restrict__ large_first) {
+k_seg_scan(Ctrl* __restrict__ ctrl, uint32_t* __restrict__ hist,
+           const uint32_t* __restrict__ large_first, const SegRoute route) {
     static_assert(NP == 4 || NP == 8, "32-bit or 64-bit keys");
     __shared__ uint32_t s_warp[32];
+    __shared__ uint32_t s_max[RADIX / 32], s_runs[RADIX / 32];
+    __shared__ uint32_t s_start[RADIX];      // first items of digit 3's buckets
+    __shared__ uint32_t s_first[RADIX + 1];  // first items of the runs, and the segment's end
+    __shared__ uint32_t s_base[2];           // first tile, first run
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t p = tid >> 8;
     pdl_launch_next();
@@ -244,10 +275,51 @@ k_seg_scan(const Ctrl* __restrict__ ctrl, uint32_t* __restrict__ hist,
             if (lane >= o) x += y;
         }
         if (lane == 31) s_warp[warp] = x;
+        const uint32_t most = __reduce_max_sync(0xffffffffu, v);
+        if (p == PASSES - 1 && lane == 0) s_max[warp & 7] = most;
         __syncthreads();
         uint32_t offv = 0;
         for (uint32_t w = p * (RADIX / 32); w < warp; ++w) offv += s_warp[w];
-        h[tid] = large_first[g] + offv + x - v;
+        const uint32_t lo = large_first[g];
+        const uint32_t start = offv + x - v;
+        h[tid] = lo + start;
+        if (NP == 4 && route.geo != nullptr) {
+            uint32_t size = 0, biggest = 0;
+            for (uint32_t w = 0; w < RADIX / 32; ++w) {
+                size += s_warp[w];  // digit 0 counts every item
+                biggest = max(biggest, s_max[w]);
+            }
+            const bool msd = biggest <= MSD_SEG_BUCKET && biggest < size;
+            const uint32_t b = tid & (RADIX - 1);
+            if (p == PASSES - 1) s_start[b] = start;
+            __syncthreads();
+            // Bucket b starts a run where its stretch is not that of the bucket
+            // before (empty buckets start where the next one does).
+            const uint32_t stretch = MSD_SEG_CAPACITY - (msd ? biggest : 0u);
+            const bool starts = p == PASSES - 1 && msd &&
+                                (b == 0 || start / stretch != s_start[b - 1] / stretch);
+            const uint32_t vote = __ballot_sync(0xffffffffu, starts);
+            if (p == PASSES - 1 && lane == 0) s_runs[warp & 7] = __popc(vote);
+            __syncthreads();
+            uint32_t at = __popc(vote & lanemask_lt()), runs = 0;
+            for (uint32_t w = 0; w < RADIX / 32; ++w) {
+                if (w < (warp & 7)) at += s_runs[w];
+                runs += s_runs[w];
+            }
+            if (starts) s_first[at] = start;
+            if (tid == 0) {
+                s_first[runs] = size;
+                const uint32_t tiles = (size + route.tile - 1) / route.tile;
+                s_base[0] = msd ? atomicAdd(&ctrl->msd_tiles, tiles)
+                                : route.max_tiles - tiles - atomicAdd(&ctrl->lsd_tiles, tiles);
+                if (msd) s_base[1] = atomicAdd(&ctrl->chunk_count, runs);
+            }
+            __syncthreads();
+            write_tiles(route.geo, lo, size, s_base[0], g, route.tile, tid, 1024);
+            if (tid < runs)
+                route.chunks[s_base[1] + tid] =
+                    make_uint2(lo + s_first[tid], s_first[tid + 1] - s_first[tid]);
+        }
         __syncthreads();
     }
 }

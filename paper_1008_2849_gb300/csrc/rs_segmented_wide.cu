@@ -90,9 +90,9 @@ rs_status run(K* keys, V* vals, uint32_t n, const uint32_t* offsets, uint32_t nu
     // Segments of up to kWideWarpMax items: one warp each; every longer one
     // is large (no one-CTA class for wide items).
     note_launch_begin(KK_SEG_PLAN, stream);
-    k_seg_plan<<<1, 1024, 0, stream>>>(offsets, num_segments, n, tile, kWideWarpMax, kWideWarpMax,
-                                       ctrl, di.sticky, tile_geo, tiny_list, small_list,
-                                       large_first, NP);
+    k_seg_plan<<<(num_segments + 1023) / 1024, 1024, 0, stream>>>(
+        offsets, num_segments, n, tile, kWideWarpMax, kWideWarpMax, ctrl, di.sticky, tile_geo,
+        L.max_tiles, tiny_list, small_list, large_first, L.max_large, NP);
     note_launch_end(KK_SEG_PLAN, stream);
     if (cudaPeekAtLastError() != cudaSuccess) return RS_ERR_CUDA;
     st = warp_sort<K, V, PAIRS>(keys, vals, offsets, tiny_list, ctrl, key_type, di.sm_count, stream);
@@ -116,7 +116,7 @@ rs_status run(K* keys, V* vals, uint32_t n, const uint32_t* offsets, uint32_t nu
     }
     note_launch_end(KK_SEG_HIST, stream);
     note_launch_begin(KK_SEG_SCAN, stream);
-    k_seg_scan<NP><<<di.sm_count * 2, 1024, 0, stream>>>(ctrl, gofs, large_first);
+    k_seg_scan<NP><<<di.sm_count * 2, 1024, 0, stream>>>(ctrl, gofs, large_first, SegRoute{});
     note_launch_end(KK_SEG_SCAN, stream);
     if (cudaPeekAtLastError() != cudaSuccess) return RS_ERR_CUDA;
 

@@ -17,7 +17,7 @@ struct SmallWork {
     int32_t step;
     const uint32_t* list_count;
     const Ctrl* ctrl;
-    uint32_t single_n;  // off == nullptr: the array's items; list == nullptr: see k_bin_sort
+    uint32_t single_n;  // off == nullptr: the array's items
     uint32_t key_type;
 };
 
@@ -29,12 +29,10 @@ rs_status grid_of(const SmallWork& w, uint32_t per_sm, uint32_t* grid) {
     return st;
 }
 
-// The word of the bin sort: the key alone; for pairs 64 bits.
 template <bool PAIRS, int THREADS, int MIN_BLOCKS>
 rs_status launch_bin_shape(const SmallWork& w, cudaStream_t stream) {
-    using W = std::conditional_t<PAIRS, unsigned long long, uint32_t>;
-    using L = BinSortSmem<uint32_t, uint32_t, W, PAIRS, THREADS, false>;
-    auto kern = k_bin_sort<uint32_t, uint32_t, W, PAIRS, THREADS, MIN_BLOCKS, false>;
+    using L = BinSortSmem<uint32_t, uint32_t, PAIRS, THREADS, false>;
+    auto kern = k_bin_sort<uint32_t, uint32_t, PAIRS, THREADS, MIN_BLOCKS>;
     static DeviceOnce smem_set;
     rs_status st = allow_smem_once(kern, L::BYTES, smem_set);
     if (st != RS_OK) return st;
@@ -124,6 +122,13 @@ rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* sr
     if (long_buckets || bits == 4) return launch_small_any(small_sort_capacity(), bits, w, stream);
     return vals != nullptr ? launch_bin_shape<true, 640, 2>(w, stream)
                            : launch_bin_shape<false, 640, 2>(w, stream);
+}
+
+rs_status launch_run_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
+                           const uint32_t* src_vals, const uint32_t* runs, const uint32_t* count,
+                           const Ctrl* ctrl, int bits, uint32_t key_type, cudaStream_t stream) {
+    const SmallWork w{keys, vals, src_keys, src_vals, runs, runs, 0, count, ctrl, 0, key_type};
+    return launch_small_any(SMALL_MID_MAX, bits, w, stream);
 }
 
 rs_status launch_small_lists(uint32_t* keys, uint32_t* vals, const uint32_t* off,

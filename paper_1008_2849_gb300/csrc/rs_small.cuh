@@ -159,8 +159,8 @@ k_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uint
 // k_small_sort: one CTA sorts a whole array of at most CAP = THREADS * ITEMS
 // items in shared memory: 32 / BITS stable counting-sort passes between two
 // shared buffers.  Arrays are the segments listed from `list` on (every
-// `step`-th entry; count in *list_count), with list == nullptr those of
-// the segments 0, 1, ... that hold more than single_n items and at most CAP, or with off == nullptr the single
+// `step`-th entry; count in *list_count), with list == nullptr the
+// segments 0, 1, ..., with step == 0 the ranges (first item, items) in `list`, or with off == nullptr the single
 // array [0, single_n).  The 4-bit form only; 8-bit digits take k_bin_sort.
 // Per pass: per-warp digit counts, their prefix over (digit, warp), then every
 // warp ranks its items slot by slot (peers from one ballot per digit bit,
@@ -201,10 +201,15 @@ k_small_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uin
     for (uint32_t idx = blockIdx.x; idx < count; idx += gridDim.x) {
         uint32_t lo = 0, m = single_n;
         if (off != nullptr) {
-            const uint32_t s = list != nullptr ? list[(ptrdiff_t)idx * step] : idx;
-            lo = off[s];
-            m = off[s + 1] - lo;
-            if (list == nullptr && (m <= single_n || m > CAP)) continue;
+            if (step == 0) {
+                lo = list[2 * idx];
+                m = list[2 * idx + 1];
+            } else {
+                const uint32_t s = list != nullptr ? list[(ptrdiff_t)idx * step] : idx;
+                lo = off[s];
+                m = off[s + 1] - lo;
+            }
+            if (m == 0 || m > CAP) continue;
         }
         for (uint32_t i = tid; i < m; i += THREADS) {
             s_k[i] = key_to_ordered(src_keys[lo + i], key_type);
