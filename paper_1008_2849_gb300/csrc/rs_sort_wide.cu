@@ -12,7 +12,6 @@ namespace rs {
 
 namespace {
 
-constexpr int HIST8_THREADS = 512;
 constexpr int B_WIDE = 2, W_WIDE = 8;
 
 uint32_t wide_tile(bool key64, uint32_t val_bytes) {
@@ -107,13 +106,20 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
 
     if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
     if (key64) {
-        uint32_t grid = (uint32_t)di.sm_count * 4u;
-        const uint32_t need = (n + HIST8_THREADS - 1) / HIST8_THREADS;
+        const bool few = n <= (1u << 21), typed = key_type != KEY_U64;
+        constexpr int T4 = 512, T16 = 1024;
+        const size_t smem = (few ? HIST8_COL_WORDS<4> : HIST8_COL_WORDS<16>) * sizeof(uint32_t);
+        auto kern = few ? (typed ? k_hist8<T4, 4, true> : k_hist8<T4, 4, false>)
+                        : (typed ? k_hist8<T16, 16, true> : k_hist8<T16, 16, false>);
+        static DeviceOnce smem_set[4];  // per instance
+        st = allow_smem_once(kern, smem, smem_set[(few ? 2 : 0) + (typed ? 1 : 0)]);
+        if (st != RS_OK) return st;
+        const uint32_t threads = few ? T4 : T16;
+        uint32_t grid = (uint32_t)di.sm_count * (few ? 2u : 1u);
+        const uint32_t need = (uint32_t)(((size_t)n + 4 * threads - 1) / (4 * threads));
         if (grid > need) grid = need;
-        auto kern = key_type == KEY_U64 ? k_hist8<HIST8_THREADS, false>
-                                        : k_hist8<HIST8_THREADS, true>;
         note_launch_begin(KK_HIST, stream);
-        kern<<<grid, HIST8_THREADS, 0, stream>>>(
+        kern<<<grid, threads, smem, stream>>>(
             static_cast<const unsigned long long*>(keys), n, &ctrl->hist[0][0],
             static_cast<uint4*>(status[0]), (uint32_t)(status_bytes / sizeof(uint4)), key_type);
         note_launch_end(KK_HIST, stream);
