@@ -56,10 +56,11 @@ struct BinSortSmem {
     // Up to the power of two at or above CAP bins (chunks, whose words have no room
     // for more: 2048 or 4096), scanned by the largest power of two of threads.
     static constexpr uint32_t BIN_BITS =
-        CAP <= 1024 ? 10 : CAP <= (CHUNKS ? 2560 : 2048) ? 11 : CHUNKS || CAP <= 4096 ? 12 : 13;
+        CAP <= 512 ? 9 : CAP <= 1024 ? 10 : CAP <= (CHUNKS ? 2560 : 2048) ? 11 : CHUNKS || CAP <= 4096 ? 12 : 13;
     static constexpr uint32_t MAX_BINS = 1u << BIN_BITS;
     static constexpr uint32_t SCANNERS = THREADS >= 1024 ? 1024 : THREADS >= 512 ? 512
-                                         : THREADS >= 256 ? 256 : 128;
+                                         : THREADS >= 256 ? 256
+                                         : THREADS >= 128 ? 128 : 64;
     static constexpr uint32_t COUNTERS = (THREADS / 32) * RADIX * 4;
     static constexpr uint32_t BINS = MAX_BINS * 4 > COUNTERS ? MAX_BINS * 4 : COUNTERS;
     static constexpr uint32_t WORDS = (CAP + 2 * ITEMS) * (uint32_t)sizeof(K);
@@ -101,20 +102,35 @@ __device__ __forceinline__ void sort8(W (&w)[8]) {
     order(2, 4), order(3, 5);
     order(1, 2), order(3, 4), order(5, 6);
 }
-// Sorts the eight words at p (16-byte aligned, in shared memory).
+// Its last steps: merges w[0..3] and w[4..7], each sorted.
 template <typename W>
+__device__ __forceinline__ void merge8(W (&w)[8]) {
+    auto order = [&](int i, int j) {
+        const W a = w[i], b = w[j];
+        w[i] = min(a, b);
+        w[j] = max(a, b);
+    };
+    order(0, 4), order(1, 5), order(2, 6), order(3, 7);
+    order(2, 4), order(3, 5);
+    order(1, 2), order(3, 4), order(5, 6);
+}
+// Sorts the eight words at p (16-byte aligned, in shared memory); HALVES: the first
+// and the last four are sorted already.
+template <bool HALVES, typename W>
 __device__ __forceinline__ void sort_window(W* p) {
     constexpr int VECS = 8 * sizeof(W) / 16;
     union {
         uint4 v[VECS];
         W w[8];
     } u;
-    // Any order will do for the loads: turned so that the eight lanes of a
-    // 16-byte access fall into 32 different banks.
-    const int turn = (threadIdx.x * VECS >> 3) & (VECS - 1);
+    // Any order (HALVES: of the halves) will do for the loads: turned so that the
+    // eight lanes of a 16-byte access fall into 32 different banks (two into each,
+    // for halves of 64-bit words).
+    const int turn = (threadIdx.x * VECS >> 3) & (HALVES ? VECS / 2 : VECS - 1);
 #pragma unroll
     for (int i = 0; i < VECS; ++i) u.v[i] = reinterpret_cast<const uint4*>(p)[i ^ turn];
-    sort8(u.w);
+    if constexpr (HALVES) merge8(u.w);
+    else sort8(u.w);
 #pragma unroll
     for (int i = 0; i < VECS; ++i) reinterpret_cast<uint4*>(p)[i] = u.v[i];
 }
@@ -526,9 +542,9 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 if (tid == 0) s_bigs = 0;  // for the next array (read above, before a barrier)
                 __syncthreads();
             }
-            if (tid < windows) sort_window(s_w + 8 * tid);
+            if (tid < windows) sort_window<false>(s_w + 8 * tid);
             __syncthreads();
-            if (tid < windows) sort_window(s_w + 8 * tid + 4);
+            if (tid < windows) sort_window<true>(s_w + 8 * tid + 4);
             if (PAIRS) cp_async_wait_all();
             __syncthreads();
             // ---- 4. stored in order -----------------------------------------

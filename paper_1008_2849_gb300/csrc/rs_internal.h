@@ -250,13 +250,11 @@ rs_status launch_single_sort(uint32_t* keys, uint32_t* vals, uint32_t n, int bit
                              uint32_t key_type, cudaStream_t stream);
 uint32_t small_sort_capacity();
 
-// One-warp sort in shared memory: of every tiny segment listed by the
-// segmented planner (off != nullptr), or of the single array [0, single_n)
-// with single_n <= warp_sort_capacity().  bits: digit width, 4 or 8.
-rs_status launch_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* off,
-                           const uint32_t* tiny_list, const Ctrl* ctrl, uint32_t single_n,
-                           int bits, uint32_t key_type, cudaStream_t stream,
-                           const uint32_t* src_keys = nullptr, const uint32_t* src_vals = nullptr);
+// The same sorts of the tiny segments listed by the planner (at most
+// warp_sort_capacity() items each): by a CTA of two warps, or with bits = 4 one warp.
+rs_status launch_tiny_list(uint32_t* keys, uint32_t* vals, const uint32_t* off,
+                           const uint32_t* tiny_list, const Ctrl* ctrl, int bits,
+                           uint32_t key_type, cudaStream_t stream);
 uint32_t warp_sort_capacity();
 
 // Workspace layout of a segmented sort of n items in num_segments segments.

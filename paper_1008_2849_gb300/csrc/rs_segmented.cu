@@ -93,7 +93,7 @@ rs_status enqueue_sort_segmented(uint32_t* keys, uint32_t* vals, uint32_t n,
 
     // Tiny and small segments: independent of the large ones (disjoint ranges).
     if (warp_max >= 2) {
-        st = launch_warp_sort(keys, vals, offsets, tiny_list, ctrl, 0, ck.small_bits, key_type,
+        st = launch_tiny_list(keys, vals, offsets, tiny_list, ctrl, ck.small_bits, key_type,
                               stream);
         if (st != RS_OK) return st;
     }

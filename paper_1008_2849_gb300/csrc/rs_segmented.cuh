@@ -3,8 +3,7 @@
 // A segmented sort sorts every segment [off[s], off[s+1]) of one array on its
 // own (the paper has no segmented case; this is the plain definition applied
 // per segment).  Segments are routed by size (rs_small.cuh has the first two):
-//   tiny (2 <= size <= warp_max): k_warp_sort, one warp per segment, the whole
-//       segment in that warp's shared memory for every pass;
+//   tiny (2 <= size <= warp_max): k_bin_sort with a CTA of two warps per segment;
 //   small (warp_max < size <= small_max): k_bin_sort (rs_bin_sort.cuh), one CTA
 //       per segment, the whole segment on chip -- one read and one write of
 //       every item either way;

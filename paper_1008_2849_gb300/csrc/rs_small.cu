@@ -89,20 +89,20 @@ rs_status launch_small_any(uint32_t max_items, int bits, const SmallWork& w,
                              : launch_small_size<false>(max_items, bits, w, stream);
 }
 
-template <int BITS, bool PAIRS>
-rs_status launch_warp_bits(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,
-                           const uint32_t* src_vals, const uint32_t* off,
-                           const uint32_t* list, const Ctrl* ctrl, uint32_t single_n,
-                           uint32_t grid, uint32_t key_type, cudaStream_t stream) {
-    using L = WarpSortSmem<WARP_SORT_ITEMS, BITS, PAIRS>;
-    auto kern = k_warp_sort<WARP_SORT_ITEMS, BITS, PAIRS>;
+template <bool PAIRS>
+rs_status launch_warp4(const SmallWork& w, cudaStream_t stream) {
+    using L = WarpSortSmem<WARP_SORT_ITEMS, 4, PAIRS>;
+    auto kern = k_warp_sort<WARP_SORT_ITEMS, 4, PAIRS>;
     static DeviceOnce smem_set;
     rs_status st = allow_smem_once(kern, L::BYTES, smem_set);
     if (st != RS_OK) return st;
+    uint32_t grid = 0;
+    st = grid_of(w, 3, &grid);
+    if (st != RS_OK) return st;
     note_launch_begin(KK_WARP, stream);
-    const cudaError_t e =
-        launch_after_previous(kern, dim3(grid), dim3(WARP_SORT_THREADS), L::BYTES, stream, keys,
-                              vals, src_keys, src_vals, off, list, ctrl, single_n, key_type);
+    const cudaError_t e = launch_after_previous(kern, dim3(grid), dim3(WARP_SORT_THREADS), L::BYTES,
+                                                stream, w.keys, w.vals, w.off, w.list, w.ctrl,
+                                                w.key_type);
     note_launch_end(KK_WARP, stream);
     return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
@@ -162,27 +162,15 @@ rs_status launch_single_sort(uint32_t* keys, uint32_t* vals, uint32_t n, int bit
     return launch_small_any(n, bits, w, stream);
 }
 
-rs_status launch_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* off,
-                           const uint32_t* tiny_list, const Ctrl* ctrl, uint32_t single_n,
-                           int bits, uint32_t key_type, cudaStream_t stream,
-                           const uint32_t* src_keys, const uint32_t* src_vals) {
-    if (off == nullptr && single_n > warp_sort_capacity()) return RS_ERR_INVALID_ARG;
-    DeviceInfo di;
-    rs_status st = device_info(&di);
-    if (st != RS_OK) return st;
-    const uint32_t grid = off == nullptr ? 1u : (uint32_t)di.sm_count * 3u;
-    const bool pairs = vals != nullptr;
-    const uint32_t* sk = src_keys ? src_keys : keys;
-    const uint32_t* sv = src_keys ? src_vals : vals;
+rs_status launch_tiny_list(uint32_t* keys, uint32_t* vals, const uint32_t* off,
+                           const uint32_t* tiny_list, const Ctrl* ctrl, int bits,
+                           uint32_t key_type, cudaStream_t stream) {
+    const SmallWork w{keys, vals, keys, vals, off, tiny_list, 1, &ctrl->tiny_count, ctrl, 0,
+                      key_type};
     if (bits == 4)
-        return pairs ? launch_warp_bits<4, true>(keys, vals, sk, sv, off, tiny_list, ctrl, single_n,
-                                                 grid, key_type, stream)
-                     : launch_warp_bits<4, false>(keys, vals, sk, sv, off, tiny_list, ctrl,
-                                                  single_n, grid, key_type, stream);
-    return pairs ? launch_warp_bits<8, true>(keys, vals, sk, sv, off, tiny_list, ctrl, single_n,
-                                             grid, key_type, stream)
-                 : launch_warp_bits<8, false>(keys, vals, sk, sv, off, tiny_list, ctrl, single_n,
-                                              grid, key_type, stream);
+        return vals != nullptr ? launch_warp4<true>(w, stream) : launch_warp4<false>(w, stream);
+    return vals != nullptr ? launch_bin_shape<true, 64, 16>(w, stream)
+                           : launch_bin_shape<false, 64, 16>(w, stream);
 }
 
 }  // namespace rs

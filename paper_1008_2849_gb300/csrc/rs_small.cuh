@@ -1,15 +1,11 @@
-// rs_small.cuh -- sorts of arrays that fit in on-chip memory by counting passes:
-// the one-warp sort (k_warp_sort) and the one-CTA sort with 4-bit digits
-// (k_small_sort; the default one-CTA sort is k_bin_sort).  Both run the
+// rs_small.cuh -- sorts of arrays that fit in on-chip memory by counting passes of
+// 4-bit digits: the one-warp sort (k_warp_sort) and the one-CTA sort
+// (k_small_sort), the alternative of the bin sort (rs_bin_sort.cuh).  Both run the
 // stable counting-sort passes of Sec. 3 between two shared-memory buffers, so
-// every item is read from and written to global memory once.  The digit width
-// BITS is a template parameter: 8 bits (four passes, 256 buckets, as in the
-// scatter passes) or 4 bits (eight passes, 16 buckets) -- which is faster
-// depends on the array size, and the autotuner picks it per size class.
-// Either width gives the same stable order.  Typed keys (key_type) are mapped
-// onto their ordered words when read and back when written.  An array is read
-// from src_keys / src_vals and written to keys / vals at the same offsets (the
-// same arrays for an in-place sort; the other buffer after an MSD pass).
+// every item is read from and written to global memory once.  Typed keys
+// (key_type) are mapped onto their ordered words when read and back when written.
+// k_small_sort reads from src_keys / src_vals and writes to keys / vals at the same
+// offsets (the same arrays for an in-place sort; the other buffer after an MSD pass).
 #pragma once
 
 #include "rs_device.cuh"
@@ -37,8 +33,7 @@ struct WarpSortSmem {
 // ---------------------------------------------------------------------------
 // k_warp_sort: every warp sorts whole arrays of at most 32 * ITEMS items, one
 // at a time, in its own shared-memory region, with no CTA-wide barrier.
-// Arrays are the segments listed in `list` (count ctrl->tiny_count), or with
-// off == nullptr the single array [0, single_n).  Per pass: the digit counts
+// Arrays are the segments listed in `list` (count ctrl->tiny_count).  Per pass: the digit counts
 // of the array (shared atomics), their exclusive prefix over digits (each
 // lane scans 2^BITS / 32 counters, then a warp scan), then the items slot by
 // slot in input order: the lanes holding the same digit come from one ballot
@@ -49,9 +44,8 @@ struct WarpSortSmem {
 // ---------------------------------------------------------------------------
 template <int ITEMS, int BITS, bool PAIRS>
 __global__ void __launch_bounds__(WARP_SORT_THREADS)
-k_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uint32_t* src_vals,
-            const uint32_t* __restrict__ off, const uint32_t* __restrict__ list,
-            const Ctrl* __restrict__ ctrl, uint32_t single_n, uint32_t key_type) {
+k_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* __restrict__ off,
+            const uint32_t* __restrict__ list, const Ctrl* __restrict__ ctrl, uint32_t key_type) {
     using L = WarpSortSmem<ITEMS, BITS, PAIRS>;
     pdl_launch_next();
     pdl_wait();  // the kernel before this one (planner, MSD pass) is complete
@@ -68,21 +62,14 @@ k_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys, const uint
     uint32_t* const cnt = s_k + (PAIRS ? 4 : 2) * CAP;
     const uint32_t lt = lanemask_lt();
 
-    uint32_t count = 1;
-    if (off != nullptr) {
-        if (ctrl->err != 0) return;
-        count = ctrl->tiny_count;
-    }
+    if (ctrl->err != 0) return;
+    const uint32_t count = ctrl->tiny_count;
     for (uint32_t idx = blockIdx.x * WARPS + warp; idx < count; idx += gridDim.x * WARPS) {
-        uint32_t lo = 0, m = single_n;
-        if (off != nullptr) {
-            const uint32_t s = list[idx];
-            lo = off[s];
-            m = off[s + 1] - lo;
-        }
+        const uint32_t s = list[idx];
+        const uint32_t lo = off[s], m = off[s + 1] - lo;
         for (uint32_t i = lane; i < m; i += 32) {
-            s_k[i] = key_to_ordered(src_keys[lo + i], key_type);
-            if (PAIRS) s_v[i] = src_vals[lo + i];
+            s_k[i] = key_to_ordered(keys[lo + i], key_type);
+            if (PAIRS) s_v[i] = vals[lo + i];
         }
         uint32_t cur = 0;
         for (uint32_t p = 0; p < NPASS; ++p) {
