@@ -138,13 +138,14 @@ __device__ __forceinline__ void sort_window(W* p) {
 // ---------------------------------------------------------------------------
 // sort_in_global: one CTA sorts the m items at a (stable, in place) by counting
 // passes over the 8-bit digits that differ, between a and b of the same size,
-// through counters s_cnt[THREADS / 32][RADIX], s_base[RADIX] and s_hist[RADIX].
+// through counters s_cnt[THREADS / 32][RADIX], s_base[RADIX] and s_hist[RADIX].  The
+// result is left in a, or with to_b in b.
 // For the rare chunk that the top-digits order leaves too long for the chip:
 // about 1 item per ns, so it counts on there being few of them.
 // ---------------------------------------------------------------------------
 template <typename K, typename V, bool PAIRS, int THREADS>
-__device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, uint32_t m,
-                                            uint32_t key_type, uint32_t* s_cnt, uint32_t* s_base,
+__device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, bool to_b,
+                                            uint32_t m, uint32_t key_type, uint32_t* s_cnt, uint32_t* s_base,
                                             uint32_t* s_hist) {
     constexpr uint32_t WARPS = THREADS / 32, SLOTS = 4, TILE = THREADS * SLOTS;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -214,10 +215,10 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
         }
         in_a = !in_a;
     }
-    if (!in_a) {
+    if (in_a == to_b) {
         for (uint32_t i = tid; i < m; i += THREADS) {
-            a_k[i] = b_k[i];
-            if (PAIRS) a_v[i] = b_v[i];
+            (to_b ? b_k : a_k)[i] = (to_b ? a_k : b_k)[i];
+            if (PAIRS) (to_b ? b_v : a_v)[i] = (to_b ? a_v : b_v)[i];
         }
         __syncthreads();
     }
@@ -229,9 +230,11 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
 // listed in `list` (every `step`-th entry from it; count in *list_count), or with
 // list == nullptr the segments 0, 1, ..., or with step == 0 the ranges (first item,
 // items) in `list`; or with off == nullptr the single array [0, single_n).
-// CHUNKS: the segments 0, 1, ... (list == nullptr), sorted in place; longer ones
-// than CAP in global memory, with the other buffer at spare_keys / spare_vals
-// (sort_in_global); their keys share the single_n highest bits.
+// CHUNKS: the chunks 0, 1, ... of the top-digits order (list == nullptr), read from
+// keys / vals or spare_keys / spare_vals (ctrl->chunk_src) and sorted by the digits
+// from ctrl->chunk_digit on already (32-bit keys: the single_n highest bits of a chunk
+// are the same); longer ones than CAP are sorted in global memory
+// (sort_in_global).
 //
 // For an array of m items, with nb = 2^bb bins (m <= nb < 2m; chunks at most
 // MAX_BINS):
@@ -257,7 +260,7 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, u
 // The word has the width of the key: the key itself without values; else the key's
 // distance from the smallest, moved up until the largest has its highest bit set, with
 // the index in the lowest bits.  In chunks, whose keys share as many bits as an index
-// takes, that is the whole key.  Elsewhere its lowest bits may be lost: words that differ in their index only are put in order by their
+// takes, that is the whole distance.  Elsewhere its lowest bits may be lost: words that differ in their index only are put in order by their
 // keys in step 4 (for 4096 keys that spread evenly, eight such pairs).
 //
 // What bounds it: instruction issue (135 warp instructions per 32 pairs, 61 % of the
@@ -306,7 +309,8 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
            const uint32_t* __restrict__ list_count, const Ctrl* __restrict__ ctrl,
            uint32_t single_n, uint32_t key_type, K* spare_keys, V* spare_vals) {
     using L = BinSortSmem<K, V, PAIRS, THREADS, CHUNKS>;
-    constexpr bool WHOLE = !PAIRS || CHUNKS;  // words hold whole keys
+    constexpr bool WHOLE = !PAIRS || CHUNKS;            // words hold whole keys
+    constexpr bool BY_PREFIX = CHUNKS && sizeof(K) == 4;  // 32-bit chunks all are
     constexpr int ITEMS = L::ITEMS;
     constexpr uint32_t WARPS = THREADS / 32;
     constexpr uint32_t SCANNERS = L::SCANNERS;
@@ -331,6 +335,11 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         if (ctrl->err != 0) return;
         count = *list_count;
     }
+    K sorted = 0;  // chunks: the bits of the digits they are sorted by
+    if (CHUNKS && count != 0) {
+        sorted = ~K(0) << (8 * ctrl->chunk_digit);
+        if (ctrl->chunk_src != 0) src_keys = spare_keys, src_vals = spare_vals;
+    }
     const bool typed = key_type != KEY_U32 && key_type != KEY_U64;
     if (tid == 0) s_min = ~K(0), s_max = 0, s_bigs = 0;
     for (uint32_t idx = blockIdx.x; idx < count; idx += gridDim.x) {
@@ -345,14 +354,15 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 m = off[s + 1] - lo;
             }
             if (!CHUNKS && (m == 0 || m > L::CAP)) continue;
-            if (CHUNKS && m < 2) continue;
+            if (CHUNKS && m == 0) continue;
             if constexpr (CHUNKS) {
                 if (m > L::CAP) {
                     __syncthreads();  // the array before is done with shared memory
+                    const bool b = ctrl->chunk_src != 0;
                     sort_in_global<K, V, PAIRS, THREADS>(
-                        keys + lo, PAIRS ? vals + lo : nullptr, spare_keys + lo,
-                        PAIRS ? spare_vals + lo : nullptr, m, key_type, s_bin,
-                        reinterpret_cast<uint32_t*>(s_w),
+                        (b ? spare_keys : keys) + lo, PAIRS ? (b ? spare_vals : vals) + lo : nullptr,
+                        (b ? keys : spare_keys) + lo, PAIRS ? (b ? vals : spare_vals) + lo : nullptr,
+                        b, m, key_type, s_bin, reinterpret_cast<uint32_t*>(s_w),
                         reinterpret_cast<uint32_t*>(s_w) + RADIX);
                     continue;
                 }
@@ -373,11 +383,16 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) k[j] = key_to_ordered(k[j], key_type);
         }
-        // Chunks: their keys share the single_n highest bits.
-        K least, most, range = ~K(0) >> (CHUNKS ? single_n : 0u);
+        K least, most;
         if constexpr (CHUNKS) {
-            least = key_to_ordered(from[0], key_type) & ~range;
-            most = least | range;
+            if constexpr (BY_PREFIX) {  // the keys share their single_n highest bits
+                const K low_bits = ~K(0) >> single_n;
+                least = key_to_ordered(from[0], key_type) & ~low_bits;
+                most = least | low_bits;
+            } else {  // the ends' sorted digits say
+                least = key_to_ordered(from[0], key_type) & sorted;
+                most = key_to_ordered(from[m - 1], key_type) | ~sorted;
+            }
             __syncthreads();  // the bins are zero; the array before is done with the rest
         } else {
             K lo_k = ~K(0), not_hi = ~K(0);
@@ -398,28 +413,31 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
             __syncthreads();
             least = s_min;
             most = s_max;
-            range = (most - least) | 1;
         }
+        const K range = (most - least) | 1;
         if (PAIRS) {
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
                 if (tid + j * THREADS < m)
                     cp_async_elem(s_v + tid + j * THREADS, src_vals + lo + tid + j * THREADS);
         }
-        const uint32_t top = CHUNKS ? single_n : leading_zeros(range);  // zero bits of a distance
+        const uint32_t top = BY_PREFIX ? single_n : leading_zeros(range);  // bits of 0 in all
         // Bins: distance * scale / 2^32, of the (high words of the) distances moved up
-        // by `top`; scale = nb * 2^32 / (range + 1), rounded down.
-        const uint32_t scale =
-            CHUNKS ? nb
-                   : (uint32_t)(((unsigned long long)nb << 32) /
-                                ((unsigned long long)high_word((K)(range << top)) + 1));
+        // by `top`; scale is nb * 2^32 / (range + 1), or up to 2e-6 of it less (a
+        // quotient of floats, kept below the exact one, so that every bin is below nb).
+        uint32_t scale = nb;
+        if constexpr (!BY_PREFIX)
+            scale = (uint32_t)(__fdividef((float)nb * 4294967296.0f,
+                                          (float)high_word((K)(range << top))) * 0.999999f);
         // Scanning thread t scans the `per` consecutive bins from t * per on,
         // four at a time; their groups of four are swizzled so that the eight
         // lanes of a 16-byte access fall into 32 different banks.
         const uint32_t per = nb > SCANNERS ? nb / SCANNERS : 1u;  // 1, 2, 4, 8 or 16
         const uint32_t swizzle = per > 4 ? (per / 4 - 1) << 2 : 0u;
         auto bin_of = [&](K x) {
-            const uint32_t b = __umulhi(high_word((K)((CHUNKS ? x : x - least) << top)), scale);
+            const uint32_t b = BY_PREFIX
+                                   ? high_word((K)(x << top)) >> (32 - bb)
+                                   : __umulhi(high_word((K)((x - least) << top)), scale);
             return b ^ ((b >> 3) & swizzle);
         };
 
@@ -517,15 +535,15 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         __syncthreads();
         const uint32_t bigs = s_bigs;
 
-        // (Chunks whose words would not hold whole keys take the digit passes too;
-        // the choice of chunks leaves none.)
+        // (Chunks whose words would not hold whole keys take the digit passes too: none
+        // by prefix; by position, where the keys are sparse.)
         if (work <= m && (!CHUNKS || ib <= top)) {
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
                 if (tid + j * THREADS < m) {
                     const uint32_t i = tid + j * THREADS;
                     K w = k[j];
-                    if (PAIRS && CHUNKS) w = (w << top) | (K)i;  // (least << top is 0)
+                    if (PAIRS && CHUNKS) w = ((BY_PREFIX ? w : w - least) << top) | (K)i;
                     if (PAIRS && !CHUNKS) w = ((w - least) << top >> ib << ib) | (K)i;
                     s_w[s_bin[bin_of(k[j])] + at[j]] = w;
                     if (!WHOLE) s_k[i] = k[j];
@@ -557,7 +575,7 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                     const uint32_t i = (uint32_t)w & imask;
                     K key;
                     if constexpr (WHOLE) {
-                        key = PAIRS ? (K)(w >> top) | least : w;
+                        key = PAIRS ? (K)(w >> top) + least : w;
                     } else {
                         // Words next to each other may differ in their index only
                         // because the key's last bits did not fit: those few

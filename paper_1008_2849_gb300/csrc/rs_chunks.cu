@@ -1,5 +1,7 @@
 // rs_chunks.cu -- the end of the top-digits order, for items of every width: the
 // chunk bounds and the on-chip sorts of the chunks.
+#include <algorithm>
+
 #include "rs_bin_sort.cuh"
 #include "rs_hist_plan.cuh"
 #include "rs_internal.h"
@@ -34,11 +36,16 @@ rs_status run(K* keys, V* vals, K* spare_keys, V* spare_vals, uint32_t n, const 
     DeviceInfo di;
     const rs_status st = device_info(&di);
     if (st != RS_OK) return st;
+    // At most 2^bits chunks by prefix, or one every capacity / 2 items.
+    const size_t by_position = sizeof(K) == 8 ? ((size_t)n + top.capacity / 2 - 1) /
+                                                    (top.capacity / 2) : 0;
+    const size_t most = std::max(size_t(1) << top.bits, by_position);
     const uint32_t ways = top.bits <= 14 ? 32 : 8;
     note_launch_begin(KK_CHUNK_BOUNDS, stream);
     const cudaError_t e = launch_after_previous(
-        ways == 32 ? k_chunk_bounds<K, 32> : k_chunk_bounds<K, 8>, dim3((ways << top.bits) / 256),
-        dim3(256), 0, stream, (const K*)keys, n, ctrl, top.bits, key_type, off);
+        ways == 32 ? k_chunk_bounds<K, 32> : k_chunk_bounds<K, 8>,
+        dim3((uint32_t)((ways * most + 255) / 256)), dim3(256), 0, stream, (const K*)keys,
+        (const K*)spare_keys, n, ctrl, top.bits, key_type, off);
     note_launch_end(KK_CHUNK_BOUNDS, stream);
     if (e != cudaSuccess) return RS_ERR_CUDA;
 #define RS_CHUNKS(T, B)                                                                     \

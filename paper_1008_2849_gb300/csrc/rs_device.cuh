@@ -58,7 +58,10 @@ struct Ctrl {
     // (chunk_count counts their runs) and of those that take all passes.
     uint32_t msd_tiles;
     uint32_t lsd_tiles;
-    uint32_t pad[4];               // keep hist 64-byte aligned
+    uint32_t chunk_digit;          // top-digits order: the lowest digit with a pass
+    uint32_t chunk_step;           // chunks by position, this many items apart (0: by prefix)
+    uint32_t chunk_src;            // chunks read from: 0 caller's arrays, 1 alternate buffers
+    uint32_t pad[1];               // keep hist 64-byte aligned
     uint32_t hist[PASSES64][RADIX];  // digit histograms (H); 0..3 for 32-bit keys
     uint32_t gofs[PASSES64][RADIX];  // first output slot of every bucket (G)
 };

@@ -211,6 +211,11 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
 // share (the digits may be even one by one and not together).  Chunks that are
 // too long all the same are sorted in global memory by one CTA each, so a
 // sample that misses them costs time, not correctness.
+//
+// 64-bit keys that are not even may still take the passes by their two to four highest
+// digits that differ, if that saves two passes or more and the sample has no crowd of
+// keys that these digits do not tell apart (normal doubles: three passes instead of
+// eight).  Their chunks are chunk_step items long, up to the next change of prefix.
 // ---------------------------------------------------------------------------
 constexpr uint32_t TOP_SAMPLES = 4096;
 constexpr uint32_t TOP_MAX_BITS = 16;
@@ -223,10 +228,12 @@ struct PlanArgs {
     const void* keys;
     uint32_t n, key_type, bucket_cap;
     uint32_t* msd_off;
-    uint32_t top_bits;
+    uint32_t top_bits, chunk_step;
 };
 
-// Dynamic shared memory: 2 << top_bits bytes when top_bits is set.
+// Dynamic shared memory when top_bits is set: 2 << top_bits bytes, and at least
+// 2 << TOP_HASH_BITS.
+constexpr uint32_t TOP_HASH_BITS = 13;
 template <int NPASS>
 __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     extern __shared__ uint4 s_dyn[];
@@ -273,10 +280,10 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     uint32_t executed = 0;
     for (uint32_t q = 0; q < NPASS; ++q) executed += s_trivial[q] ? 0 : 1;
     bool top = !msd && top_bits != 0 && !s_uneven && executed >= 3;
-    if (top) {  // the same for every thread
+    const bool deep = NPASS == 8 && top_bits != 0 && executed >= 4;
+    uint32_t low = 0;  // the lowest digit with a pass
+    if (top || deep) {  // the same for every thread
         uint32_t* const s_pair = reinterpret_cast<uint32_t*>(s_dyn);  // two 16-bit counts a word
-        const uint32_t chunks = 1u << top_bits;
-        for (uint32_t i = tid; i < (chunks + 7) / 8; i += 1024) s_dyn[i] = make_uint4(0, 0, 0, 0);
         const K* const keys = static_cast<const K*>(plan.keys);
         constexpr uint32_t PER = TOP_SAMPLES / 1024;
         const uint32_t stride = n / TOP_SAMPLES;
@@ -288,19 +295,47 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
             r ^= r >> 15;
             r *= 0x85EBCA6Bu;
             const uint32_t at = (uint32_t)(((uint64_t)i * n) / TOP_SAMPLES) + __umulhi(r, stride);
-            k[q] = keys[at];
+            k[q] = key_to_ordered(keys[at], plan.key_type);
         }
-        __syncthreads();
+        // Whether no cell of the 2^bits that `cell` tells apart holds over `most` keys.
+        auto spread = [&](uint32_t bits, uint32_t most, auto cell) -> bool {
+            __syncthreads();
+            if (tid == 0) s_uneven = 0;
+            for (uint32_t i = tid; i < (1u << bits) / 8; i += 1024)
+                s_dyn[i] = make_uint4(0, 0, 0, 0);
+            __syncthreads();
 #pragma unroll
-        for (uint32_t q = 0; q < PER; ++q) {
-            const uint32_t c =
-                (uint32_t)(key_to_ordered(k[q], plan.key_type) >> (8 * sizeof(K) - top_bits));
-            const uint32_t was = atomicAdd(&s_pair[c >> 1], 1u << (16 * (c & 1)));
-            if (((was >> (16 * (c & 1))) & 0xffffu) >= 2 * (TOP_SAMPLES >> top_bits) + 12)
-                s_uneven = 1;
+            for (uint32_t q = 0; q < PER; ++q) {
+                const uint32_t c = cell(k[q]);
+                const uint32_t was = atomicAdd(&s_pair[c >> 1], 1u << (16 * (c & 1)));
+                if (((was >> (16 * (c & 1))) & 0xffffu) >= most) s_uneven = 1;
+            }
+            __syncthreads();
+            return !s_uneven;
+        };
+        if (top) {
+            low = NPASS - 2;
+            top = spread(top_bits, 2 * (TOP_SAMPLES >> top_bits) + 12,
+                         [&](K x) { return (uint32_t)(x >> (8 * sizeof(K) - top_bits)); });
         }
-        __syncthreads();
-        top = !s_uneven;
+        if (deep && !top) {
+            const uint32_t most =
+                (uint32_t)(2ull * TOP_SAMPLES * plan.chunk_step / n) + 10;
+            uint32_t passes = 0;
+            for (low = NPASS; !top && low-- > 0;) {
+                if (s_trivial[low]) continue;
+                ++passes;
+                if (passes > 4 || passes + 2 > executed) break;
+                if (passes < 2) continue;
+                top = spread(TOP_HASH_BITS, most, [&](K x) {
+                    const unsigned long long h =
+                        (unsigned long long)(x >> (8 * low)) * 0x9E3779B97F4A7C15ull;
+                    return (uint32_t)(h >> (64 - TOP_HASH_BITS));
+                });
+                if (top) break;
+            }
+            if (tid == 0 && top) ctrl->chunk_step = plan.chunk_step;
+        }
     }
     if (msd && (tid >> 8) == PASSES - 1) {
         plan.msd_off[b] = first3;
@@ -309,9 +344,11 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     if (tid != 0) return;
     ctrl->dir[MSD_SLOT] = msd ? DIR_A_TO_B : DIR_SKIP;
     ctrl->small_count = msd ? RADIX : 0u;
-    ctrl->chunk_count = top ? 1u << top_bits : 0u;
+    const uint32_t step = top ? ctrl->chunk_step : 0u;  // written above, by this thread
+    ctrl->chunk_count = !top ? 0u : step != 0 ? (n + step - 1) / step : 1u << top_bits;
+    ctrl->chunk_digit = low;
     bool skip[NPASS];
-    for (uint32_t q = 0; q < NPASS; ++q) skip[q] = msd || s_trivial[q] || (top && q < NPASS - 2);
+    for (uint32_t q = 0; q < NPASS; ++q) skip[q] = msd || s_trivial[q] || (top && q < low);
     if (!msd && !top && (executed & 1)) {
         for (uint32_t q = 0; q < NPASS; ++q)
             if (skip[q]) { skip[q] = false; break; }
@@ -325,35 +362,58 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
             parity ^= 1;
         }
     }
+    ctrl->chunk_src = parity;
 }
 
 // ---------------------------------------------------------------------------
 // k_chunk_bounds: the chunks of the top-digits order, once the array is sorted
-// by its top 16 bits: off[c] = the first key with its top_bits highest bits
-// equal to c or more, off[1 << top_bits] = n.  WAYS lanes search together for
-// each bound in the bucket of its highest digit (G of that digit says where it
-// lies), reading WAYS keys at a time that cut what is left into WAYS + 1 parts:
-// dependent reads are what takes the time, and 32 ways need 3 to 4 of them where
-// halving needs 13 to 16 (14 us for 8192 chunks of 2^24 keys).  Many chunks take
-// fewer ways, for the keys read.
+// by its top digits, chunk_digit and above: off[c] = the first item of chunk c,
+// off[chunk_count] = n.  Chunks by prefix: the first key with its top_bits highest
+// bits equal to c or more.  Chunks by position: the first key with the prefix of
+// item c * chunk_step.
+// WAYS lanes search together for each bound (by prefix, in the bucket of its highest
+// digit: G of that digit says where it lies; by position, in a stretch before the item
+// that is made longer until it holds another prefix), reading WAYS keys at a time that
+// cut what is left into WAYS + 1 parts: dependent reads are what takes the time, and 32
+// ways need 3 to 4 of them where halving needs 13 to 16 (14 us for 8192 chunks of 2^24
+// keys).  Many chunks take fewer ways, for the keys read.
 // ---------------------------------------------------------------------------
 template <typename K, int WAYS>
 __global__ void __launch_bounds__(256)
-k_chunk_bounds(const K* __restrict__ keys, uint32_t n, const Ctrl* __restrict__ ctrl,
-               uint32_t top_bits, uint32_t key_type, uint32_t* __restrict__ off) {
+k_chunk_bounds(const K* __restrict__ keys_a, const K* __restrict__ keys_b, uint32_t n,
+               const Ctrl* __restrict__ ctrl, uint32_t top_bits, uint32_t key_type,
+               uint32_t* __restrict__ off) {
     pdl_launch_next();
     pdl_wait();  // the scatter passes are complete
-    if (ctrl->chunk_count == 0) return;
-    const uint32_t chunks = 1u << top_bits;
+    const uint32_t chunks = ctrl->chunk_count;
+    if (blockIdx.x * (256 / WAYS) >= chunks) return;
+    const K* const keys = ctrl->chunk_src ? keys_b : keys_a;
     const uint32_t way = threadIdx.x % WAYS;
     const uint32_t first_lane = (threadIdx.x & 31) / WAYS * WAYS;
-    // (chunks is a multiple of the bounds per CTA: the grid is exact.)
-    const uint32_t c = (blockIdx.x * 256 + threadIdx.x) / WAYS;
-    if (c == 0 && way == 0) off[chunks] = n;
-    const uint32_t* const g = ctrl->gofs[sizeof(K) - 1];
-    const uint32_t b = c >> (top_bits - RADIX_BITS);
-    uint32_t lo = g[b], hi = b + 1 < RADIX ? g[b + 1] : n;  // the answer is in [lo, hi]
-    const K want = (K)c << (8 * sizeof(K) - top_bits);
+    // (Lanes past the last chunk search for it too, with their warp.)
+    const uint32_t mine = (blockIdx.x * 256 + threadIdx.x) / WAYS;
+    const uint32_t c = mine < chunks ? mine : chunks - 1;
+    if (mine == 0 && way == 0) off[chunks] = n;
+    const uint32_t step = ctrl->chunk_step;
+    uint32_t lo, hi;  // the answer is in [lo, hi]
+    K want;           // the first key not below it
+    if (step == 0) {
+        const uint32_t* const g = ctrl->gofs[sizeof(K) - 1];
+        const uint32_t b = c >> (top_bits - RADIX_BITS);
+        lo = g[b];
+        hi = b + 1 < RADIX ? g[b + 1] : n;
+        want = (K)c << (8 * sizeof(K) - top_bits);
+    } else {
+        const uint32_t shift = 8 * ctrl->chunk_digit;
+        hi = c * step;
+        want = key_to_ordered(keys[hi], key_type) >> shift << shift;
+        uint32_t width = step;
+        lo = hi > width ? hi - width : 0;
+        while (lo > 0 && key_to_ordered(keys[lo], key_type) >= want) {
+            width = width < (1u << 28) ? width * 8 : width;
+            lo = lo > width ? lo - width : 0;
+        }
+    }
     while (__any_sync(0xffffffffu, lo < hi)) {
         const uint32_t part = (hi - lo) / (WAYS + 1) + 1;  // keys left of the first cut, at most
         const uint32_t at = lo + (way + 1) * part - 1;
@@ -365,7 +425,7 @@ k_chunk_bounds(const K* __restrict__ keys, uint32_t n, const Ctrl* __restrict__ 
         hi = min(hi, next + part - 1);
         lo = min(next, hi);
     }
-    if (way == 0) off[c] = lo;
+    if (way == 0 && mine < chunks) off[c] = lo;
 }
 
 // ---------------------------------------------------------------------------

@@ -100,10 +100,11 @@ rs_status enqueue_plan(const PlanArgs& plan, cudaStream_t stream) {
     static DeviceOnce smem_set;
     const rs_status st = allow_smem_once(k_plan<NPASS>, TOP_PLAN_SMEM, smem_set);
     if (st != RS_OK) return st;
+    const uint32_t bits = plan.top_bits > TOP_HASH_BITS ? plan.top_bits : TOP_HASH_BITS;
     note_launch_begin(KK_PLAN, stream);
-    const cudaError_t e = launch_after_previous(
-        k_plan<NPASS>, dim3(1), dim3(1024), plan.top_bits ? sizeof(uint16_t) << plan.top_bits : 0,
-        stream, plan);
+    const cudaError_t e =
+        launch_after_previous(k_plan<NPASS>, dim3(1), dim3(1024),
+                              plan.top_bits ? sizeof(uint16_t) << bits : 0, stream, plan);
     note_launch_end(KK_PLAN, stream);
     return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
@@ -186,7 +187,7 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     const TopOrder top = ck.msd != 0 ? top_order(n) : TopOrder{0, 0};
     uint32_t* msd_off = reinterpret_cast<uint32_t*>(ws + L.msd_off);
     const PlanArgs plan{ctrl, keys, n, key_type, bucket_capacity(long_buckets),
-                        msd ? msd_off : nullptr, top.bits};
+                        msd ? msd_off : nullptr, top.bits, 0u};
 
     if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
     st = enqueue_hist4(keys, n, &ctrl->hist[0][0], status[0], status_bytes, key_type, stream);

@@ -140,3 +140,41 @@ def test_32_bit_keys_with_64_bit_values(rs):
     place = np.argsort(k.view(np.int32), kind="stable")
     assert np.array_equal(to_host(kd), k[place])
     assert np.array_equal(vd.cpu().numpy().view(np.uint64), v[place])
+
+
+def _uneven_keys(kind, n, seed):
+    rng = np.random.default_rng(seed)
+    if kind == "normal":
+        return rng.standard_normal(n).view(np.uint64)
+    if kind == "low40":   # the top digits never differ
+        return rng.integers(0, 1 << 40, n, dtype=np.uint64)
+    if kind == "and2":
+        return rng.integers(0, 1 << 63, n, dtype=np.uint64) & rng.integers(0, 1 << 63, n, dtype=np.uint64)
+    if kind == "hidden crowd":  # some 6000 keys of one prefix, too few to be sampled
+        k = rng.standard_normal(n).view(np.uint64)
+        k[11:12_011:2] = (k[11:12_011:2] & np.uint64(0xFFFF)) | np.uint64(0x3FF1234500000000)
+        return k
+    return np.sort(rng.standard_normal(n)).view(np.uint64)[::-1].copy()  # "reverse"
+
+
+@pytest.mark.parametrize("n", [1 << 14, 65_537, (1 << 20) + 5, 4_500_003])
+@pytest.mark.parametrize("key_type,value_bits", [("u64", 0), ("i64", 32), ("f64", 64)])
+def test_uneven_wide_keys(rs, n, key_type, value_bits):
+    """Keys that take more than two passes by their highest digits, and chunks by
+    position: 64-bit keys that crowd, with digits that never differ, and with a
+    crowd that the plan cannot see."""
+    import torch
+    for kind in ("normal", "low40", "and2", "hidden crowd", "reverse"):
+        k = _uneven_keys(kind, n, 7 + n % 11)
+        v = None
+        if value_bits:
+            v = np.arange(n, dtype=np.uint64 if value_bits == 64 else np.uint32)
+        kd = torch.from_numpy(k.view(np.int64)).cuda()
+        vd = None
+        if v is not None:
+            vd = torch.from_numpy(v.view(np.int64 if value_bits == 64 else np.int32)).cuda()
+        rs.sort_kv(kd, vd, key_type)
+        ko, vo = oracle.sort_kv(k, v, key_type)
+        assert np.array_equal(kd.cpu().numpy().view(np.uint64), ko), kind
+        if v is not None:
+            assert np.array_equal(vd.cpu().numpy().view(v.dtype), vo), kind
