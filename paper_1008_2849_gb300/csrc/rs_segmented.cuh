@@ -176,7 +176,7 @@ k_seg_hist(const uint32_t* __restrict__ keys, const Ctrl* __restrict__ ctrl,
     };
     // Counts the keys [lo, hi): up to 3 before the first 16-byte boundary
     // and up to 3 after the last one one by one, the rest as 16-byte
-    // vectors, two in flight per thread.
+    // vectors, four in flight per thread.
     auto count_range = [&](uint32_t lo, uint32_t hi) {
         const uint32_t* src = keys + lo;
         const uint32_t m = hi - lo;
@@ -184,15 +184,19 @@ k_seg_hist(const uint32_t* __restrict__ keys, const Ctrl* __restrict__ ctrl,
         if (head > m) head = m;
         const uint32_t nvec = (m - head) >> 2;
         const uint4* body = reinterpret_cast<const uint4*>(src + head);
-        uint32_t v = tid;
-        for (; v + T < nvec; v += 2 * T) {
-            const uint4 x = ld_stream(body + v), y = ld_stream(body + v + T);
-            count_key(x.x); count_key(x.y); count_key(x.z); count_key(x.w);
-            count_key(y.x); count_key(y.y); count_key(y.z); count_key(y.w);
-        }
-        if (v < nvec) {
-            const uint4 x = ld_stream(body + v);
-            count_key(x.x); count_key(x.y); count_key(x.z); count_key(x.w);
+        constexpr uint32_t LOADS = 4;
+        for (uint32_t v = tid; v < nvec; v += LOADS * T) {
+            uint4 x[LOADS];
+#pragma unroll
+            for (uint32_t u = 0; u < LOADS; ++u)
+                if (v + u * T < nvec) x[u] = ld_stream(body + v + u * T);
+#pragma unroll
+            for (uint32_t u = 0; u < LOADS; ++u) {
+                if (v + u * T < nvec) {
+                    count_key(x[u].x), count_key(x[u].y);
+                    count_key(x[u].z), count_key(x[u].w);
+                }
+            }
         }
         const uint32_t tail = head + nvec * 4;
         if (tid < head) count_key(ld_stream(src + tid));
