@@ -88,6 +88,8 @@ class RsError(RuntimeError):
 def lib():
     """The loaded librs.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -124,10 +126,20 @@ def _dev_ptr(t, name: str, width: int = 4) -> int:
     return t.data_ptr()
 
 
-def _stream_handle(stream) -> int:
+def _current_stream_handle() -> int:
+    """The current stream's handle.  torch.cuda.current_stream() builds a Stream
+    object for it, 2.9 us of the 7.3 that a call of sort_keys_ex took on the host;
+    the handle alone takes 0.2 where torch offers it."""
     import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch._C._cuda_getDevice())
+
+
+def _stream_handle(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return _current_stream_handle()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
