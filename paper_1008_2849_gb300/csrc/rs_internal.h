@@ -175,8 +175,8 @@ rs_status enqueue_sort11(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_
 
 // Wide items: 64-bit keys (eight passes; key_type KEY_U64, KEY_I64 or
 // KEY_F64) carrying no, 32-bit or 64-bit values (val_bytes 0, 4 or 8), and
-// 32-bit keys (KEY_U32, KEY_I32, KEY_F32) carrying 64-bit values.  Every
-// array size takes the scatter passes.
+// 32-bit keys (KEY_U32, KEY_I32, KEY_F32) carrying 64-bit values.  Arrays of up to
+// kWideSmallMax items are sorted on chip, longer ones take scatter passes.
 Layout layout_wide(size_t n, bool key64, uint32_t val_bytes);
 rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_type,
                             uint32_t val_bytes, cudaStream_t stream, void* workspace,
@@ -233,6 +233,14 @@ rs_status launch_bucket_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* sr
                               const uint32_t* src_vals, const uint32_t* off,
                               const uint32_t* count, const Ctrl* ctrl, bool long_buckets,
                               int bits, uint32_t key_type, cudaStream_t stream);
+// The bin sort of wide items (rs_small_wide.cu): of the single array [0, n), n <=
+// kWideSmallMax, and of the segments of up to as many items that are listed by size.
+constexpr uint32_t kWideSmallMax = 4096;
+rs_status launch_single_wide(void* keys, void* vals, uint32_t n, uint32_t key_type,
+                             uint32_t val_bytes, cudaStream_t stream);
+rs_status launch_lists_wide(void* keys, void* vals, const uint32_t* off, const uint32_t* tiny_list,
+                            const uint32_t* small_list, uint32_t entries, const Ctrl* ctrl,
+                            uint32_t key_type, uint32_t val_bytes, cudaStream_t stream);
 // One-CTA sorts on chip of *count ranges (first item, items) at `runs`, of at most 4096
 // items each.
 rs_status launch_run_sorts(uint32_t* keys, uint32_t* vals, const uint32_t* src_keys,

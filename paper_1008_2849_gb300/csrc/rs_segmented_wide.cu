@@ -1,8 +1,8 @@
 // rs_segmented_wide.cu -- host side of the segmented sort of wide items:
 // 64-bit keys (eight passes) with no, 32-bit or 64-bit values, and 32-bit
 // keys with 64-bit values (four passes); unsigned or typed keys.  Segments
-// of up to kWideWarpMax items are sorted by one warp each in shared memory;
-// every longer segment takes the segmented scatter passes.
+// of up to kWideSmallMax items are sorted on chip by one CTA each; every longer
+// segment takes the segmented scatter passes.
 #include "rs_internal.h"
 #include "rs_onesweep_launch.cuh"
 #include "rs_segmented.cuh"
@@ -12,8 +12,7 @@ namespace rs {
 
 namespace {
 
-constexpr int kWideWarpItems = 8;                             // one warp: up to 256 items
-constexpr uint32_t kWideWarpMax = 32u * kWideWarpItems;
+constexpr uint32_t kLeastLarge = kWideSmallMax + 1;  // items of the smallest large segment
 constexpr int B_SEG = 2, W_SEG = 8;
 
 uint32_t wide_items(bool key64, uint32_t val_bytes) {
@@ -47,21 +46,6 @@ rs_status seg_pass(uint32_t key_type, K* ka, V* va, K* kb, V* vb, uint32_t n, ui
         key_type | ROLE_MAP_PASSES, stream);
 }
 
-template <typename K, typename V, bool PAIRS>
-rs_status warp_sort(K* keys, V* vals, const uint32_t* off, const uint32_t* tiny_list,
-                    const Ctrl* ctrl, uint32_t key_type, int sm_count, cudaStream_t stream) {
-    using L = WideWarpSmem<K, V, PAIRS, kWideWarpItems>;
-    auto kern = k_warp_sort_wide<K, V, PAIRS, kWideWarpItems>;
-    static DeviceOnce smem_set;
-    rs_status st = allow_smem_once(kern, L::BYTES, smem_set);
-    if (st != RS_OK) return st;
-    note_launch_begin(KK_WARP, stream);
-    kern<<<sm_count * 4, WIDE_WARP_THREADS, L::BYTES, stream>>>(keys, vals, off, tiny_list, ctrl,
-                                                               key_type);
-    note_launch_end(KK_WARP, stream);
-    return cudaPeekAtLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
-}
-
 // The whole sequence for one combination of key and value widths.
 template <typename K, typename V, bool PAIRS>
 rs_status run(K* keys, V* vals, uint32_t n, const uint32_t* offsets, uint32_t num_segments,
@@ -87,15 +71,14 @@ rs_status run(K* keys, V* vals, uint32_t n, const uint32_t* offsets, uint32_t nu
     if (L.max_large > 0 &&
         cudaMemsetAsync(gofs, 0, (size_t)L.max_large * NP * RADIX * 4, stream) != cudaSuccess)
         return RS_ERR_CUDA;
-    // Segments of up to kWideWarpMax items: one warp each; every longer one
-    // is large (no one-CTA class for wide items).
     note_launch_begin(KK_SEG_PLAN, stream);
     k_seg_plan<<<(num_segments + 1023) / 1024, 1024, 0, stream>>>(
-        offsets, num_segments, n, tile, kWideWarpMax, kWideWarpMax, ctrl, di.sticky, tile_geo,
-        L.max_tiles, tiny_list, small_list, large_first, L.max_large, NP);
+        offsets, num_segments, n, tile, warp_sort_capacity(), kWideSmallMax, ctrl, di.sticky,
+        tile_geo, L.max_tiles, tiny_list, small_list, large_first, L.max_large, NP);
     note_launch_end(KK_SEG_PLAN, stream);
     if (cudaPeekAtLastError() != cudaSuccess) return RS_ERR_CUDA;
-    st = warp_sort<K, V, PAIRS>(keys, vals, offsets, tiny_list, ctrl, key_type, di.sm_count, stream);
+    st = launch_lists_wide(keys, vals, offsets, tiny_list, small_list, num_segments, ctrl, key_type,
+                           PAIRS ? (uint32_t)sizeof(V) : 0u, stream);
     if (st != RS_OK) return st;
 
     note_launch_begin(KK_SEG_HIST, stream);
@@ -139,7 +122,7 @@ rs_status run(K* keys, V* vals, uint32_t n, const uint32_t* offsets, uint32_t nu
 SegLayout seg_layout_wide(size_t n, bool key64, uint32_t val_bytes, uint32_t num_segments) {
     SegLayout L{};
     const size_t tile = (size_t)kWideThreads * wide_items(key64, val_bytes);
-    const size_t large = std::min<size_t>(num_segments, n / (kWideWarpMax + 1) + 1);
+    const size_t large = std::min<size_t>(num_segments, n / kLeastLarge + 1);
     const uint32_t np = key64 ? PASSES64 : PASSES;
     L.max_large = (uint32_t)large;
     L.max_tiles = (uint32_t)((n + tile - 1) / tile + large);

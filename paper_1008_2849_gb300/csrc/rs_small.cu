@@ -1,9 +1,7 @@
-// rs_small.cu -- host launchers of the on-chip sorts (rs_small.cuh): the
-// one-warp sort and the one-CTA sort, each at digit width 4 or 8.
-#include <type_traits>
-
-#include "rs_internal.h"
+// rs_small.cu -- host launchers of the on-chip sorts of 32-bit keys with no or 32-bit
+// values: the bin sort (rs_bin_sort.cuh), or the 4-bit counting passes of rs_small.cuh.
 #include "rs_bin_sort.cuh"
+#include "rs_internal.h"
 #include "rs_small.cuh"
 
 namespace rs {
