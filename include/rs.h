@@ -187,8 +187,9 @@ size_t rs_workspace_bytes64(size_t n, int with_values);
  * ones work the same way; Sec. 4 leaves K general.  64-bit keys take eight
  * passes (K = 64, D = 8) and a value of any width moves with its key.
  * 32-bit keys with no or 32-bit values take the calls above (same workspace
- * size, same kernels); every other combination takes the scatter passes for
- * every array size (no on-chip sort of small arrays, no MSD-first order).
+ * size, same kernels); every other combination sorts arrays of up to 4096 items
+ * on chip in one launch, and longer ones by the scatter passes, or by the highest
+ * digits first and on chip from there where the keys allow it.
  * d_keys is aligned to its key width, d_vals to its value width; keys and
  * values do not overlap; n < 2^32; workspace_bytes >=
  * rs_workspace_bytes_kv(n, key_type, value_bits), the workspace 256-byte
@@ -209,9 +210,9 @@ size_t rs_workspace_bytes_kv(size_t n, int key_type, int value_bits);
  * rs_sort_pairs_segmented (nondecreasing, last entry <= n, each segment
  * < 2^30 items; a bad table is reported as RS_ERR_BAD_SEGMENTS and nothing
  * is written).  32-bit keys with no or 32-bit values take the 32-bit
- * segmented sorts; every other combination sorts segments of up to 256
- * items in one warp each (in shared memory) and every longer one with the
- * scatter passes (eight for 64-bit keys).  Pointer, alignment, overlap and
+ * segmented sorts; every other combination sorts segments of up to 4096
+ * items on chip, one CTA each, and every longer one with the scatter passes (eight
+ * for 64-bit keys).  Pointer, alignment, overlap and
  * type rules as for rs_sort_kv_ex; workspace_bytes >=
  * rs_workspace_bytes_kv_segmented(n, key_type, value_bits, num_segments),
  * 256-byte aligned.  Asynchronous on cuda_stream, in place, stable;

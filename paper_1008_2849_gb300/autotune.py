@@ -13,8 +13,9 @@ under every candidate setting and keeps the fastest:
   width;
 * segmented batches: the tile shape of the segmented scatter passes and the
   largest segment sorted by the one-CTA sort (4096 or 8192); for batches of
-  short arrays the largest segment sorted by the one-warp sort and the digit
-  width of the on-chip sorts (4 bits, eight passes, or 8 bits, four passes).
+  short arrays the largest segment listed apart (two-warp CTAs of the bin sort,
+  or one warp in 4-bit passes) and which on-chip sorts run (8: the bin sort; 4: the
+  counting sorts by 4-bit digits).
 
 Results never depend on the settings, only speed does.  The table is JSON:
 

@@ -13,18 +13,18 @@
    uniform; AND of 2, 3 and 4 uniform words; 256 distinct values; all keys
    equal; sorted; reverse sorted; low 16 bits only.  Each step sorts a fresh
    copy (1 GiB, larger than L2) with rs_sort_pairs_ex; reported are pairs/s
-   (median step) and the number of scatter passes that ran -- a digit that is
+   (median step) and the number of scatter passes that ran: two where the keys
+   are sorted on chip from there, else one for every digit -- a digit that is
    the same for every key makes its pass the identity, and it is skipped.
 3. Typed keys at 2^27 pairs of random 32-bit words (seed 21), read as
    signed integers and as IEEE floats (rs_sort_typed_ex); and float-key
    pairs of 2^14..2^26 items with two scatter-pass instances per pass
    against one (RS_TUNE_TYPED_SPLIT), as graph replays.
 4. 64-bit keys with 32-bit values, 2^27 pairs of random words (seed 22),
-   eight passes (rs_sort64_ex).
+   rs_sort64_ex.
 5. Wide items through rs_sort_kv_ex at 2^27 items of random words (seed
-   23): 32-bit keys with 64-bit values (four passes), 64-bit keys (unsigned
-   and IEEE binary64) with 64-bit values and signed 64-bit keys alone (eight
-   passes).
+   23): 32-bit keys with 64-bit values, 64-bit keys (unsigned and IEEE binary64)
+   with 64-bit values and signed 64-bit keys alone.
 6. Digit width of the whole-array sort: four 8-bit passes (rs_sort_pairs_ex,
    rs_sort_keys_ex) against three 11/11/10-bit passes (rs_sort_digits11_ex)
    with every tile shape of its scatter kernel, pairs and keys only of
@@ -158,9 +158,8 @@ def main(argv=None) -> int:
         rs.check_stream()
         # Scatter-pass launches per sort; a launch whose pass is skipped
         # returns at once (it is still counted as a launch).
-        hist = rs.digit_histograms(k).cpu().numpy().view(np.uint32)
         sweep[dist] = {"seed": 3 + i, "ms": ms, "pairs_per_s": n / (ms / 1e3),
-                       "passes_executed": _executed_passes(hist, n),
+                       "passes_executed": _executed_passes(ws, 4),
                        "scatter_launches_per_sort": launches // (a.steps + a.warmup)}
         del k
     out["pairs_2^27_distributions"] = sweep
@@ -186,7 +185,7 @@ def main(argv=None) -> int:
     # pass (half the launches), each as the replay of a captured graph.
     out["typed_f32_pairs_split_vs_single"] = _typed_split_sweep(torch, rs, inputs, stream, a)
 
-    # 4. 64-bit keys (eight passes) with 32-bit values, 2^27 pairs of random
+    # 4. 64-bit keys with 32-bit values, 2^27 pairs of random
     # words (seed 22): 1 GiB of keys.
     hi = inputs.splitmix32(22, n, 0).astype(np.uint64)
     lo = inputs.splitmix32(22, n, 1).astype(np.uint64)
@@ -204,7 +203,8 @@ def main(argv=None) -> int:
                 a.warmup)
     rs.check_stream()
     out["pairs_2^27_key64_value32"] = {"ms": ms, "pairs_per_s": n / (ms / 1e3),
-                                       "bytes_per_pair_per_pass": 24, "passes": 8}
+                                       "bytes_per_pair_per_pass": 24,
+                                       "passes": _executed_passes(ws, 8)}
     del kb, vb, ws, raw
 
     # 5. wide items (rs_sort_kv_ex), 2^27 items of random words (seed 23)
@@ -235,12 +235,12 @@ def main(argv=None) -> int:
         ms = _timed(torch, stream, lambda: rs.sort_kv_ex(kb, vb, key_type, ws, stream), restore,
                     a.steps, a.warmup)
         rs.check_stream()
-        passes = 8 if kw == 8 else 4
+        passes = _executed_passes(ws, 8 if kw == 8 else 4)
         per_pass = 2 * (kw + value_bits // 8)
         wide["%s_keys_%d_bit_values" % (key_type, value_bits)] = {
             "ms": ms, "items_per_s": n / (ms / 1e3), "passes": passes,
             "bytes_per_item_per_pass": per_pass,
-            "scatter_tb_per_s": n * per_pass * passes / (ms / 1e3) / 1e12}
+            "scatter_tb_per_s_of_whole_sort": n * per_pass * passes / (ms / 1e3) / 1e12}
         del k, kb, vb, ws, raw
     out["items_2^27_wide"] = wide
     del i64
@@ -332,13 +332,11 @@ def _typed_split_sweep(torch, rs, inputs, stream, a):
     return rows
 
 
-def _executed_passes(hist, n):
-    """Scatter passes that move data, from the digit histograms: a digit whose
-    histogram has one bucket holding all n keys is the identity and skipped;
-    one identity pass is added back when needed to keep the count even (the
-    result must end in the caller's buffer)."""
-    moving = int(sum(1 for p in range(4) if int(hist[p].max()) != n))
-    return moving + (moving & 1)
+def _executed_passes(ws, passes):
+    """Scatter passes of the last sort that moved data: those that took tiles (the
+    workspace's control block begins with the error word, then the tiles taken by
+    passes 0, 1, ...)."""
+    return int((ws[4:4 + 4 * passes].cpu().numpy().view(np.uint32) > 0).sum())
 
 
 if __name__ == "__main__":

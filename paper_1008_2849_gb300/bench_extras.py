@@ -3,8 +3,8 @@ the latency of the small keys-only sort, the batched segmented sort against
 a loop of per-array sorts, and p50/p99 latency of the serving loop against
 serial plain sorts.  Each leg samples the SM clocks while it runs.
 
-* latency: 2^20 uniform uint32 keys (seed 1), keys only, four 8-bit LSD
-  passes; device time (CUDA events) of one rs_sort_keys_ex and of one replay
+* latency: 2^20 uniform uint32 keys (seed 1), keys only;
+  device time (CUDA events) of one rs_sort_keys_ex and of one replay
   of a captured graph of it, median over the steps.  The 4 MiB array stays
   in the 129 MB L2 between steps, so this is a latency, not a roofline case.
 * batch: 4096 arrays of (uint32 key, uint32 value = index inside the array),
@@ -67,7 +67,7 @@ def latency_keys_2pow20(device_index: int, steps: int = 20, warmup: int = 5) -> 
     ok = bool(torch.equal(k.cpu(), torch.from_numpy(
         np.sort(src.cpu().numpy().view(np.uint32)).view(np.int32))))
     return {"call_ms": call_ms, "graph_replay_ms": graph_ms, "keys": n, "steps": steps,
-            "workload": "2^20 uniform uint32 keys, seed 1, keys only, 4 x 8-bit passes "
+            "workload": "2^20 uniform uint32 keys, seed 1, keys only "
                         "(L2-resident between steps)",
             "sorted": ok, "clocks": _clocks(sampler)}
 

@@ -1,8 +1,10 @@
-// rs_hist_plan.cuh -- the two small kernels that precede the scatter passes:
-//   k_hist4  one read of the keys builds all four digit histograms (the
-//            counting step of Sec. 3, for every digit at once);
+// rs_hist_plan.cuh -- the small kernels around the scatter passes:
+//   k_hist4, k_hist4_cols, k_hist8  one read of the keys builds the histograms of
+//            all four (eight) digits (the counting step of Sec. 3, for every
+//            digit at once);
 //   k_plan   exclusive prefix over the buckets of every digit (Sec. 3 "prefix
-//            sum"; Alg. 2 PrefixSum) and the pass plan.
+//            sum"; Alg. 2 PrefixSum), the order of the digits and the pass plan;
+//   k_chunk_bounds  where the chunks of the top-digits order begin.
 #pragma once
 
 #include <type_traits>

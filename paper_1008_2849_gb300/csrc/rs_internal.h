@@ -67,8 +67,9 @@ int smallest_tile();
 constexpr int kTypedShape = 3;
 
 // Per size class tuning (chosen by the autotuner): tile shapes (indices into
-// kTileConfigs), the largest array / segment sorted by the one-warp sort and
-// by the one-CTA sort, and the digit width of those two sorts.
+// kTileConfigs), the largest array / segment sorted on chip (small_max; up to warp_max
+// in the smallest CTAs), and the on-chip sorts taken (small_bits: 8, the bin sort, or
+// 4, the counting sorts by 4-bit digits).
 struct ClassKnobs {
     int tile_pairs;
     int tile_keys;

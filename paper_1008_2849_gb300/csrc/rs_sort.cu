@@ -163,8 +163,7 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     rs_status st = device_info(&di);
     if (st != RS_OK) return st;
     const ClassKnobs& ck = knobs().cls[size_class(n)];
-    // A single small array takes one CTA (one warp alone measured slower);
-    // the one-warp sort serves batches of short segments and MSD buckets.
+    // A single small array takes one CTA.
     if (n <= (uint32_t)ck.small_max && n <= small_sort_capacity())
         return launch_single_sort(keys, vals, n, ck.small_bits, key_type, stream);
     // Three passes of 11/11/10-bit digits, where the size class takes them
