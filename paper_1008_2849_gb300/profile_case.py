@@ -8,7 +8,7 @@ Builds librs.so if needed, copies the input to the GPU, runs rs_sort_pairs_ex
 status.  It times nothing: a profiler (ncu) around it sees exactly the
 library's kernels (per sort of 2^25 items and more: one histogram, one plan, four
 scatter-pass launches, of which those the plan leaves out return at once, the chunk
-boundaries and four chunk sorts by size).  With --digits11 SHAPE it runs rs_sort_digits11_ex instead (three
+boundaries and the sort of the chunks).  With --digits11 SHAPE it runs rs_sort_digits11_ex instead (three
 passes of 11/11/10-bit digits, scatter-kernel tile shape SHAPE; per sort:
 three counting, three scan and three scatter launches).  2^26 pairs is 256
 MiB per array, more than the L2, and small enough for a many-pass capture to
