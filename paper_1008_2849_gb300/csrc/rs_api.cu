@@ -221,6 +221,7 @@ const char* kernel_kind_name(int kind) {
     case KK_D11_SCAN: return "d11_scan";
     case KK_D11_DOWN: return "d11_down";
     case KK_CHUNK_BOUNDS: return "chunk_bounds";
+    case KK_CLEAR: return "clear";
     default: return nullptr;
     }
 }

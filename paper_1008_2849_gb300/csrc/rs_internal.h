@@ -30,6 +30,7 @@ enum KernelKind : int {
     KK_D11_SCAN = 10,
     KK_D11_DOWN = 11,
     KK_CHUNK_BOUNDS = 12,
+    KK_CLEAR = 13,
     KK_COUNT
 };
 const char* kernel_kind_name(int kind);
@@ -198,8 +199,12 @@ rs_status enqueue_histograms(const uint32_t* keys, uint32_t n, uint32_t* hist,
                              cudaStream_t stream);
 // The same, added into hist (zeroed by the caller), counting the digits of
 // the ordered words of typed keys, and clearing clear_bytes at `clear`.
+// (after_clear: enqueue_clear was the last launch on the stream.)
 rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* clear,
-                        size_t clear_bytes, uint32_t key_type, cudaStream_t stream);
+                        size_t clear_bytes, uint32_t key_type, cudaStream_t stream,
+                        bool after_clear = false);
+// Zeroes the control block.
+rs_status enqueue_clear(Ctrl* ctrl, cudaStream_t stream);
 // The plan kernel (rs_hist_plan.cuh), for keys of NPASS digits.
 struct PlanArgs;
 template <int NPASS> rs_status enqueue_plan(const PlanArgs& plan, cudaStream_t stream);
@@ -308,6 +313,16 @@ cudaError_t launch_after_previous(void (*kern)(Params...), dim3 grid, dim3 block
     cfg.attrs = attr;
     cfg.numAttrs = knobs().pdl ? 1u : 0u;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
+// A histogram kernel: beside the clearing of its counts, when that is the launch before.
+template <typename... Params, typename... Args>
+cudaError_t launch_hist(bool after_clear, void (*kern)(Params...), dim3 grid, dim3 block,
+                        size_t smem, cudaStream_t stream, Args&&... args) {
+    if (after_clear)
+        return launch_after_previous(kern, grid, block, smem, stream, std::forward<Args>(args)...);
+    kern<<<grid, block, smem, stream>>>(std::forward<Args>(args)...);
+    return cudaPeekAtLastError();
 }
 
 // One bit per device (ordinal < 64) for one-time host setup of a kernel

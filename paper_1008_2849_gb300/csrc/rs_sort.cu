@@ -43,8 +43,16 @@ Layout layout_for(size_t n, bool pairs) {
     return L;
 }
 
+rs_status enqueue_clear(Ctrl* ctrl, cudaStream_t stream) {
+    note_launch_begin(KK_CLEAR, stream);
+    k_clear_ctrl<<<1, 1024, 0, stream>>>(reinterpret_cast<uint4*>(ctrl));
+    note_launch_end(KK_CLEAR, stream);
+    return cudaPeekAtLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
+}
+
 rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* clear,
-                        size_t clear_bytes, uint32_t key_type, cudaStream_t stream) {
+                        size_t clear_bytes, uint32_t key_type, cudaStream_t stream,
+                        bool after_clear) {
     DeviceInfo di;
     rs_status st = device_info(&di);
     if (st != RS_OK) return st;
@@ -69,10 +77,11 @@ rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* 
         const uint32_t need = few ? (vec4 + 2 * T8 - 1) / (2 * T8) : (vec4 + T32 - 1) / T32;
         if (grid > need) grid = need > 0 ? need : 1;
         note_launch_begin(KK_HIST, stream);
-        kern<<<grid, few ? T8 : T32, smem, stream>>>(keys, n, hist, static_cast<uint4*>(clear),
-                                         (uint32_t)(clear_bytes / sizeof(uint4)), key_type);
+        const cudaError_t e = launch_hist(
+            after_clear, kern, dim3(grid), dim3(few ? T8 : T32), smem, stream, keys, n, hist,
+            static_cast<uint4*>(clear), (uint32_t)(clear_bytes / sizeof(uint4)), key_type);
         note_launch_end(KK_HIST, stream);
-        return cudaPeekAtLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
+        return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
     }
     const bool typed = key_type != KEY_U32;
     auto kern = typed ? k_hist4<HIST_THREADS, HIST_LEADER, true>
@@ -188,8 +197,9 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     const PlanArgs plan{ctrl, keys, n, key_type, bucket_capacity(long_buckets),
                         msd ? msd_off : nullptr, top.bits, 0u};
 
-    if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
-    st = enqueue_hist4(keys, n, &ctrl->hist[0][0], status[0], status_bytes, key_type, stream);
+    st = enqueue_clear(ctrl, stream);
+    if (st != RS_OK) return st;
+    st = enqueue_hist4(keys, n, &ctrl->hist[0][0], status[0], status_bytes, key_type, stream, true);
     if (st != RS_OK) return st;
     st = enqueue_plan<PASSES>(plan, stream);
     if (st != RS_OK) return st;

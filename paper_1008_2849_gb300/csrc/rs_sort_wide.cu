@@ -108,7 +108,8 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
     void* alt_v = val_bytes ? ws + L.alt_vals : nullptr;
     const uint32_t npass = key64 ? PASSES64 : PASSES;
 
-    if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
+    st = enqueue_clear(ctrl, stream);
+    if (st != RS_OK) return st;
     if (key64) {
         const bool few = n <= (1u << 21), typed = key_type != KEY_U64;
         constexpr int T4 = 512, T16 = 1024;
@@ -123,14 +124,15 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
         const uint32_t need = (uint32_t)(((size_t)n + 4 * threads - 1) / (4 * threads));
         if (grid > need) grid = need;
         note_launch_begin(KK_HIST, stream);
-        kern<<<grid, threads, smem, stream>>>(
+        const cudaError_t e = launch_hist(
+            true, kern, dim3(grid), dim3(threads), smem, stream,
             static_cast<const unsigned long long*>(keys), n, &ctrl->hist[0][0],
             static_cast<uint4*>(status[0]), (uint32_t)(status_bytes / sizeof(uint4)), key_type);
         note_launch_end(KK_HIST, stream);
-        if (cudaPeekAtLastError() != cudaSuccess) return RS_ERR_CUDA;
+        if (e != cudaSuccess) return RS_ERR_CUDA;
     } else {
         st = enqueue_hist4(static_cast<const uint32_t*>(keys), n, &ctrl->hist[0][0], status[0],
-                           status_bytes, key_type, stream);
+                           status_bytes, key_type, stream, true);
         if (st != RS_OK) return st;
     }
     // Keys that spread evenly: two passes, then chunks on chip (see enqueue_sort).
