@@ -203,8 +203,9 @@ rs_status enqueue_histograms(const uint32_t* keys, uint32_t n, uint32_t* hist,
 rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* clear,
                         size_t clear_bytes, uint32_t key_type, cudaStream_t stream,
                         bool after_clear = false);
-// Zeroes the control block.
-rs_status enqueue_clear(Ctrl* ctrl, cudaStream_t stream);
+// Zeroes the control block, and more_bytes (a multiple of 16) at `more`.
+rs_status enqueue_clear(Ctrl* ctrl, cudaStream_t stream, void* more = nullptr,
+                        size_t more_bytes = 0);
 // The plan kernel (rs_hist_plan.cuh), for keys of NPASS digits.
 struct PlanArgs;
 template <int NPASS> rs_status enqueue_plan(const PlanArgs& plan, cudaStream_t stream);
@@ -315,7 +316,8 @@ cudaError_t launch_after_previous(void (*kern)(Params...), dim3 grid, dim3 block
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// A histogram kernel: beside the clearing of its counts, when that is the launch before.
+// A first kernel: beside the clearing of its counts (it waits for that before it uses
+// them), when that is the launch before.
 template <typename... Params, typename... Args>
 cudaError_t launch_hist(bool after_clear, void (*kern)(Params...), dim3 grid, dim3 block,
                         size_t smem, cudaStream_t stream, Args&&... args) {

@@ -80,16 +80,15 @@ rs_status enqueue_sort_segmented(uint32_t* keys, uint32_t* vals, uint32_t n,
     uint32_t warp_max = (uint32_t)ck.warp_max;
     if (warp_max > warp_sort_capacity()) warp_max = warp_sort_capacity();
 
-    if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
-    if (L.max_large > 0 &&
-        cudaMemsetAsync(gofs, 0, (size_t)L.max_large * PASSES * RADIX * 4, stream) != cudaSuccess)
-        return RS_ERR_CUDA;
+    st = enqueue_clear(ctrl, stream, gofs, (size_t)L.max_large * PASSES * RADIX * 4);
+    if (st != RS_OK) return st;
     note_launch_begin(KK_SEG_PLAN, stream);
-    k_seg_plan<<<(num_segments + 1023) / 1024, 1024, 0, stream>>>(
-        offsets, num_segments, n, tile, warp_max, small_max, ctrl, di.sticky, tile_geo,
-        L.max_tiles, tiny_list, small_list, large_first, L.max_large);
+    const cudaError_t planned = launch_after_previous(
+        k_seg_plan, dim3((num_segments + 1023) / 1024), dim3(1024), 0, stream, offsets,
+        num_segments, n, tile, warp_max, small_max, ctrl, di.sticky, tile_geo, L.max_tiles,
+        tiny_list, small_list, large_first, L.max_large, (uint32_t)PASSES);
     note_launch_end(KK_SEG_PLAN, stream);
-    if (cudaPeekAtLastError() != cudaSuccess) return RS_ERR_CUDA;
+    if (planned != cudaSuccess) return RS_ERR_CUDA;
 
     // Tiny and small segments: independent of the large ones (disjoint ranges).
     if (warp_max >= 2) {

@@ -67,16 +67,15 @@ rs_status run(K* keys, V* vals, uint32_t n, const uint32_t* offsets, uint32_t nu
     const uint32_t tile = (uint32_t)kWideThreads * wide_items(sizeof(K) == 8, PAIRS ? sizeof(V) : 0);
     const size_t status_vec4 = (L.status1 - L.status0) / sizeof(uint4);
 
-    if (cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), stream) != cudaSuccess) return RS_ERR_CUDA;
-    if (L.max_large > 0 &&
-        cudaMemsetAsync(gofs, 0, (size_t)L.max_large * NP * RADIX * 4, stream) != cudaSuccess)
-        return RS_ERR_CUDA;
+    st = enqueue_clear(ctrl, stream, gofs, (size_t)L.max_large * NP * RADIX * 4);
+    if (st != RS_OK) return st;
     note_launch_begin(KK_SEG_PLAN, stream);
-    k_seg_plan<<<(num_segments + 1023) / 1024, 1024, 0, stream>>>(
-        offsets, num_segments, n, tile, warp_sort_capacity(), kWideSmallMax, ctrl, di.sticky,
-        tile_geo, L.max_tiles, tiny_list, small_list, large_first, L.max_large, NP);
+    const cudaError_t planned = launch_after_previous(
+        k_seg_plan, dim3((num_segments + 1023) / 1024), dim3(1024), 0, stream, offsets,
+        num_segments, n, tile, warp_sort_capacity(), kWideSmallMax, ctrl, di.sticky, tile_geo,
+        L.max_tiles, tiny_list, small_list, large_first, L.max_large, (uint32_t)NP);
     note_launch_end(KK_SEG_PLAN, stream);
-    if (cudaPeekAtLastError() != cudaSuccess) return RS_ERR_CUDA;
+    if (planned != cudaSuccess) return RS_ERR_CUDA;
     st = launch_lists_wide(keys, vals, offsets, tiny_list, small_list, num_segments, ctrl, key_type,
                            PAIRS ? (uint32_t)sizeof(V) : 0u, stream);
     if (st != RS_OK) return st;

@@ -1,5 +1,7 @@
 // rs_sort.cu -- histogram and plan kernels, workspace layout and the
 // enqueue sequence of one unsegmented sort.
+#include <algorithm>
+
 #include "rs_internal.h"
 #include "rs_hist_plan.cuh"
 
@@ -43,9 +45,12 @@ Layout layout_for(size_t n, bool pairs) {
     return L;
 }
 
-rs_status enqueue_clear(Ctrl* ctrl, cudaStream_t stream) {
+rs_status enqueue_clear(Ctrl* ctrl, cudaStream_t stream, void* more, size_t more_bytes) {
+    const size_t vecs = more_bytes / sizeof(uint4);
+    const uint32_t grid = (uint32_t)std::min<size_t>(1 + vecs / 8192, 512);
     note_launch_begin(KK_CLEAR, stream);
-    k_clear_ctrl<<<1, 1024, 0, stream>>>(reinterpret_cast<uint4*>(ctrl));
+    k_clear_ctrl<<<grid, 1024, 0, stream>>>(reinterpret_cast<uint4*>(ctrl),
+                                            static_cast<uint4*>(more), vecs);
     note_launch_end(KK_CLEAR, stream);
     return cudaPeekAtLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
