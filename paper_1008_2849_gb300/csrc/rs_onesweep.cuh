@@ -205,8 +205,9 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
         }
         if (tile0 >= num_tiles) return;
     }
-    // The MSD-first order's only pass is the first and the last.
-    const bool only_pass = slot == MSD_SLOT;
+    // The MSD-first order's only pass is the first and the last.  (Whole arrays skip every
+    // other one then, so the plan says so itself.)
+    const bool only_pass = SEG && slot == MSD_SLOT;
     if (key_type & (ROLE_PLAIN_PASSES | ROLE_MAP_PASSES)) {
         // One of the two instances of a typed sort's pass: keep the pass if
         // it is this instance's (an executed first or last pass needs the
