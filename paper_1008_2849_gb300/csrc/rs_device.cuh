@@ -152,6 +152,19 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// Grid-stride loop over [0, n): calls f(i, left) for i = first, first + stride, ...,
+// left = n - i > 0 being the items from i on.  It ends by what is left, as i + stride
+// may not fit 32 bits (arrays hold up to 2^32 - 1 items).
+template <typename F>
+__host__ __device__ __forceinline__ void strided(uint32_t first, uint32_t stride, uint32_t n,
+                                                 F&& f) {
+    for (uint32_t i = first; i < n; i += stride) {
+        const uint32_t left = n - i;
+        f(i, left);
+        if (left <= stride) break;
+    }
+}
+
 // Streaming load: the data is read exactly once per pass, so ask for it to be
 // evicted first and not to displace the lines where scattered writes merge.
 __device__ __forceinline__ uint32_t ld_stream(const uint32_t* p) { return __ldcs(p); }

@@ -508,14 +508,14 @@ k_hist8(const unsigned long long* __restrict__ keys, uint32_t n, uint32_t* __res
     __syncthreads();
     uint32_t* const mycol = s_col + tid % COLS;
     constexpr uint32_t LOADS = 4;  // in flight per thread
-    for (uint32_t i = gtid; i < n; i += LOADS * gsize) {
+    strided(gtid, LOADS * gsize, n, [&](uint32_t i, uint32_t left) {
         unsigned long long v[LOADS];
 #pragma unroll
         for (uint32_t u = 0; u < LOADS; ++u)
-            v[u] = (size_t)i + u * gsize < n ? __ldcs(keys + i + u * gsize) : 0ull;
+            v[u] = u * gsize < left ? __ldcs(keys + i + u * gsize) : 0ull;
 #pragma unroll
         for (uint32_t u = 0; u < LOADS; ++u) {
-            if ((size_t)i + u * gsize < n) {
+            if (u * gsize < left) {
                 unsigned long long k = v[u];
                 if (TYPED) k = key_to_ordered(k, key_type);
                 const uint32_t lo = (uint32_t)k, hi = (uint32_t)(k >> 32);
@@ -527,7 +527,7 @@ k_hist8(const unsigned long long* __restrict__ keys, uint32_t n, uint32_t* __res
                 }
             }
         }
-    }
+    });
     __syncthreads();
     pdl_wait();  // the counts are zero
     for (uint32_t bin = tid; bin < PASSES64 * RADIX; bin += THREADS) {

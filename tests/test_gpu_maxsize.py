@@ -116,3 +116,41 @@ def test_digits11_keys_max_size(rs):
     assert _sums(torch, k) == s_in
     del k
     torch.cuda.empty_cache()
+
+
+def test_key64_max_size(rs):
+    """2^32 - 1 64-bit keys: the histogram's index runs up to its limit, the order is
+    that of eight passes with 64-bit look-back words."""
+    import torch
+    need = 16 * N + (8 << 30) + (16 << 30)  # keys, workspace, and room for the checks
+    if torch.cuda.mem_get_info()[0] < need:
+        pytest.skip("the GPU holds fewer free bytes than the arrays take")
+    k = torch.empty(N, dtype=torch.int64, device="cuda")
+    words = k.view(torch.int32)
+    for c in range(0, 2 * N, CHUNK):
+        m = min(CHUNK, 2 * N - c)
+        inputs.splitmix32_torch(303, m, 0, start=c, out=words[c:c + m])
+
+    def sums():
+        s1 = torch.zeros((), dtype=torch.int64, device="cuda")
+        s2 = torch.zeros((), dtype=torch.int64, device="cuda")
+        for c in range(0, N, CHUNK):
+            u = k[c:c + CHUNK]
+            s1 += u.sum()
+            s2 += (u * u).sum()        # both wrap modulo 2^64
+        return int(s1), int(s2)
+
+    s_in = sums()
+    nbytes = rs.workspace_bytes_kv(N, "u64", 0)
+    raw = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
+    pad = -raw.data_ptr() % 256
+    rs.sort_kv_ex(k, None, "u64", raw[pad:pad + nbytes])
+    rs.check_stream()
+    del raw
+    for c in range(0, N, CHUNK):
+        u = k[c:c + CHUNK + 1] ^ -(1 << 63)   # unsigned order as a signed one
+        assert bool((u[1:] >= u[:-1]).all()), c
+        del u
+    assert sums() == s_in
+    del k, words
+    torch.cuda.empty_cache()
