@@ -46,9 +46,8 @@ __device__ __forceinline__ void list_small(Ctrl* ctrl, uint32_t s, uint32_t size
 }
 
 // Shared-memory plan of k_bin_sort: bin words (or the counters of the digit
-// passes), binned words with room for the last windows' padding, keys (unless words
-// hold them whole) and values in input order, and the list of bins that the windows
-// do not cover.
+// passes), binned words with room for the last windows' padding, and keys (unless words
+// hold them whole) and values in input order.
 template <typename K, typename V, bool PAIRS, int THREADS, bool CHUNKS>
 struct BinSortSmem {
     static constexpr uint32_t ITEMS = 8;  // a thread's items, and the width of a window
@@ -61,13 +60,15 @@ struct BinSortSmem {
     static constexpr uint32_t SCANNERS = THREADS >= 1024 ? 1024 : THREADS >= 512 ? 512
                                          : THREADS >= 256 ? 256
                                          : THREADS >= 128 ? 128 : 64;
+    static constexpr uint32_t PER = MAX_BINS / SCANNERS;  // bins that a thread scans
+    static_assert(PER == 4 || PER == 8 || PER == 16, "whole groups of four, swizzled");
     static constexpr uint32_t COUNTERS = (THREADS / 32) * RADIX * 4;
     static constexpr uint32_t BINS = MAX_BINS * 4 > COUNTERS ? MAX_BINS * 4 : COUNTERS;
     static constexpr uint32_t WORDS = (CAP + 2 * ITEMS) * (uint32_t)sizeof(K);
     static constexpr uint32_t KEYS = PAIRS && !CHUNKS ? CAP * (uint32_t)sizeof(K) : 0;
     static constexpr uint32_t VALS = PAIRS ? CAP * (uint32_t)sizeof(V) : 0;
-    static constexpr uint32_t BIG = (CAP / 6 + 1) * 4;
-    static constexpr size_t BYTES = BINS + WORDS + KEYS + VALS + BIG;
+    static constexpr uint32_t NEED = (THREADS + 1) * 4;
+    static constexpr size_t BYTES = BINS + WORDS + KEYS + VALS + NEED;
     static_assert(BINS % 16 == 0 && WORDS % 16 == 0 && VALS % 16 == 0, "aligned parts");
 };
 
@@ -133,6 +134,53 @@ __device__ __forceinline__ void sort_window(W* p) {
     else sort8(u.w);
 #pragma unroll
     for (int i = 0; i < VECS; ++i) reinterpret_cast<uint4*>(p)[i] = u.v[i];
+}
+
+// Puts the words of the window at p (its first `left` ones) that agree but for the index
+// in their `ib` lowest bits in the order of keys[index], then index.  Returns whether
+// any moved.
+template <typename W>
+__device__ __forceinline__ bool order_ties(W* p, const W* keys, uint32_t ib, uint32_t imask,
+                                           int left) {
+    constexpr int VECS = 8 * sizeof(W) / 16;
+    union {
+        uint4 v[VECS];
+        W w[8];
+    } u;
+#pragma unroll
+    for (int i = 0; i < VECS; ++i) u.v[i] = reinterpret_cast<const uint4*>(p)[i];
+    bool again = false, changed = false;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) again |= i + 1 < left && (u.w[i] ^ u.w[i + 1]) >> ib == 0;
+    if (!again) return false;
+    constexpr bool CACHED = sizeof(W) == 4;  // the keys fit the registers too
+    W key[CACHED ? 8 : 1];
+    if constexpr (CACHED) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) key[i] = i < left ? keys[(uint32_t)u.w[i] & imask] : W(0);
+    }
+#pragma unroll 1
+    while (again) {
+        again = false;
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+            const W a = u.w[i], b = u.w[i + 1];
+            if (i + 1 < left && (a ^ b) >> ib == 0) {
+                const W ka = CACHED ? key[CACHED ? i : 0] : keys[(uint32_t)a & imask];
+                const W kb = CACHED ? key[CACHED ? i + 1 : 0] : keys[(uint32_t)b & imask];
+                if (kb < ka || (kb == ka && b < a)) {
+                    u.w[i] = b, u.w[i + 1] = a;
+                    if constexpr (CACHED) key[i] = kb, key[i + 1] = ka;
+                    again = changed = true;
+                }
+            }
+        }
+    }
+    if (changed) {
+#pragma unroll
+        for (int i = 0; i < VECS; ++i) reinterpret_cast<uint4*>(p)[i] = u.v[i];
+    }
+    return changed;
 }
 
 // ---------------------------------------------------------------------------
@@ -247,59 +295,54 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, b
 //     are in the stable order of its items.
 //  3. The words are sorted up to the order inside bins, of about one item each.
 //     Every thread sorts the window of eight words [8t, 8t + 8) in registers, then
-//     [8t + 4, 8t + 12): every bin of at most five lies within one of them.
-//     Longer bins are listed in step 2 and sorted before, one warp per bin, by
-//     counting the smaller words.
+//     [8t + 4, 8t + 12), and so on in turns: blocks of four words in an odd-even
+//     merge, of which r rounds sort every bin that lies in r blocks.  Two or three
+//     rounds of all sort most bins; a longer one asks for more of the windows over it
+//     (s_need).
 //  4. Words leave in order, as keys, with the values their indices point to.
-// Arrays whose keys crowd into few bins (the work of the listed bins is known
-// after step 2; the line is at one comparison by a warp for each item, and at
-// WARP_BIN_MAX items in a bin) take one
-// stable counting pass per 8-bit digit that differs instead: ranks from ballots
-// and per-warp counters, items exchanged through shared memory.
+// Bins too long for that hold one key each (`alike`): then the bins alone are the
+// order, and the index of an item inside its bin (two counting passes over (first
+// position, index), none without values).  Or keys crowd: arrays then take one stable
+// counting pass per 8-bit digit that differs, ranks from ballots and per-warp counters,
+// items exchanged through shared memory.  An array of one key keeps its order.
 //
 // The word has the width of the key: the key itself without values; else the key's
 // distance from the smallest, moved up until the largest has its highest bit set, with
 // the index in the lowest bits.  In chunks, whose keys share as many bits as an index
-// takes, that is the whole distance.  Elsewhere its lowest bits may be lost: words that differ in their index only are put in order by their
-// keys in step 4 (for 4096 keys that spread evenly, eight such pairs).
+// takes, that is the whole distance.  Elsewhere its lowest bits may be lost: words that
+// differ in their index only are put in order by their keys, in step 4 where they are
+// few (for 4096 keys that spread evenly, eight such pairs; a recount of the group by
+// each of its items), or by windows in registers (order_ties).
 //
 // What bounds it: instruction issue (135 warp instructions per 32 pairs, 61 % of the
 // issue slots) and shared-memory wavefronts (28 per 32 pairs: counting atomic, bin
 // read, word write and value read at random conflicts, 3.3 each; windows 4, bins 3;
 // the pipe is 60 % busy), where four digit passes take over 100; seven barriers are
-// hidden by the other CTA on the SM.  Ranking every item by a loop over its bin
+// hidden by the other CTA on the SM.  Digit passes take about 130 warp instructions
+// each per 32 items (61 % of the issue slots).  Ranking every item by a loop over its bin
 // instead of the windows took 194 instructions, most of them in diverged loops.
+// Long bins sorted by a warp each instead of by rounds of windows: 1024 segments of
+// 4096 to 2^20 pairs (194 M), each key four times, 6.86 ms, now 4.07; 16 times 6.98,
+// 4.30 (four scatter passes: 4.47); 2^25 keys four times each 1257 us, 513.
 // Measured: chunks of 2^28 pairs 1.51 ms (2.12 by loops), of 2^28 keys 1.24; the
 // 8,900 arrays of 513 to 4096 pairs among 2^15 short ones 1366 us in digit passes by
 // 512-thread CTAs, 170 now; one array of 1000 keys 20.4 us against 6.6.
 // ---------------------------------------------------------------------------
-constexpr uint32_t WINDOW_BIN_MAX = 5;  // the longest bin that the windows sort
-constexpr uint32_t WARP_BIN_MAX = 128;  // the longest bin that a warp sorts
-
-// One warp sorts the c <= WARP_BIN_MAX words of a bin: every word goes to the
-// number of words below it (TIES: equal ones in their present order).
-template <typename W, bool TIES>
-__device__ __forceinline__ void sort_bin(W* bin, uint32_t c, uint32_t lane) {
-    constexpr uint32_t R = WARP_BIN_MAX / 32;
-    W w[R];
-    uint32_t pos[R];
-#pragma unroll
-    for (uint32_t r = 0; r < R; ++r) {
-        w[r] = bin[r * 32 + lane < c ? r * 32 + lane : 0];
-        pos[r] = 0;
-    }
-    for (uint32_t q = 0; q < c; ++q) {
-        const W o = bin[q];
-#pragma unroll
-        for (uint32_t r = 0; r < R; ++r)
-            if (r * 32 < c)
-                pos[r] += o < w[r] || (TIES && o == w[r] && q < r * 32 + lane) ? 1u : 0u;
-    }
-    __syncwarp();
-#pragma unroll
-    for (uint32_t r = 0; r < R; ++r)
-        if (r * 32 + lane < c) bin[pos[r]] = w[r];
-}
+// The most rounds of windows, of which r sort bins of up to 4r - 3 words, and from how
+// many on it is looked whether every bin holds one key.  Where 32-bit words lose bits of
+// their keys, bins that long often need those put right too.  4096 segments of 256 to
+// 65536 pairs with 12, 24, 32 and 48 rounds at most: 64 equal keys each 1626, 1550, 1489
+// and 1371 us; ANDs of three words -, 1565, 1605 and 1758.
+template <typename K, bool PAIRS, int THREADS, bool CHUNKS> struct Rounds {
+    static constexpr bool LOSSY = sizeof(K) == 4 && PAIRS && !CHUNKS;
+    static constexpr uint32_t MOST = !LOSSY ? 48 : THREADS <= 64 ? 12 : 24;
+    static constexpr uint32_t LOOK = sizeof(K) == 4 && PAIRS ? MOST : 12;
+    // That every window takes: a third of 32-bit words costs less than to find out which
+    // windows need it (2^28 pairs 4.80 and 4.87 ms a call), of 64-bit words more (2^26:
+    // 2.17 and 2.10).
+    static constexpr uint32_t ALL = sizeof(K) == 4 ? 3 : 2;
+};
+constexpr uint32_t FEW_ROUNDS = 3;  // up to which step 4 puts lost bits right
 
 template <typename K, typename V, bool PAIRS, int THREADS, int MIN_BLOCKS,
           bool CHUNKS = false>
@@ -311,6 +354,7 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
     using L = BinSortSmem<K, V, PAIRS, THREADS, CHUNKS>;
     constexpr bool WHOLE = !PAIRS || CHUNKS;            // words hold whole keys
     constexpr bool BY_PREFIX = CHUNKS && sizeof(K) == 4;  // 32-bit chunks all are
+    using R = Rounds<K, PAIRS, THREADS, CHUNKS>;
     constexpr int ITEMS = L::ITEMS;
     constexpr uint32_t WARPS = THREADS / 32;
     constexpr uint32_t SCANNERS = L::SCANNERS;
@@ -323,11 +367,9 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
     K* const s_w = reinterpret_cast<K*>(parts);
     K* const s_k = reinterpret_cast<K*>(parts + L::WORDS);
     V* const s_v = reinterpret_cast<V*>(parts + L::WORDS + L::KEYS);
-    uint32_t* const s_big =
-        reinterpret_cast<uint32_t*>(parts + L::WORDS + L::KEYS + L::VALS);
+    uint32_t* const s_need = reinterpret_cast<uint32_t*>(parts + L::WORDS + L::KEYS + L::VALS);
     __shared__ K s_min, s_max;
-    __shared__ uint32_t s_sum[32], s_work[32];
-    __shared__ uint32_t s_bigs;
+    __shared__ uint32_t s_sum[32], s_longest[32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     uint32_t count = 1;
@@ -341,7 +383,7 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         if (ctrl->chunk_src != 0) src_keys = spare_keys, src_vals = spare_vals;
     }
     const bool typed = key_type != KEY_U32 && key_type != KEY_U64;
-    if (tid == 0) s_min = ~K(0), s_max = 0, s_bigs = 0;
+    if (tid == 0) s_min = ~K(0), s_max = 0;
     for (uint32_t idx = blockIdx.x; idx < count; idx += gridDim.x) {
         uint32_t lo = 0, m = single_n;
         if (off != nullptr) {
@@ -377,8 +419,11 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         const uint32_t bb = CHUNKS && bits > L::BIN_BITS ? L::BIN_BITS : bits;
         const uint32_t ib = PAIRS ? bits : 0u;
         const uint32_t nb = 1u << bb;
-        for (uint32_t b = tid; b < (nb + 3) / 4; b += THREADS)
+        const uint32_t zeroed = (nb > L::PER ? nb : L::PER) / 4;
+        for (uint32_t b = tid; b < zeroed; b += THREADS)
             reinterpret_cast<uint4*>(s_bin)[b] = make_uint4(0, 0, 0, 0);
+        s_need[tid] = 0;
+        if (tid == 0) s_need[THREADS] = 0;
         if (typed) {
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) k[j] = key_to_ordered(k[j], key_type);
@@ -413,6 +458,17 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
             __syncthreads();
             least = s_min;
             most = s_max;
+            if (least == most) {  // one key: the items stay in their order
+                __syncthreads();  // all have read it
+                if (tid == 0) s_min = ~K(0), s_max = 0;  // for the next array
+                if (src_keys == keys) continue;
+#pragma unroll 1
+                for (uint32_t i = tid; i < m; i += THREADS) {
+                    keys[lo + i] = from[i];
+                    if (PAIRS) vals[lo + i] = src_vals[lo + i];
+                }
+                continue;
+            }
         }
         const K range = (most - least) | 1;
         if (PAIRS) {
@@ -429,16 +485,14 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         if constexpr (!BY_PREFIX)
             scale = (uint32_t)(__fdividef((float)nb * 4294967296.0f,
                                           (float)high_word((K)(range << top))) * 0.999999f);
-        // Scanning thread t scans the `per` consecutive bins from t * per on,
-        // four at a time; their groups of four are swizzled so that the eight
-        // lanes of a 16-byte access fall into 32 different banks.
-        const uint32_t per = nb > SCANNERS ? nb / SCANNERS : 1u;  // 1, 2, 4, 8 or 16
-        const uint32_t swizzle = per > 4 ? (per / 4 - 1) << 2 : 0u;
+        // Scanning thread t scans the PER consecutive bins from t * PER on, four at a
+        // time; their groups of four are swizzled so that the eight lanes of a 16-byte
+        // access fall into 32 different banks.
+        constexpr uint32_t PER = L::PER, SWIZZLE = (PER / 4 - 1) << 2;
+        auto swizzled = [](uint32_t b) { return b ^ ((b >> 3) & SWIZZLE); };
         auto bin_of = [&](K x) {
-            const uint32_t b = BY_PREFIX
-                                   ? high_word((K)(x << top)) >> (32 - bb)
-                                   : __umulhi(high_word((K)((x - least) << top)), scale);
-            return b ^ ((b >> 3) & swizzle);
+            return swizzled(BY_PREFIX ? high_word((K)(x << top)) >> (32 - bb)
+                                      : __umulhi(high_word((K)((x - least) << top)), scale));
         };
 
         // ---- 1. count, keeping each item's place among its bin's items ------
@@ -449,37 +503,24 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
         __syncthreads();
 
         // ---- 2. exclusive prefix over the bins ------------------------------
-        // Bins become first positions.  Returns the work of the long bins, which
-        // are listed as (first position, count << 16).
-        auto scan_bins = [&](auto per_) {
-            constexpr uint32_t PER = decltype(per_)::value;
+        // Bins become first positions; `longest` is the longest bin's length.
+        uint32_t longest = 0;
+        {
             const bool scans = tid < SCANNERS && tid * PER < nb;
             uint32_t c[PER];
-            uint32_t sum = 0, work = 0;
-            constexpr uint32_t VECS = PER >= 4 ? PER / 4 : 1;
+            uint32_t sum = 0;
+            constexpr uint32_t VECS = PER / 4;
             uint4* const vec = reinterpret_cast<uint4*>(s_bin) + tid * VECS;
             const uint32_t turn = (tid * PER >> 5) & (VECS - 1);  // the swizzle of its groups
-            if constexpr (PER >= 4) {
 #pragma unroll
-                for (uint32_t g = 0; g < VECS; ++g) {
-                    const uint4 x = scans ? vec[g ^ turn] : make_uint4(0, 0, 0, 0);
-                    c[4 * g] = x.x, c[4 * g + 1] = x.y, c[4 * g + 2] = x.z, c[4 * g + 3] = x.w;
-                }
-            } else {
-#pragma unroll
-                for (uint32_t q = 0; q < PER; ++q) c[q] = scans ? s_bin[tid * PER + q] : 0u;
+            for (uint32_t g = 0; g < VECS; ++g) {
+                const uint4 x = scans ? vec[g ^ turn] : make_uint4(0, 0, 0, 0);
+                c[4 * g] = x.x, c[4 * g + 1] = x.y, c[4 * g + 2] = x.z, c[4 * g + 3] = x.w;
             }
-            uint32_t longest = 0;
 #pragma unroll
             for (uint32_t q = 0; q < PER; ++q) {
                 sum += c[q];
                 longest = max(longest, c[q]);
-            }
-            if (longest > WINDOW_BIN_MAX) {
-#pragma unroll
-                for (uint32_t q = 0; q < PER; ++q)
-                    if (c[q] > WINDOW_BIN_MAX)
-                        work += c[q] <= WARP_BIN_MAX ? (c[q] + 31) / 32 * c[q] : L::CAP + 1;
             }
             uint32_t x = sum;
 #pragma unroll
@@ -487,57 +528,50 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
                 if (lane >= o) x += y;
             }
-            const uint32_t warp_work = __reduce_add_sync(0xffffffffu, work);
+            longest = __reduce_max_sync(0xffffffffu, longest);
             if (lane == 31) {
                 s_sum[warp] = x;
-                s_work[warp] = warp_work;
+                s_longest[warp] = longest;
             }
             __syncthreads();
             const uint32_t before = lane < warp ? s_sum[lane] : 0u;
-            const uint32_t all = lane < WARPS ? s_work[lane] : 0u;
+            longest = __reduce_max_sync(0xffffffffu, lane < WARPS ? s_longest[lane] : 0u);
             uint32_t run = __reduce_add_sync(0xffffffffu, before) + x - sum;
-            if (longest > WINDOW_BIN_MAX) {
-                uint32_t at_bin = run;
-#pragma unroll
-                for (uint32_t q = 0; q < PER; ++q) {
-                    if (c[q] > WINDOW_BIN_MAX)
-                        s_big[atomicAdd(&s_bigs, 1u)] = at_bin | (c[q] << 16);
-                    at_bin += c[q];
-                }
-            }
 #pragma unroll
             for (uint32_t q = 0; q < PER; ++q) {
                 const uint32_t e = run;
                 run += c[q];
                 c[q] = e;
             }
-            if constexpr (PER >= 4) {
 #pragma unroll
-                for (uint32_t g = 0; g < VECS; ++g)
-                    if (scans) vec[g ^ turn] = make_uint4(c[4 * g], c[4 * g + 1], c[4 * g + 2],
-                                                          c[4 * g + 3]);
-            } else {
-#pragma unroll
-                for (uint32_t q = 0; q < PER; ++q)
-                    if (scans) s_bin[tid * PER + q] = c[q];
-            }
-            return __reduce_add_sync(0xffffffffu, all);
-        };
-        uint32_t work;
-        constexpr uint32_t MAX_PER = L::MAX_BINS / SCANNERS;
-        static_assert(MAX_PER >= 4 && MAX_PER <= 16, "see the dispatch below");
-        if (per == 1) work = scan_bins(std::integral_constant<uint32_t, 1>{});
-        else if (per == 2) work = scan_bins(std::integral_constant<uint32_t, 2>{});
-        else if (per == 4 || MAX_PER == 4) work = scan_bins(std::integral_constant<uint32_t, 4>{});
-        else if (per == 8 || MAX_PER == 8) work = scan_bins(std::integral_constant<uint32_t, 8>{});
-        else work = scan_bins(std::integral_constant<uint32_t, MAX_PER>{});
+            for (uint32_t g = 0; g < VECS; ++g)
+                if (scans)
+                    vec[g ^ turn] = make_uint4(c[4 * g], c[4 * g + 1], c[4 * g + 2], c[4 * g + 3]);
+        }
         if (tid == 0) s_min = ~K(0), s_max = 0;  // for the next array
         __syncthreads();
-        const uint32_t bigs = s_bigs;
 
+        // Windows of words, in as many rounds as the longest bin takes; or where it is too
+        // long for that, and every bin holds one key (`alike`), none for keys only.
         // (Chunks whose words would not hold whole keys take the digit passes too: none
         // by prefix; by position, where the keys are sparse.)
-        if (work <= m && (!CHUNKS || ib <= top)) {
+        uint32_t rounds = (longest + 6) / 4;
+        bool windowed = !CHUNKS || ib <= top, alike = false;
+        if (rounds > R::LOOK) {
+            K* const first_of = s_w;  // a key of every bin, at the bin's first position
+#pragma unroll
+            for (int j = 0; j < ITEMS; ++j)
+                if (tid + j * THREADS < m) first_of[s_bin[bin_of(k[j])]] = k[j];
+            __syncthreads();
+            bool same = true;
+#pragma unroll
+            for (int j = 0; j < ITEMS; ++j)
+                if (tid + j * THREADS < m) same &= first_of[s_bin[bin_of(k[j])]] == k[j];
+            alike = __syncthreads_and(same);
+            if (alike || rounds > R::MOST) windowed = alike && !PAIRS;
+            if (alike) rounds = 0;
+        }
+        if (windowed) {
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
                 if (tid + j * THREADS < m) {
@@ -550,56 +584,93 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 }
             // Padding above every word, to the end of the last window.
             const uint32_t windows = (m + 7) / 8;
+            const uint32_t imask = (1u << bits) - 1;
             if (tid < 8 * windows + 8 - m) s_w[m + tid] = ~K(0);
             __syncthreads();
             // ---- 3. the order inside bins ----------------------------------
-            if (bigs != 0) {
-                for (uint32_t g = warp; g < bigs; g += WARPS) {
-                    sort_bin<K, !PAIRS>(s_w + (s_big[g] & 0xffffu), s_big[g] >> 16, lane);
+            if (rounds != 0) {
+                if (rounds > R::ALL && tid < SCANNERS && tid * PER < nb) {
+                    // The rounds that the windows over the longer bins take.
+                    uint32_t first = s_bin[swizzled(tid * PER)];
+#pragma unroll 1
+                    for (uint32_t b = tid * PER + 1; b <= tid * PER + PER; ++b) {
+                        const uint32_t end = b < nb ? s_bin[swizzled(b)] : m;
+                        if (end - first > 4 * R::ALL - 3)
+#pragma unroll 1
+                            for (uint32_t w = first / 8; w * 8 < end; ++w)
+                                atomicMax(&s_need[w], (end - first + 6) / 4);
+                        first = end;
+                    }
                 }
-                if (tid == 0) s_bigs = 0;  // for the next array (read above, before a barrier)
-                __syncthreads();
+                if (tid < windows) sort_window<false>(s_w + 8 * tid);
+#pragma unroll 1
+                for (uint32_t r = 1; r < rounds; ++r) {
+                    __syncthreads();
+                    if (tid < windows &&
+                        (r < R::ALL || r < s_need[tid] || ((r & 1) && r < s_need[tid + 1])))
+                        sort_window<true>(s_w + 8 * tid + 4 * (r & 1));
+                }
+                if constexpr (!WHOLE) {
+                    // Words next to each other may differ in their index only because the
+                    // key's last bits did not fit: those are put in order by their keys,
+                    // until no window of either row has changed.  (Few of them: in step 4.)
+                    uint32_t done = rounds > FEW_ROUNDS ? 0 : 2;
+#pragma unroll 1
+                    for (uint32_t r = 0; done < 2; ++r) {
+                        __syncthreads();
+                        const uint32_t at_ = 8 * tid + 4 * (r & 1);
+                        const bool changed =
+                            tid < windows &&
+                            order_ties(s_w + at_, s_k, ib, imask, (int)m - (int)at_);
+                        done = __syncthreads_or(changed) ? 0 : done + 1;
+                    }
+                }
             }
-            if (tid < windows) sort_window<false>(s_w + 8 * tid);
-            __syncthreads();
-            if (tid < windows) sort_window<true>(s_w + 8 * tid + 4);
             if (PAIRS) cp_async_wait_all();
             __syncthreads();
             // ---- 4. stored in order -----------------------------------------
-            const uint32_t imask = (1u << bits) - 1;
+            uint32_t tied = 0;  // items whose word differs from a neighbour's in the index only
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) {
-                uint32_t at_ = tid + j * THREADS;
+                const uint32_t at_ = tid + j * THREADS;
                 if (at_ < m) {
                     const K w = s_w[at_];
+                    if (!WHOLE && rounds <= FEW_ROUNDS &&
+                        ((at_ > 0 && (s_w[at_ - 1] ^ w) >> ib == 0) ||
+                         (at_ + 1 < m && (s_w[at_ + 1] ^ w) >> ib == 0))) {
+                        tied |= 1u << j;
+                        continue;
+                    }
                     const uint32_t i = (uint32_t)w & imask;
                     K key;
-                    if constexpr (WHOLE) {
-                        key = PAIRS ? (K)(w >> top) + least : w;
-                    } else {
-                        // Words next to each other may differ in their index only
-                        // because the key's last bits did not fit: those few
-                        // items find their places among each other by the keys.
-                        key = s_k[i];
-                        const K t = w >> ib;
-                        const bool below = at_ > 0 && s_w[at_ - 1] >> ib == t;
-                        const bool above = at_ + 1 < m && s_w[at_ + 1] >> ib == t;
-                        if (below || above) {
-                            uint32_t lo_ = at_, hi_ = at_ + 1;
-                            while (lo_ > 0 && s_w[lo_ - 1] >> ib == t) --lo_;
-                            while (hi_ < m && s_w[hi_] >> ib == t) ++hi_;
-                            at_ = lo_;
-                            for (uint32_t q = lo_; q < hi_; ++q) {
-                                const uint32_t o = (uint32_t)s_w[q] & imask;
-                                const K ok = s_k[o];
-                                at_ += ok < key || (ok == key && o < i) ? 1u : 0u;
-                            }
-                        }
-                    }
+                    if constexpr (WHOLE) key = PAIRS ? (K)(w >> top) + least : w;
+                    else key = s_k[i];
                     if (typed) key = key_from_ordered(key, key_type);
                     keys[lo + at_] = key;
                     if (PAIRS) vals[lo + at_] = s_v[i];
                 }
+            }
+            // Those find their places among each other by their keys.
+#pragma unroll 1
+            for (; !WHOLE && tied != 0; tied &= tied - 1) {
+                const uint32_t at_ = tid + (__ffs(tied) - 1) * THREADS;
+                const K w = s_w[at_];
+                const uint32_t i = (uint32_t)w & imask;
+                K key = s_k[i];
+                uint32_t to = at_, last = at_;
+#pragma unroll 1
+                while (to > 0 && (s_w[to - 1] ^ w) >> ib == 0) --to;
+#pragma unroll 1
+                while (last + 1 < m && (s_w[last + 1] ^ w) >> ib == 0) ++last;
+#pragma unroll 1
+                for (uint32_t q = to; q <= last; ++q) {
+                    const uint32_t o = (uint32_t)s_w[q] & imask;
+                    const K ok = s_k[o];
+                    to += ok < key || (ok == key && o < i) ? 1u : 0u;
+                }
+                if (typed) key = key_from_ordered(key, key_type);
+                keys[lo + to] = key;
+                if (PAIRS) vals[lo + to] = s_v[i];
             }
         } else {
             // ---- digit passes ------------------------------------------------
@@ -614,24 +685,32 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
             const uint32_t lt = lanemask_lt();
             uint32_t* const row = s_bin + warp * RADIX;
             V v[PAIRS ? ITEMS : 1];
+            // alike: words of the bin's first position above the item's index.
+            constexpr uint32_t INDEX_BITS = 13, INDEX_MASK = (1u << INDEX_BITS) - 1;
+            static_assert(L::CAP <= 1u << INDEX_BITS, "positions and indices fit");
+            const bool by_bin = PAIRS && alike;
             if (PAIRS) cp_async_wait_all();
             __syncthreads();
-            if (tid == 0) s_bigs = 0;  // for the next array
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) {
                 if (j < mine) {
                     k[j] = key_to_ordered(from[me + j * 32], key_type);
-                    if (PAIRS) v[j] = s_v[me + j * 32];
+                    if (by_bin) k[j] = (K)s_bin[bin_of(k[j])] << INDEX_BITS | (me + j * 32);
+                    else if (PAIRS) v[j] = s_v[me + j * 32];
                 }
             }
-            for (uint32_t p = 0; p < sizeof(K); ++p) {
-                if (least >> (8 * p) == most >> (8 * p)) break;  // the rest is the same in all
+            __syncthreads();  // the bins are read: counters take their place
+#pragma unroll 1
+            for (uint32_t shift = by_bin ? INDEX_BITS : 0;
+                 by_bin ? shift < INDEX_BITS + bits
+                        : shift < 8 * sizeof(K) && least >> shift != most >> shift;
+                 shift += RADIX_BITS) {
                 for (uint32_t b = lane; b < RADIX; b += 32) row[b] = 0;
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < ITEMS; ++j) {
                     if (j < ipt) {
-                        const uint32_t d = (uint32_t)(k[j] >> (8 * p)) & (RADIX - 1);
+                        const uint32_t d = (uint32_t)(k[j] >> shift) & (RADIX - 1);
                         const uint32_t live = prefix_lanes(me - lane + j * 32, m);
                         const uint32_t peers = match_label<RADIX_BITS>(d) & live;
                         const uint32_t lead = __ffs(peers) - 1;
@@ -644,13 +723,13 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 __syncthreads();
                 // Thread t turns the counts of its consecutive digits into
                 // every warp's first position of the digit.
-                constexpr uint32_t PER = RADIX > THREADS ? RADIX / THREADS : 1;
-                uint32_t c[PER], sum = 0;
+                constexpr uint32_t DIGITS = RADIX > THREADS ? RADIX / THREADS : 1;
+                uint32_t c[DIGITS], sum = 0;
                 bool trivial = false;
 #pragma unroll
-                for (uint32_t q = 0; q < PER; ++q) {
+                for (uint32_t q = 0; q < DIGITS; ++q) {
                     c[q] = 0;
-                    const uint32_t d = tid * PER + q;
+                    const uint32_t d = tid * DIGITS + q;
                     if (d < RADIX)
                         for (uint32_t w = 0; w < WARPS; ++w) c[q] += s_bin[w * RADIX + d];
                     trivial |= c[q] == m;
@@ -668,14 +747,21 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 const uint32_t before = lane < warp ? s_sum[lane] : 0u;
                 uint32_t run = __reduce_add_sync(0xffffffffu, before) + x - sum;
 #pragma unroll
-                for (uint32_t q = 0; q < PER; ++q) {
-                    const uint32_t d = tid * PER + q;
+                for (uint32_t q = 0; q < DIGITS; ++q) {
+                    const uint32_t d = tid * DIGITS + q;
                     if (d < RADIX) {
                         uint32_t r = run;
-                        for (uint32_t w = 0; w < WARPS; ++w) {
-                            const uint32_t t = s_bin[w * RADIX + d];
-                            s_bin[w * RADIX + d] = r;
-                            r += t;
+                        constexpr uint32_t BATCH = WARPS < 6 ? WARPS : 6;  // reads in flight
+                        for (uint32_t w0 = 0; w0 < WARPS; w0 += BATCH) {
+                            uint32_t t[BATCH];
+#pragma unroll
+                            for (uint32_t w = 0; w < BATCH; ++w)
+                                t[w] = w0 + w < WARPS ? s_bin[(w0 + w) * RADIX + d] : 0u;
+#pragma unroll
+                            for (uint32_t w = 0; w < BATCH; ++w) {
+                                if (w0 + w < WARPS) s_bin[(w0 + w) * RADIX + d] = r;
+                                r += t[w];
+                            }
                         }
                     }
                     run += c[q];
@@ -684,9 +770,9 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
 #pragma unroll
                 for (int j = 0; j < ITEMS; ++j) {
                     if (j < mine) {
-                        at[j] += row[(uint32_t)(k[j] >> (8 * p)) & (RADIX - 1)];
+                        at[j] += row[(uint32_t)(k[j] >> shift) & (RADIX - 1)];
                         s_w[at[j]] = k[j];
-                        if (PAIRS) s_v[at[j]] = v[j];
+                        if (PAIRS && !by_bin) s_v[at[j]] = v[j];
                     }
                 }
                 __syncthreads();
@@ -694,10 +780,21 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 for (int j = 0; j < ITEMS; ++j) {
                     if (j < mine) {
                         k[j] = s_w[me + j * 32];
-                        if (PAIRS) v[j] = s_v[me + j * 32];
+                        if (PAIRS && !by_bin) v[j] = s_v[me + j * 32];
                     }
                 }
                 __syncthreads();
+            }
+            if (by_bin) {
+#pragma unroll
+                for (int j = 0; j < ITEMS; ++j) {
+                    if (j < mine) {
+                        const uint32_t i = (uint32_t)k[j] & INDEX_MASK;
+                        k[j] = key_to_ordered(from[i], key_type);
+                        v[PAIRS ? j : 0] = s_v[i];
+                    }
+                }
+                __syncthreads();  // every key is read before any is stored
             }
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) {
