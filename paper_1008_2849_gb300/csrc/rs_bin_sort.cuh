@@ -67,7 +67,7 @@ struct BinSortSmem {
     static constexpr uint32_t WORDS = (CAP + 2 * ITEMS) * (uint32_t)sizeof(K);
     static constexpr uint32_t KEYS = PAIRS && !CHUNKS ? CAP * (uint32_t)sizeof(K) : 0;
     static constexpr uint32_t VALS = PAIRS ? CAP * (uint32_t)sizeof(V) : 0;
-    static constexpr uint32_t NEED = (THREADS + 1) * 4;
+    static constexpr uint32_t NEED = (THREADS + 1) * 4;  // a flag for each window
     static constexpr size_t BYTES = BINS + WORDS + KEYS + VALS + NEED;
     static_assert(BINS % 16 == 0 && WORDS % 16 == 0 && VALS % 16 == 0, "aligned parts");
 };
@@ -186,20 +186,24 @@ __device__ __forceinline__ bool order_ties(W* p, const W* keys, uint32_t ib, uin
 // ---------------------------------------------------------------------------
 // sort_in_global: one CTA sorts the m items at a (stable, in place) by counting
 // passes over the 8-bit digits that differ, between a and b of the same size,
-// through counters s_cnt[THREADS / 32][RADIX], s_base[RADIX] and s_hist[RADIX].  The
-// result is left in a, or with to_b in b.
+// through counters s_cnt[THREADS / 32][RADIX], s_base[RADIX] and s_hist[RADIX]; all ordered
+// keys lie in [least, most].  The result is left in a, or with to_b in b.
 // For the rare chunk that the top-digits order leaves too long for the chip:
-// about 1 item per ns, so it counts on there being few of them.
+// about 4 ns an item of 32 bits (one key in 0.1 % of 2^28 pairs adds 1 ms), so the plan
+// counts on there being few of them, and short ones.
 // ---------------------------------------------------------------------------
 template <typename K, typename V, bool PAIRS, int THREADS>
 __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, bool to_b,
-                                            uint32_t m, uint32_t key_type, uint32_t* s_cnt, uint32_t* s_base,
-                                            uint32_t* s_hist) {
+                                               uint32_t m, uint32_t key_type, K least, K most,
+                                               uint32_t* s_cnt, uint32_t* s_base,
+                                               uint32_t* s_hist) {
     constexpr uint32_t WARPS = THREADS / 32, SLOTS = 4, TILE = THREADS * SLOTS;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = lanemask_lt();
     bool in_a = true;
+#pragma unroll 1
     for (uint32_t p = 0; p < sizeof(K); ++p) {
+        if (least >> (8 * p) == most >> (8 * p)) break;  // the rest is the same in all
         const K* const sk = in_a ? a_k : b_k;
         const V* const sv = in_a ? a_v : b_v;
         K* const dk = in_a ? b_k : a_k;
@@ -297,8 +301,8 @@ __device__ __forceinline__ void sort_in_global(K* a_k, V* a_v, K* b_k, V* b_v, b
 //     Every thread sorts the window of eight words [8t, 8t + 8) in registers, then
 //     [8t + 4, 8t + 12), and so on in turns: blocks of four words in an odd-even
 //     merge, of which r rounds sort every bin that lies in r blocks.  Two or three
-//     rounds of all sort most bins; a longer one asks for more of the windows over it
-//     (s_need).
+//     rounds of all sort most bins; the windows over longer ones take as many as the
+//     longest needs (s_need).
 //  4. Words leave in order, as keys, with the values their indices point to.
 // Bins too long for that hold one key each (`alike`): then the bins alone are the
 // order, and the index of an item inside its bin (two counting passes over (first
@@ -337,9 +341,9 @@ template <typename K, bool PAIRS, int THREADS, bool CHUNKS> struct Rounds {
     static constexpr bool LOSSY = sizeof(K) == 4 && PAIRS && !CHUNKS;
     static constexpr uint32_t MOST = !LOSSY ? 48 : THREADS <= 64 ? 12 : 24;
     static constexpr uint32_t LOOK = sizeof(K) == 4 && PAIRS ? MOST : 12;
-    // That every window takes: a third of 32-bit words costs less than to find out which
-    // windows need it (2^28 pairs 4.80 and 4.87 ms a call), of 64-bit words more (2^26:
-    // 2.17 and 2.10).
+    // That every window takes.  A third round of all windows of 64-bit words costs more
+    // than to leave out those that do not need it (2^26 pairs 2.13 ms and 2.08), and of
+    // 32-bit words gains a little where keys repeat a few times.
     static constexpr uint32_t ALL = sizeof(K) == 4 ? 3 : 2;
 };
 constexpr uint32_t FEW_ROUNDS = 3;  // up to which step 4 puts lost bits right
@@ -401,10 +405,14 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                 if (m > L::CAP) {
                     __syncthreads();  // the array before is done with shared memory
                     const bool b = ctrl->chunk_src != 0;
+                    K* const a_k = (b ? spare_keys : keys) + lo;
+                    K* const b_k = (b ? keys : spare_keys) + lo;
                     sort_in_global<K, V, PAIRS, THREADS>(
-                        (b ? spare_keys : keys) + lo, PAIRS ? (b ? spare_vals : vals) + lo : nullptr,
-                        (b ? keys : spare_keys) + lo, PAIRS ? (b ? vals : spare_vals) + lo : nullptr,
-                        b, m, key_type, s_bin, reinterpret_cast<uint32_t*>(s_w),
+                        a_k, PAIRS ? (b ? spare_vals : vals) + lo : nullptr, b_k,
+                        PAIRS ? (b ? vals : spare_vals) + lo : nullptr, b, m, key_type,
+                        key_to_ordered(a_k[0], key_type) & sorted,
+                        key_to_ordered(a_k[m - 1], key_type) | ~sorted, s_bin,
+                        reinterpret_cast<uint32_t*>(s_w),
                         reinterpret_cast<uint32_t*>(s_w) + RADIX);
                     continue;
                 }
@@ -579,8 +587,15 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
                     K w = k[j];
                     if (PAIRS && CHUNKS) w = ((BY_PREFIX ? w : w - least) << top) | (K)i;
                     if (PAIRS && !CHUNKS) w = ((w - least) << top >> ib << ib) | (K)i;
-                    s_w[s_bin[bin_of(k[j])] + at[j]] = w;
+                    const uint32_t first = s_bin[bin_of(k[j])];
+                    s_w[first + at[j]] = w;
                     if (!WHOLE) s_k[i] = k[j];
+                    if (at[j] >= 4 * R::ALL - 3) {  // in a longer bin: its windows
+                        s_need[(first + at[j]) / 8] = 1;
+                        if (at[j] == 4 * R::ALL - 3)
+                            for (uint32_t x = first / 8; x < (first + at[j]) / 8; ++x)
+                                s_need[x] = 1;
+                    }
                 }
             // Padding above every word, to the end of the last window.
             const uint32_t windows = (m + 7) / 8;
@@ -589,25 +604,12 @@ k_bin_sort(K* keys, V* vals, const K* src_keys, const V* src_vals,
             __syncthreads();
             // ---- 3. the order inside bins ----------------------------------
             if (rounds != 0) {
-                if (rounds > R::ALL && tid < SCANNERS && tid * PER < nb) {
-                    // The rounds that the windows over the longer bins take.
-                    uint32_t first = s_bin[swizzled(tid * PER)];
-#pragma unroll 1
-                    for (uint32_t b = tid * PER + 1; b <= tid * PER + PER; ++b) {
-                        const uint32_t end = b < nb ? s_bin[swizzled(b)] : m;
-                        if (end - first > 4 * R::ALL - 3)
-#pragma unroll 1
-                            for (uint32_t w = first / 8; w * 8 < end; ++w)
-                                atomicMax(&s_need[w], (end - first + 6) / 4);
-                        first = end;
-                    }
-                }
                 if (tid < windows) sort_window<false>(s_w + 8 * tid);
 #pragma unroll 1
                 for (uint32_t r = 1; r < rounds; ++r) {
                     __syncthreads();
                     if (tid < windows &&
-                        (r < R::ALL || r < s_need[tid] || ((r & 1) && r < s_need[tid + 1])))
+                        (r < R::ALL || s_need[tid] != 0 || ((r & 1) && s_need[tid + 1] != 0)))
                         sort_window<true>(s_w + 8 * tid + 4 * (r & 1));
                 }
                 if constexpr (!WHOLE) {
