@@ -228,9 +228,14 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
 // its top 16 bits, and every chunk of keys with the same top_bits highest
 // bits (about n >> top_bits of them) is sorted on chip by the rest.  "Evenly":
 // no bucket of either digit holds over twice its share, at least three passes
-// would run otherwise, and of TOP_SAMPLES keys no chunk holds far more than its
-// share (the digits may be even one by one and not together).  Chunks that are
-// too long all the same are sorted in global memory by one CTA each, so a
+// would run otherwise, and in a sample of the keys (the digits may be even one by one
+// and not together)
+//  - no chunk holds far more than its share: one hot key;
+//  - the pairs of keys in one chunk are not far over those of even keys: few prefixes,
+//    whose chunks are long (2^27 pairs with 10,000 prefixes 7.48 ms instead of 2.88);
+//  - few keys are equal: chunks of repeated keys take the on-chip sorts longer (2^27 pairs
+//    with 100,000 distinct keys 5.92 ms instead of 2.92, with 16 million 2.83 and 2.90).
+// Chunks that are too long all the same are sorted in global memory by one CTA each, so a
 // sample that misses them costs time, not correctness.
 //
 // 64-bit keys that are not even may still take the passes by their two to four highest
@@ -238,9 +243,39 @@ k_hist4_cols(const uint32_t* __restrict__ keys, uint32_t n, uint32_t* __restrict
 // keys that these digits do not tell apart (normal doubles: three passes instead of
 // eight).  Their chunks are chunk_step items long, up to the next change of prefix.
 // ---------------------------------------------------------------------------
-constexpr uint32_t TOP_SAMPLES = 4096;
+constexpr uint32_t TOP_MAX_SAMPLES = 8192;
 constexpr uint32_t TOP_MAX_BITS = 16;
-constexpr size_t TOP_PLAN_SMEM = (size_t(1) << TOP_MAX_BITS) * sizeof(uint16_t);
+
+// Keys sampled: 8192 of 2^27 32-bit keys and more (repeated keys show by the sample's
+// square over n; 3 us of 2.4 ms), else 4096.
+__host__ __device__ constexpr uint32_t top_samples(uint32_t n, bool key64) {
+    return !key64 && n >= (1u << 27) ? TOP_MAX_SAMPLES : 4096u;
+}
+// Times that every key may occur before the passes by all digits are the faster ones: 6 to
+// 10 of 32-bit keys (2^25 to 2^27 of them, without or with values); of 64-bit keys 300 (2^22
+// pairs), 50 (2^25).
+__host__ __device__ constexpr uint32_t top_repeats(uint32_t n, bool key64) {
+    return !key64 ? 8u : n >= (1u << 24) ? 48u : 192u;
+}
+// The least number of repeated keys in the sample that tells of so many times.  (64-bit
+// arrays below 2^22 items are not looked at: it takes 5 us, and they gain 60.)
+__host__ __device__ constexpr uint32_t top_equal_limit(uint32_t n, bool key64) {
+    if (key64 && n < (1u << 22)) return ~0u;
+    const unsigned long long s = top_samples(n, key64);
+    const unsigned long long least = top_repeats(n, key64) * s * s / (2ull * n);
+    return least < 2 ? 2u : least < s ? (uint32_t)least : (uint32_t)s;
+}
+// Samples of one key that tell of a chunk too long for one CTA to gain by: 0.1 % of 32-bit
+// keys (2^25 pairs 879 us instead of 774 by all digits, with 0.05 % 773), 0.2 % of 64-bit.
+__host__ __device__ constexpr uint32_t top_hot_limit(bool key64, uint32_t samples) {
+    return samples / 4096 * (key64 ? 8 : 3);
+}
+// The most pairs of samples in one of 2^bits cells: four standard deviations over those of
+// even keys.
+__device__ __forceinline__ uint32_t top_pair_limit(uint32_t samples, uint32_t bits) {
+    const uint32_t even = (uint32_t)((unsigned long long)samples * samples / 2 >> bits);
+    return even + (uint32_t)(4.0f * sqrtf((float)even));
+}
 
 // What the plan works on; bucket_cap and msd_off for the MSD-first order
 // (msd_off == nullptr: not allowed), top_bits for the top-digits order.
@@ -252,9 +287,18 @@ struct PlanArgs {
     uint32_t top_bits, chunk_step;
 };
 
-// Dynamic shared memory when top_bits is set: 2 << top_bits bytes, and at least
-// 2 << TOP_HASH_BITS.
+// Dynamic shared memory of k_plan when top_bits is set: two bytes for each cell of the
+// 2^top_bits or 2^TOP_HASH_BITS, and where repeated keys are looked for at least a table of
+// twice the samples with five bytes a slot.
 constexpr uint32_t TOP_HASH_BITS = 13;
+constexpr size_t top_plan_smem(uint32_t n, uint32_t top_bits, bool key64) {
+    const size_t cells = sizeof(uint16_t) << (top_bits > TOP_HASH_BITS ? top_bits : TOP_HASH_BITS);
+    const size_t samples = top_samples(n, key64);
+    const size_t table = top_equal_limit(n, key64) < samples ? 5 * 2 * samples : 0;
+    return cells > table ? cells : table;
+}
+constexpr size_t TOP_PLAN_SMEM = sizeof(uint16_t) << TOP_MAX_BITS;
+static_assert(TOP_PLAN_SMEM >= 10 * TOP_MAX_SAMPLES, "the table too");
 template <int NPASS>
 __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     extern __shared__ uint4 s_dyn[];
@@ -263,6 +307,7 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_trivial[NPASS];
     __shared__ uint32_t s_big, s_uneven;
+    __shared__ uint32_t s_part[32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t b = tid & (RADIX - 1);
     Ctrl* const ctrl = plan.ctrl;
@@ -306,49 +351,110 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     if (top || deep) {  // the same for every thread
         uint32_t* const s_pair = reinterpret_cast<uint32_t*>(s_dyn);  // two 16-bit counts a word
         const K* const keys = static_cast<const K*>(plan.keys);
-        constexpr uint32_t PER = TOP_SAMPLES / 1024;
-        const uint32_t stride = n / TOP_SAMPLES;
+        constexpr uint32_t PER = NPASS == 4 ? TOP_MAX_SAMPLES / 1024 : 4;
+        const uint32_t samples = top_samples(n, NPASS == 8);
+        const uint32_t stride = n / samples;
         K k[PER];
 #pragma unroll
-        for (uint32_t q = 0; q < PER; ++q) {  // one key of each of TOP_SAMPLES parts
+        for (uint32_t q = 0; q < PER; ++q) {  // one key of each of `samples` parts
             const uint32_t i = q * 1024 + tid;
             uint32_t r = i * 0x9E3779B1u;
             r ^= r >> 15;
             r *= 0x85EBCA6Bu;
-            const uint32_t at = (uint32_t)(((uint64_t)i * n) / TOP_SAMPLES) + __umulhi(r, stride);
-            k[q] = key_to_ordered(keys[at], plan.key_type);
+            const uint32_t at = (uint32_t)(((uint64_t)i * n) / samples) + __umulhi(r, stride);
+            k[q] = i < samples ? key_to_ordered(keys[at], plan.key_type) : K(0);
         }
-        // Whether no cell of the 2^bits that `cell` tells apart holds over `most` keys.
-        auto spread = [&](uint32_t bits, uint32_t most, auto cell) -> bool {
+        // The sum of x over the threads (one barrier).
+        auto sum_of = [&](uint32_t x) -> uint32_t {
+            x = __reduce_add_sync(0xffffffffu, x);
+            if (lane == 0) s_part[warp] = x;
+            __syncthreads();
+            return __reduce_add_sync(0xffffffffu, s_part[lane]);
+        };
+        // Keys that occur more than once in the sample, by a table of it (of 64-bit keys, of
+        // 32 bits of their hashes), which holds all words but ~0.  One key that occurs
+        // top_hot_limit times sets s_uneven.
+        auto repeated_keys = [&]() -> uint32_t {
+            constexpr uint32_t EMPTY = ~0u;
+            const uint32_t slots = 2 * samples;  // a power of two
+            uint32_t* const slot = s_pair;
+            uint32_t* const again = s_pair + slots;  // a byte for each: its further samples
+#pragma unroll 1
+            for (uint32_t i = tid; i < slots * 5 / 16; i += 1024) {
+                const uint32_t v = i < slots / 4 ? EMPTY : 0u;
+                s_dyn[i] = make_uint4(v, v, v, v);
+            }
+            if (tid == 0) s_uneven = 0;
+            __syncthreads();
+            uint32_t found = 0;
+#pragma unroll
+            for (uint32_t q = 0; q < PER; ++q) {
+                const unsigned long long h = (unsigned long long)k[q] * 0x9E3779B97F4A7C15ull;
+                const uint32_t word = NPASS == 4 ? (uint32_t)k[q] : (uint32_t)(h >> 32);
+                if (q * 1024 + tid >= samples || word == EMPTY) continue;
+                uint32_t at = (uint32_t)(h >> 16) & (slots - 1);
+                uint32_t was = atomicCAS(&slot[at], EMPTY, word);
+#pragma unroll 1
+                while (was != EMPTY && was != word) {  // at most half of the slots are taken
+                    at = (at + 1) & (slots - 1);
+                    was = atomicCAS(&slot[at], EMPTY, word);
+                }
+                if (was != word) continue;
+                // (A byte that overflows has passed the limit.)
+                const uint32_t before =
+                    atomicAdd(&again[at / 4], 1u << 8 * (at % 4)) >> 8 * (at % 4) & 0xffu;
+                found += before == 0;
+                if (before + 2 >= top_hot_limit(NPASS == 8, samples)) s_uneven = 1;
+            }
+            return sum_of(found);
+        };
+        // Whether no cell of the 2^bits that `cell` tells apart holds over `most` keys,
+        // and all no more than `most_pairs` pairs of keys in one cell.
+        auto spread = [&](uint32_t bits, uint32_t most, uint32_t most_pairs, auto cell) -> bool {
             __syncthreads();
             if (tid == 0) s_uneven = 0;
             for (uint32_t i = tid; i < (1u << bits) / 8; i += 1024)
                 s_dyn[i] = make_uint4(0, 0, 0, 0);
             __syncthreads();
+            uint32_t pairs = 0;
 #pragma unroll
             for (uint32_t q = 0; q < PER; ++q) {
+                if (NPASS == 4 && q * 1024 + tid >= samples) continue;
                 const uint32_t c = cell(k[q]);
-                const uint32_t was = atomicAdd(&s_pair[c >> 1], 1u << (16 * (c & 1)));
-                if (((was >> (16 * (c & 1))) & 0xffffu) >= most) s_uneven = 1;
+                const uint32_t was =
+                    atomicAdd(&s_pair[c >> 1], 1u << (16 * (c & 1))) >> (16 * (c & 1)) & 0xffffu;
+                if (was >= most) s_uneven = 1;
+                pairs += was;
             }
-            __syncthreads();
-            return !s_uneven;
+            return sum_of(pairs) <= most_pairs && !s_uneven;
         };
+        const uint32_t equal = top_equal_limit(n, NPASS == 8);
+        // (32-bit keys with a digit that is the same in all are not looked at.)
+        bool repeat = false;
+        if (equal < samples && (NPASS == 8 || executed == NPASS)) {
+            __syncthreads();  // s_uneven was read
+            repeat = repeated_keys() >= equal || s_uneven;
+        }
         if (top) {
             low = NPASS - 2;
-            top = spread(top_bits, 2 * (TOP_SAMPLES >> top_bits) + 12,
-                         [&](K x) { return (uint32_t)(x >> (8 * sizeof(K) - top_bits)); });
+            top = !repeat && spread(top_bits, 2 * (samples >> top_bits) + 12,
+                                    top_pair_limit(samples, top_bits), [&](K x) {
+                                        return (uint32_t)(x >> (8 * sizeof(K) - top_bits));
+                                    });
         }
-        if (deep && !top) {
-            const uint32_t most =
-                (uint32_t)(2ull * TOP_SAMPLES * plan.chunk_step / n) + 10;
+        if (deep && !repeat && !top) {
+            const uint32_t most = (uint32_t)(2ull * samples * plan.chunk_step / n) + 10;
+            // Pairs by the hash alone, and those of prefixes of 3/4 of a CTA's items.
+            const uint32_t most_pairs =
+                top_pair_limit(samples, TOP_HASH_BITS) +
+                (uint32_t)((3ull * plan.chunk_step / 2) * samples / 2 * samples / n);
             uint32_t passes = 0;
             for (low = NPASS; !top && low-- > 0;) {
                 if (s_trivial[low]) continue;
                 ++passes;
                 if (passes > 4 || passes + 2 > executed) break;
                 if (passes < 2) continue;
-                top = spread(TOP_HASH_BITS, most, [&](K x) {
+                top = spread(TOP_HASH_BITS, most, most_pairs, [&](K x) {
                     const unsigned long long h =
                         (unsigned long long)(x >> (8 * low)) * 0x9E3779B97F4A7C15ull;
                     return (uint32_t)(h >> (64 - TOP_HASH_BITS));

@@ -114,11 +114,11 @@ rs_status enqueue_plan(const PlanArgs& plan, cudaStream_t stream) {
     static DeviceOnce smem_set;
     const rs_status st = allow_smem_once(k_plan<NPASS>, TOP_PLAN_SMEM, smem_set);
     if (st != RS_OK) return st;
-    const uint32_t bits = plan.top_bits > TOP_HASH_BITS ? plan.top_bits : TOP_HASH_BITS;
+    const size_t smem =
+        plan.top_bits ? top_plan_smem(plan.n, plan.top_bits, NPASS == PASSES64) : 0;
     note_launch_begin(KK_PLAN, stream);
     const cudaError_t e =
-        launch_after_previous(k_plan<NPASS>, dim3(1), dim3(1024),
-                              plan.top_bits ? sizeof(uint16_t) << bits : 0, stream, plan);
+        launch_after_previous(k_plan<NPASS>, dim3(1), dim3(1024), smem, stream, plan);
     note_launch_end(KK_PLAN, stream);
     return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }

@@ -1,0 +1,136 @@
+"""GPU tests of which order the plan chooses, read from the control block at the start of
+the workspace, beside the results against the CPU oracle: keys that repeat or share few
+prefixes take the passes by all digits, as does an array with one hot key; wide items and
+large segments take the orders that their other tests mean to reach."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1008_2849_gb300 import inputs
+from tests.gpu_util import oracle_sort, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+# Words of the control block (rs_device.cuh).
+CHUNKS, MSD_TILES, LSD_TILES, STEP, SRC = 25, 26, 27, 29, 30
+
+
+@pytest.fixture(scope="module")
+def rs():
+    from paper_1008_2849_gb300 import build, rs as _rs
+    build.build_library()
+    _rs.lib()
+    return _rs
+
+
+def _ctrl(ws):
+    return ws[:128].cpu().numpy().view(np.uint32)
+
+
+def _workspace(nbytes):
+    import torch
+    raw = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
+    pad = -raw.data_ptr() % 256
+    return raw[pad:pad + nbytes]
+
+
+def _words(rng, n, bits):
+    return rng.integers(0, 1 << bits, n, dtype=np.uint64).astype(
+        np.uint32 if bits == 32 else np.uint64)
+
+
+def _keys(kind, n, bits, seed):
+    rng = np.random.default_rng(seed)
+    name, _, count = kind.partition(" ")
+    if name == "distinct":
+        return _words(rng, int(count), bits)[rng.integers(0, int(count), n)]
+    if name == "prefixes":  # of the upper half of the bits
+        high = _words(rng, int(count), bits)[rng.integers(0, int(count), n)]
+        half = bits // 2
+        return (high >> half << half) | (_words(rng, n, bits) >> half)
+    k = _words(rng, n, bits)
+    if name == "hot":  # `count` in 1000 items have one key
+        k[rng.random(n) < float(count) / 1000] = k[0]
+    return k
+
+
+def _sort32(rs, k):
+    v = inputs.index_values(k.size)
+    ws = rs.alloc_workspace(k.size, True)
+    kd, vd = to_dev(k), to_dev(v)
+    rs.sort_pairs_ex(kd, vd, ws)
+    rs.check_stream()
+    ko, vo = oracle_sort(k, v)
+    assert np.array_equal(to_host(kd), ko) and np.array_equal(to_host(vd), vo)
+    return _ctrl(ws)
+
+
+def _sort64(rs, k, key_type="u64"):
+    import torch
+    ws = _workspace(rs.workspace_bytes_kv(k.size, key_type, 32))
+    v = np.arange(k.size, dtype=np.uint32)
+    kd, vd = torch.from_numpy(k.view(np.int64)).cuda(), to_dev(v)
+    rs.sort_kv_ex(kd, vd, key_type, ws)
+    rs.check_stream()
+    ko, vo = oracle.sort_kv(k, v, key_type)
+    assert np.array_equal(kd.cpu().numpy().view(np.uint64), ko)
+    assert np.array_equal(to_host(vd), vo)
+    return _ctrl(ws)
+
+
+@pytest.mark.parametrize("n", [1 << 25, 1 << 26])
+@pytest.mark.parametrize("kind", ["distinct 5000", "distinct 16000", "distinct 40000",
+                                  "distinct 1000000", "prefixes 3000", "prefixes 30000", "hot 4"])
+def test_32_bit_keys_that_crowd_are_refused(rs, n, kind):
+    assert _sort32(rs, _keys(kind, n, 32, n % 97 + len(kind)))[CHUNKS] == 0
+
+
+@pytest.mark.parametrize("kind", ["distinct 12000000", "uniform"])
+def test_32_bit_keys_that_spread_are_taken(rs, kind):
+    assert _sort32(rs, _keys(kind, 1 << 25, 32, 3))[CHUNKS] > 0
+
+
+@pytest.mark.parametrize("n,kind", [(1 << 22, "distinct 5000"), (1 << 24, "distinct 16000"),
+                                    (1 << 24, "distinct 40000"), (1 << 24, "prefixes 1500"),
+                                    (1 << 22, "hot 6")])
+def test_64_bit_keys_that_crowd_are_refused(rs, n, kind):
+    assert _sort64(rs, _keys(kind, n, 64, 11))[CHUNKS] == 0
+
+
+@pytest.mark.parametrize("n", [1 << 14, 100_003, (1 << 20) + 5, 4_500_003])
+def test_orders_of_64_bit_keys(rs, n):
+    c = _sort64(rs, _keys("uniform", n, 64, 5))
+    assert c[CHUNKS] > 0 and c[STEP] == 0 and c[SRC] == 0     # two passes, by prefix
+    k = np.random.default_rng(n).standard_normal(n).view(np.uint64)
+    c = _sort64(rs, k, "f64")                                  # by position
+    passes = int((c[1:9] > 0).sum())
+    assert c[CHUNKS] > 0 and c[STEP] > 0 and c[SRC] == passes % 2 and 2 <= passes <= 4
+
+
+@pytest.mark.parametrize("full", [True, False])
+def test_orders_of_segments(rs, full):
+    """Uniform segments take one pass and runs, one of equal digits the four passes; all do
+    in a workspace without the parts for the former."""
+    import torch
+    sizes = np.array([20_000, 50_000, 300_000, 5000], dtype=np.uint64)
+    off = inputs.offsets_from_sizes(sizes)
+    n = int(off[-1])
+    k = inputs.keys("uniform", n, 9)
+    k[int(off[1]):int(off[2])] &= np.uint32(0xFFFF)  # digits 3 and 2 are the same
+    v = inputs.index_values(n)
+    nbytes = rs.workspace_bytes(n, True, sizes.size)
+    if not full:  # the size before the parts of the routes: a geometry and a run list less
+        tiles = -(-n // 4096) + min(sizes.size, n // 4097 + 1)
+        runs = (n // 512 + 2 * min(sizes.size, n // 4097 + 1) + 2) * 8
+        nbytes -= -(-tiles * 16 // 256) * 256 + -(-runs // 256) * 256
+    ws = _workspace(nbytes)
+    kd, vd = to_dev(k), to_dev(v)
+    rs.sort_pairs_segmented_ex(kd, vd, to_dev(off), ws)
+    rs.check_stream()
+    ko, vo = oracle.sort_pairs_segmented(k, v, off)
+    assert np.array_equal(to_host(kd), ko) and np.array_equal(to_host(vd), vo)
+    c = _ctrl(ws)
+    assert (c[MSD_TILES] > 0) == full and (c[LSD_TILES] > 0) == full
+    torch.cuda.empty_cache()
