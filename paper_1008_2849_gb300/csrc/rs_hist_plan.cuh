@@ -389,13 +389,15 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
             uint32_t found = 0;
 #pragma unroll
             for (uint32_t q = 0; q < PER; ++q) {
-                const unsigned long long h = (unsigned long long)k[q] * 0x9E3779B97F4A7C15ull;
+                unsigned long long h = (unsigned long long)k[q] * 0x9E3779B97F4A7C15ull;
+                h = (h ^ h >> 32) * 0xD6E8FEB86659FD93ull;
                 const uint32_t word = NPASS == 4 ? (uint32_t)k[q] : (uint32_t)(h >> 32);
                 if (q * 1024 + tid >= samples || word == EMPTY) continue;
                 uint32_t at = (uint32_t)(h >> 16) & (slots - 1);
                 uint32_t was = atomicCAS(&slot[at], EMPTY, word);
+                // At most half of the slots are taken; a key that finds none is left out.
 #pragma unroll 1
-                while (was != EMPTY && was != word) {  // at most half of the slots are taken
+                for (uint32_t tries = 0; was != EMPTY && was != word && tries < 32; ++tries) {
                     at = (at + 1) & (slots - 1);
                     was = atomicCAS(&slot[at], EMPTY, word);
                 }

@@ -51,6 +51,9 @@ def _keys(kind, n, bits, seed):
         half = bits // 2
         return (high >> half << half) | (_words(rng, n, bits) >> half)
     k = _words(rng, n, bits)
+    if name == "and4":  # words that differ in few bits
+        for _ in range(3):
+            k &= _words(rng, n, bits)
     if name == "hot":  # `count` in 1000 items have one key
         k[rng.random(n) < float(count) / 1000] = k[0]
     return k
@@ -97,6 +100,28 @@ def test_32_bit_keys_that_spread_are_taken(rs, kind):
                                     (1 << 22, "hot 6")])
 def test_64_bit_keys_that_crowd_are_refused(rs, n, kind):
     assert _sort64(rs, _keys(kind, n, 64, 11))[CHUNKS] == 0
+
+
+@pytest.mark.parametrize("bits,n", [(64, 1 << 22), (64, 5_000_011), (32, 1 << 25)])
+def test_keys_that_differ_in_few_bits(rs, bits, n):
+    """The plan's table of sampled keys has to spread such keys too: 64-bit ones took
+    linear probes of some hundred slots each, 0.4 ms of the plan's one CTA."""
+    import torch
+    k = _keys("and4", n, bits, 21)
+    (_sort64 if bits == 64 else _sort32)(rs, k)
+    ws = _workspace(rs.workspace_bytes_kv(n, "u%d" % bits, 32))
+    src = torch.from_numpy(k.view(np.int64 if bits == 64 else np.int32)).cuda()
+    kd, vd = src.clone(), torch.arange(n, dtype=torch.int32, device="cuda")
+    rs.profile_enable(True)
+    try:
+        for _ in range(4):
+            kd.copy_(src)
+            rs.sort_kv_ex(kd, vd, "u%d" % bits, ws)
+        torch.cuda.synchronize()
+        launches, ms = rs.profile_read()["plan"]
+    finally:
+        rs.profile_enable(False)
+    assert launches == 4 and ms / launches < 0.1
 
 
 @pytest.mark.parametrize("n", [1 << 14, 100_003, (1 << 20) + 5, 4_500_003])
