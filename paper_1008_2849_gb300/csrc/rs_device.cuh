@@ -289,4 +289,37 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
+// f(i) for i = first, first + step, ... below end; COLD: never unrolled, to keep code short.
+template <bool COLD, typename F>
+__device__ __forceinline__ void loop(uint32_t first, uint32_t end, uint32_t step, F&& f) {
+    if constexpr (COLD) {
+#pragma unroll 1
+        for (uint32_t i = first; i < end; i += step) f(i);
+    } else {
+        for (uint32_t i = first; i < end; i += step) f(i);
+    }
+}
+
+// One slot of a warp's stable ranking by digit d: how many items before this lane's have
+// its digit, by the warp's counter row and its peer masks (zero between slots; warp-private
+// both).  By ballots, in a loop whose end the compiler cannot tell to be the same for a
+// warp's lanes, a slot takes three times the code.
+__device__ __forceinline__ uint32_t rank_slot(uint32_t d, bool live, uint32_t* row,
+                                              uint32_t* mask, uint32_t lane, uint32_t lt) {
+    if (live) atomicOr(&mask[d], 1u << lane);
+    __syncwarp();
+    uint32_t before = 0, peers = 0;
+    if (live) {
+        before = row[d];
+        peers = mask[d];
+    }
+    __syncwarp();
+    if (live && (peers & lt) == 0) {  // the first of them
+        row[d] = before + __popc(peers);
+        mask[d] = 0;
+    }
+    __syncwarp();
+    return before + __popc(peers & lt);
+}
+
 }  // namespace rs

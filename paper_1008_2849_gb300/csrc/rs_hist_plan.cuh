@@ -299,7 +299,8 @@ constexpr size_t top_plan_smem(uint32_t n, uint32_t top_bits, bool key64) {
 }
 constexpr size_t TOP_PLAN_SMEM = sizeof(uint16_t) << TOP_MAX_BITS;
 static_assert(TOP_PLAN_SMEM >= 10 * TOP_MAX_SAMPLES, "the table too");
-template <int NPASS>
+// TOP: the top-digits order may be chosen (without it the kernel is 4 KB of code, not 20).
+template <int NPASS, bool TOP>
 __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     extern __shared__ uint4 s_dyn[];
     static_assert(NPASS == 4 || NPASS == 8, "32-bit or 64-bit keys");
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t b = tid & (RADIX - 1);
     Ctrl* const ctrl = plan.ctrl;
-    const uint32_t n = plan.n, top_bits = plan.top_bits;
+    const uint32_t n = plan.n, top_bits = TOP ? plan.top_bits : 0u;
     pdl_launch_next();
     pdl_wait();  // the histograms are complete
     if (tid < NPASS) s_trivial[tid] = 0;
@@ -348,7 +349,7 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     bool top = !msd && top_bits != 0 && !s_uneven && executed >= 3;
     const bool deep = NPASS == 8 && top_bits != 0 && executed >= 4;
     uint32_t low = 0;  // the lowest digit with a pass
-    if (top || deep) {  // the same for every thread
+    if constexpr (TOP) if (top || deep) {  // the same for every thread
         uint32_t* const s_pair = reinterpret_cast<uint32_t*>(s_dyn);  // two 16-bit counts a word
         const K* const keys = static_cast<const K*>(plan.keys);
         constexpr uint32_t PER = NPASS == 4 ? TOP_MAX_SAMPLES / 1024 : 4;

@@ -160,6 +160,14 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
     constexpr uint32_t EARLY_PER = EARLY_CAP < EARLY_FIT ? EARLY_CAP : EARLY_FIT;
     constexpr uint32_t EARLY = EARLY_PER * FREE;
     constexpr uint32_t LATE_PER = (TILE - EARLY + THREADS - 1) / THREADS;
+    // Instruction caches hold about 128 KB, which the kernels of a sort share: what exceeds
+    // them is read again at the start of every pass (0.3 us a KB and sort, up to 17 us).  In
+    // the longer tile shapes, code that runs for the last tile only is therefore kept in
+    // loops (LOOPS), and the stores of pairs go by STORE_UNROLL slots: 60 KB instead of 105
+    // for pairs, 54 instead of 83 for keys.  2^27 pairs of ANDs of three words, which launch
+    // the on-chip sort in vain: 3188 us a call before, 3164 now, 3161 without that launch.
+    constexpr bool LOOPS = ITEMS > 8;
+    constexpr int STORE_UNROLL = PAIRS && LOOPS ? 13 : 64;
     static_assert(L::BYTES + 4096 <= 232448, "shared memory plan exceeds one CTA's limit");
 
     extern __shared__ uint4 s_dyn[];
@@ -229,8 +237,8 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
         if (status_clear != nullptr &&
             (ctrl->dir[slot + 1] != DIR_SKIP ||
              (slot + 1 == PASSES - 1 && ctrl->dir[MSD_SLOT] != DIR_SKIP)))
-            for (uint32_t i = blockIdx.x * THREADS + tid; i < clear_words; i += gridDim.x * THREADS)
-                status_clear[i] = 0;
+            loop<LOOPS>(blockIdx.x * THREADS + tid, clear_words, gridDim.x * THREADS,
+                        [&](uint32_t i) { status_clear[i] = 0; });
         return;
     }
     // Typed keys: map on reading in the first executed pass, back on storing
@@ -297,15 +305,12 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
         const uint32_t tail = a0 + nb;          // [tail, valid) when there is a bulk part
         if (nb < valid) {  // CTA-uniform
             bool issued = false;
-            for (uint32_t i = tid; i < head; i += THREADS) {
+            auto one = [&](uint32_t i) {
                 cp_async_elem(to + i, from + i);
                 issued = true;
-            }
-            if (nb)
-                for (uint32_t i = tail + tid; i < valid; i += THREADS) {
-                    cp_async_elem(to + i, from + i);
-                    issued = true;
-                }
+            };
+            loop<LOOPS>(tid, head, THREADS, one);
+            if (nb) loop<LOOPS>(tail + tid, valid, THREADS, one);
             if (issued) cp_async_mbar_arrive(bar);
             __syncthreads();  // every pending count is raised before the arrival below
         }
@@ -463,7 +468,8 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
         // ---- 2. rank, and stage the keys ------------------------------------
         uint32_t* const cnt = s_wcnt + warp * RADIX;
         uint32_t* const mask = smem + L::MASK + warp * RADIX;
-        uint32_t pos[ITEMS];
+        constexpr bool KEPT_POS = PAIRS && !PACKED;  // values are staged after the keys
+        uint32_t pos[KEPT_POS ? ITEMS : 1];
         auto rank_tile = [&](auto full) {
             constexpr bool FULL = decltype(full)::value;
             const uint32_t left = FULL ? WARP_ITEMS : (valid > wofs ? valid - wofs : 0u);
@@ -473,14 +479,31 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
                 uint32_t before = 0;
                 if (lane == first) before = atomicAdd(&cnt[d], (uint32_t)__popc(peers));
                 before = __shfl_sync(0xffffffffu, before, first & 31u);
-                pos[j] = before + __popc(peers & lt);
+                const uint32_t at = before + __popc(peers & lt);
+                if constexpr (KEPT_POS) pos[j] = at;
                 if constexpr (PACKED) {
-                    if (is_live) s_stage2[pos[j]] = make_uint2((uint32_t)k, val);
+                    if (is_live) s_stage2[at] = make_uint2((uint32_t)k, val);
                 } else {
-                    if (is_live) s_stage[pos[j]] = k;
+                    if (is_live) s_stage[at] = k;
                 }
             };
             const V* const vals = in_v + wofs + lane;
+            if constexpr (!FULL && !KEPT_POS && LOOPS) {
+                // The last tile of an array or segment: slot by slot, in a loop.
+#pragma unroll 6
+                for (int j = 0; j < ITEMS; ++j) {
+                    const bool is_live = j * 32 + lane < left;
+                    const K k = is_live ? read_key(keys[j * 32]) : K(0);
+                    const uint32_t val = PACKED && is_live ? (uint32_t)vals[j * 32] : 0u;
+                    const uint32_t at = rank_slot(digit_of(k), is_live, cnt, mask, lane, lt);
+                    if constexpr (PACKED) {
+                        if (is_live) s_stage2[at] = make_uint2((uint32_t)k, val);
+                    } else {
+                        if (is_live) s_stage[at] = k;
+                    }
+                }
+                return;
+            }
             K nk0 = read_key(keys[0]);
             K nk1 = ITEMS > 1 ? read_key(keys[32]) : K(0);
             uint32_t nv0 = PACKED ? (uint32_t)vals[0] : 0u;
@@ -612,8 +635,8 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
             if (SPARE) {
                 if (warp >= LB_WARPS) {
                     wait_bar(buf ^ 1);
-                    for (uint32_t w = warp - LB_WARPS; w < WARPS; w += WARPS - LB_WARPS)
-                        count_slots_of(buf ^ 1, ngeo, w);
+                    loop<LOOPS>(warp - LB_WARPS, WARPS, WARPS - LB_WARPS,
+                                [&](uint32_t w) { count_slots_of(buf ^ 1, ngeo, w); });
                 } else {
                     phase ^= 1u << (buf ^ 1);  // the count warps waited for it
                 }
@@ -668,13 +691,14 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
                     }
                 }
             };
+            constexpr int UNROLL = FULL ? STORE_UNROLL : LOOPS ? 8 : 64;
             if constexpr (FREE > 0) {
                 if (tid >= RADIX) {
-#pragma unroll
+#pragma unroll UNROLL
                     for (uint32_t k = 0; k < EARLY_PER; ++k) store_slot(k * FREE + (tid - RADIX));
                 }
             }
-#pragma unroll
+#pragma unroll UNROLL
             for (uint32_t k = 0; k < LATE_PER; ++k) {
                 const uint32_t s = EARLY + k * THREADS + tid;
                 if ((TILE - EARLY) % THREADS == 0 || s < TILE) store_slot(s);

@@ -111,14 +111,17 @@ rs_status enqueue_hist4(const uint32_t* keys, uint32_t n, uint32_t* hist, void* 
 
 template <int NPASS>
 rs_status enqueue_plan(const PlanArgs& plan, cudaStream_t stream) {
-    static DeviceOnce smem_set;
-    const rs_status st = allow_smem_once(k_plan<NPASS>, TOP_PLAN_SMEM, smem_set);
-    if (st != RS_OK) return st;
-    const size_t smem =
-        plan.top_bits ? top_plan_smem(plan.n, plan.top_bits, NPASS == PASSES64) : 0;
+    const bool top = plan.top_bits != 0;
+    auto kern = top ? k_plan<NPASS, true> : k_plan<NPASS, false>;
+    size_t smem = 0;
+    if (top) {
+        static DeviceOnce smem_set;
+        const rs_status st = allow_smem_once(kern, TOP_PLAN_SMEM, smem_set);
+        if (st != RS_OK) return st;
+        smem = top_plan_smem(plan.n, plan.top_bits, NPASS == PASSES64);
+    }
     note_launch_begin(KK_PLAN, stream);
-    const cudaError_t e =
-        launch_after_previous(k_plan<NPASS>, dim3(1), dim3(1024), smem, stream, plan);
+    const cudaError_t e = launch_after_previous(kern, dim3(1), dim3(1024), smem, stream, plan);
     note_launch_end(KK_PLAN, stream);
     return e == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
