@@ -120,7 +120,7 @@ rs_status enqueue_sort_segmented(uint32_t* keys, uint32_t* vals, uint32_t n,
     // Each large segment takes the MSD-first order or the four passes.
     const bool routed = ck.msd != 0 && workspace_bytes >= L.routed_total;
     const SegRoute route{routed ? reinterpret_cast<uint4*>(ws + L.route_geo) : nullptr,
-                         reinterpret_cast<uint2*>(ws + L.runs), L.max_tiles, tile};
+                         reinterpret_cast<uint2*>(ws + L.runs), L.max_tiles, tile, pairs};
     const cudaError_t se = launch_after_previous(k_seg_scan<PASSES>, dim3(di.sm_count * 2),
                                                  dim3(1024), 0, stream, ctrl, gofs,
                                                  (const uint32_t*)large_first, route);

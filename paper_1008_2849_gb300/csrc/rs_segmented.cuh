@@ -237,10 +237,14 @@ k_seg_hist(const uint32_t* __restrict__ keys, const Ctrl* __restrict__ ctrl,
 // digit 3 takes more than one value and no bucket of it holds more than
 // MSD_SEG_BUCKET items, one pass by digit 3 into the alternate buffers, then runs
 // of its buckets sorted on chip back into the caller's arrays; else the four
-// passes.  Segments of the first kind get tiles 0 .. msd_tiles - 1 of route.geo,
-// the others the lsd_tiles last ones; route.chunks lists (first item, items) of
-// the runs: the buckets that start in the same stretch of CAPACITY - (largest
-// bucket) items, CAPACITY in all at most.
+// passes.  Key-value segments whose digit 1 or 2 crowds (a bucket over four times its
+// share) take the passes too: the on-chip sorts of their runs would take theirs (4096
+// segments of 256 to 65536 pairs, ANDs of two words: 1670 us on chip, 1355 by the four
+// passes; 256 distinct keys: 1480 and 1279; keys alone: 1204 and 1138, but 885 and 1136).
+// Segments of the first kind get tiles 0 .. msd_tiles - 1 of route.geo, the others the
+// lsd_tiles last ones; route.chunks lists (first item, items) of the runs: the buckets
+// that start in the same stretch of CAPACITY - (largest bucket) items, CAPACITY in all
+// at most.
 // ---------------------------------------------------------------------------
 constexpr uint32_t MSD_SEG_CAPACITY = SMALL_MID_MAX;  // of the on-chip sort
 constexpr uint32_t MSD_SEG_BUCKET = MSD_SEG_CAPACITY - 512;  // so a stretch is 512 items or more
@@ -249,6 +253,7 @@ struct SegRoute {
     uint4* geo;
     uint2* chunks;
     uint32_t max_tiles, tile;
+    bool pairs;
 };
 
 template <int NP = PASSES>
@@ -257,7 +262,7 @@ k_seg_scan(Ctrl* __restrict__ ctrl, uint32_t* __restrict__ hist,
            const uint32_t* __restrict__ large_first, const SegRoute route) {
     static_assert(NP == 4 || NP == 8, "32-bit or 64-bit keys");
     __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_max[RADIX / 32], s_runs[RADIX / 32];
+    __shared__ uint32_t s_max[PASSES * RADIX / 32], s_runs[RADIX / 32];  // by warps
     __shared__ uint32_t s_start[RADIX];      // first items of digit 3's buckets
     __shared__ uint32_t s_first[RADIX + 1];  // first items of the runs, and the segment's end
     __shared__ uint32_t s_base[2];           // first tile, first run
@@ -279,7 +284,7 @@ k_seg_scan(Ctrl* __restrict__ ctrl, uint32_t* __restrict__ hist,
         }
         if (lane == 31) s_warp[warp] = x;
         const uint32_t most = __reduce_max_sync(0xffffffffu, v);
-        if (p == PASSES - 1 && lane == 0) s_max[warp & 7] = most;
+        if (lane == 0) s_max[warp] = most;
         __syncthreads();
         uint32_t offv = 0;
         for (uint32_t w = p * (RADIX / 32); w < warp; ++w) offv += s_warp[w];
@@ -287,12 +292,19 @@ k_seg_scan(Ctrl* __restrict__ ctrl, uint32_t* __restrict__ hist,
         const uint32_t start = offv + x - v;
         h[tid] = lo + start;
         if (NP == 4 && route.geo != nullptr) {
-            uint32_t size = 0, biggest = 0;
-            for (uint32_t w = 0; w < RADIX / 32; ++w) {
+            constexpr uint32_t W = RADIX / 32;  // warps of a digit
+            uint32_t size = 0, biggest = 0, big1 = 0, big2 = 0;
+            for (uint32_t w = 0; w < W; ++w) {
                 size += s_warp[w];  // digit 0 counts every item
-                biggest = max(biggest, s_max[w]);
+                biggest = max(biggest, s_max[(PASSES - 1) * W + w]);
+                big1 = max(big1, s_max[W + w]);
+                big2 = max(big2, s_max[2 * W + w]);
             }
-            const bool msd = biggest <= MSD_SEG_BUCKET && biggest < size;
+            // (A digit that is the same in all says nothing about the others.)
+            const uint32_t crowd = size / RADIX * 4;
+            const bool crowded = route.pairs && ((big1 > crowd && big1 < size) ||
+                                                 (big2 > crowd && big2 < size));
+            const bool msd = biggest <= MSD_SEG_BUCKET && biggest < size && !crowded;
             const uint32_t b = tid & (RADIX - 1);
             if (p == PASSES - 1) s_start[b] = start;
             __syncthreads();

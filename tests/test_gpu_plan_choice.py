@@ -159,3 +159,33 @@ def test_orders_of_segments(rs, full):
     c = _ctrl(ws)
     assert (c[MSD_TILES] > 0) == full and (c[LSD_TILES] > 0) == full
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("kind", ["distinct 256", "and4"])
+@pytest.mark.parametrize("pairs", [True, False])
+def test_orders_of_crowded_segments(rs, kind, pairs):
+    """Pairs of segments whose middle digits crowd take the four passes; segments whose
+    other digits are the same in all their keys are not crowded."""
+    sizes = np.array([20_000, 4097, 60_000, 9000], dtype=np.uint64)
+    off = inputs.offsets_from_sizes(sizes)
+    n = int(off[-1])
+    k = _keys(kind, n, 32, 3)
+    if kind == "and4":  # but in the top digit, so that no bucket of it is too large
+        k = (k & np.uint32(0x00FFFFFF)) | (_words(np.random.default_rng(4), n, 32)
+                                           & np.uint32(0xFF000000))
+    same = slice(int(off[0]), int(off[1]))
+    k[same] = _keys("uniform", 20_000, 32, 6) & np.uint32(0xFF0000FF)
+    v = inputs.index_values(n)
+    ws = _workspace(rs.workspace_bytes(n, pairs, sizes.size))
+    kd, vd = to_dev(k), to_dev(v)
+    if pairs:
+        rs.sort_pairs_segmented_ex(kd, vd, to_dev(off), ws)
+    else:
+        rs.sort_keys_segmented_ex(kd, to_dev(off), ws)
+    rs.check_stream()
+    ko, vo = oracle.sort_pairs_segmented(k, v, off)
+    assert np.array_equal(to_host(kd), ko)
+    if pairs:
+        assert np.array_equal(to_host(vd), vo)
+    c = _ctrl(ws)
+    assert c[MSD_TILES] > 0 and (c[LSD_TILES] > 0) == pairs
