@@ -51,13 +51,20 @@ rs_status run(K* keys, V* vals, K* spare_keys, V* spare_vals, uint32_t n, const 
 #define RS_CHUNKS(T, B)                                                                     \
     return launch_chunks<K, V, PAIRS, T, B>(keys, vals, spare_keys, spare_vals, off, ctrl,  \
                                             top.bits, key_type, di.sm_count, stream)
+    // The shapes that the orders below can ask for: 32-bit items from 2^25 on have larger
+    // chunks, wide ones 4608 items at most, and only 64-bit keys come in small arrays.
     constexpr bool WIDE = sizeof(K) == 8 || (PAIRS && sizeof(V) == 8);
-    if constexpr (WIDE) {  // the 32-bit sorts take chunks of the larger sizes only
+    if constexpr (sizeof(K) == 8) {
         if (top.capacity <= 1024) RS_CHUNKS(128, 8);
+    }
+    if constexpr (WIDE) {
         if (top.capacity <= 2560) RS_CHUNKS(320, 3);
     }
     if (top.capacity <= 4608) RS_CHUNKS(576, 2);
-    RS_CHUNKS(1024, 1);
+    if constexpr (!WIDE) {
+        if (top.capacity <= 8192) RS_CHUNKS(1024, 1);
+    }
+    return RS_ERR_UNSUPPORTED;  // no shape for it: not reached
 #undef RS_CHUNKS
 }
 
