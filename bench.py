@@ -564,7 +564,7 @@ def main():
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u32",
             "data": "synthetic",
             "config": {"workload": WORKLOAD, "n": n, "key_dist": "uniform", "seed": KEY_SEED,
-                       "values": "index", "passes": 4, "digit_bits": 8,
+                       "values": "index", "passes": roof["scatter_passes"], "digit_bits": 8,
                        "l2": "inputs larger than L2: every step sorts its own fresh 2 GiB copy",
                        "parallelism": "replicas" if world > 1 else "single GPU"},
             "roofline": roof, "e2e": e2e, "cpu_baseline": cpu,

@@ -108,11 +108,11 @@ size_t rs_workspace_bytes_digits11(size_t n, int with_values);
  * d_offsets[num_segments]) are left as they are; a single segment must hold
  * fewer than 2^30 items.  A table that breaks these rules is detected on the
  * device: nothing is written and the status is RS_ERR_BAD_SEGMENTS.
- * Segments of at most 512 items (the RS_TUNE_WARP_MAX setting) are sorted
- * by one warp each, segments of at most 4096 items (or the RS_TUNE_SMALL_MAX
- * setting, up to 8192) by one CTA each, both in shared memory; larger ones by
- * the four scatter passes of the unsegmented sort, all large segments
- * together.
+ * Segments of at most 4096 items (or the RS_TUNE_SMALL_MAX setting, up to
+ * 8192) are sorted by one CTA each in shared memory, those of at most 512 (the
+ * RS_TUNE_WARP_MAX setting) by a CTA of two warps; larger ones by scatter
+ * passes, all large segments together: one pass by the highest digit and its
+ * buckets on chip where they fit (RS_TUNE_MSD), else four.
  * Plain forms are synchronous; _ex forms as above, with
  * workspace_bytes >= rs_workspace_bytes(n, with_values, num_segments). */
 rs_status rs_sort_keys_segmented(uint32_t* d_keys, size_t n, const uint32_t* d_offsets,
@@ -189,7 +189,7 @@ size_t rs_workspace_bytes64(size_t n, int with_values);
  * 32-bit keys with no or 32-bit values take the calls above (same workspace
  * size, same kernels); every other combination sorts arrays of up to 4096 items
  * on chip in one launch, and longer ones by the scatter passes, or by the highest
- * digits first and on chip from there where the keys allow it.
+ * digits first and on chip from there where the keys allow it (RS_TUNE_MSD).
  * d_keys is aligned to its key width, d_vals to its value width; keys and
  * values do not overlap; n < 2^32; workspace_bytes >=
  * rs_workspace_bytes_kv(n, key_type, value_bits), the workspace 256-byte
@@ -373,17 +373,20 @@ typedef enum rs_tune_knob {
                                      one-CTA shared-memory sort; segments up to 4096 always
                                      take an on-chip sort */
     RS_TUNE_TILE_SEG = 5,         /* tile shape index of the segmented scatter passes */
-    RS_TUNE_WARP_MAX = 6,         /* segments up to this size (<= 512)
-                                     take the one-warp shared-memory sort; 0 turns it off */
-    RS_TUNE_SMALL_BITS = 7,       /* on-chip sorts: 8 (the default), the one-warp sort in four
-                                     8-bit passes and the one-CTA bin sort; 4, both in eight
-                                     4-bit passes */
-    RS_TUNE_MSD = 8,              /* 1 (the default): whole arrays may take the MSD-first order
-                                     of Alg. 2 (one pass by the top digit, then every bucket
-                                     sorted on chip) where the buckets fit a CTA, or from 2^25
-                                     items the top-digits order (two passes by the two highest
-                                     digits, then chunks sorted on chip) where the keys spread
-                                     evenly; 0: always the LSD passes */
+    RS_TUNE_WARP_MAX = 6,         /* segments up to this size (<= 512) are listed apart, for
+                                     CTAs of two warps (one warp a segment with
+                                     RS_TUNE_SMALL_BITS 4); 0: they take the larger CTAs */
+    RS_TUNE_SMALL_BITS = 7,       /* on-chip sorts: 8 (the default), the bin sort; 4, eight
+                                     4-bit counting passes */
+    RS_TUNE_MSD = 8,              /* 1 (the default): the highest digits may go first, where
+                                     the keys spread and what is left fits a CTA.  32-bit arrays
+                                     of up to 1,894,400 items, and segments above 4096: one pass
+                                     by the top digit, then its buckets on chip (the MSD-first
+                                     order of Alg. 2).  From 2^25 items (up to 495,976,448; with
+                                     64-bit values 271,187,968): two passes, then chunks on chip.
+                                     64-bit arrays of 2^14 to 271,187,968 items: two to four
+                                     passes, then chunks on chip.  0: always the LSD passes,
+                                     for large segments too */
     RS_TUNE_TYPED_SPLIT = 9       /* signed and float keys: sorts of at least this many items
                                      launch two instances of every scatter pass (the passes that
                                      need no key map run without it, at the unsigned speed);

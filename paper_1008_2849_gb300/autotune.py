@@ -6,9 +6,11 @@ captured CUDA graphs (rs_graph_*) of a representative synthetic workload
 under every candidate setting and keeps the fastest:
 
 * whole arrays: the tile shape of the scatter passes, for key-value and for
-  keys-only sorts; the MSD-first order of Alg. 2 (one pass by the top digit,
-  then on-chip bucket sorts; from 2^25 items two passes and on-chip chunks) or
-  the four LSD passes; from 2^24 items, four passes of 8-bit digits or three of 11/11/10 bits; for
+  keys-only sorts, on the four LSD passes (what keys that crowd take at every
+  size; the orders by the top digits run the same shapes once or twice); the
+  MSD-first order of Alg. 2 (one pass by the top digit, then on-chip bucket
+  sorts; from 2^25 items two passes and on-chip chunks) or the four LSD passes;
+  from 2^24 items, four passes of 8-bit digits or three of 11/11/10 bits; for
   arrays up to 8192 items, which take the one-CTA sort, and at which digit
   width;
 * segmented batches: the tile shape of the segmented scatter passes and the

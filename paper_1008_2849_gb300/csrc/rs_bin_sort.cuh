@@ -54,8 +54,11 @@ struct BinSortSmem {
     static constexpr uint32_t CAP = THREADS * ITEMS;
     // Up to the power of two at or above CAP bins (chunks, whose words have no room
     // for more: 2048 or 4096), scanned by the largest power of two of threads.
-    static constexpr uint32_t BIN_BITS =
-        CAP <= 512 ? 9 : CAP <= 1024 ? 10 : CAP <= (CHUNKS ? 2560 : 2048) ? 11 : CHUNKS || CAP <= 4096 ? 12 : 13;
+    static constexpr uint32_t BIN_BITS = CAP <= 512                        ? 9
+                                         : CAP <= 1024                     ? 10
+                                         : CAP <= (CHUNKS ? 2560 : 2048)   ? 11
+                                         : CHUNKS || CAP <= 4096           ? 12
+                                                                           : 13;
     static constexpr uint32_t MAX_BINS = 1u << BIN_BITS;
     static constexpr uint32_t SCANNERS = THREADS >= 1024 ? 1024 : THREADS >= 512 ? 512
                                          : THREADS >= 256 ? 256

@@ -32,8 +32,8 @@ constexpr uint32_t DIR_SKIP = 0;   // every key has the same digit: identity
 constexpr uint32_t DIR_A_TO_B = 1; // caller's arrays -> alternate buffers
 constexpr uint32_t DIR_B_TO_A = 2; // alternate buffers -> caller's arrays
 
-// Per-call control block, zeroed by one cudaMemsetAsync at the start of a
-// call.  Lives at the start of the workspace.
+// Per-call control block, at the start of the workspace; k_clear_ctrl zeroes it
+// at the start of a call.
 // Plan slots: the LSD passes 0..7 (0..3 for 32-bit keys), and MSD_SLOT for
 // the most-significant-digit pass of the MSD-first order (Alg. 2): when the plan
 // chooses it, the passes 0..3 are all DIR_SKIP, and the launch of pass 3 runs it.

@@ -15,12 +15,13 @@ namespace rs {
 
 // ---------------------------------------------------------------------------
 // k_clear_ctrl: zeroes the control block, and `vecs` 16-byte words at `more` (the counts
-// of segments).  The histogram kernel after it is
-// its programmatic dependent, which reads the keys meanwhile and waits before it adds
-// to the counts.  With a memset in its place, and the histogram after that, a call takes 2
-// to 3 us more: 2^20 keys 39.2 us instead of 37.0, 50021 pairs 30.5 instead of 28.2.
+// of segments).  The histogram kernel after it is its programmatic dependent, which reads
+// the keys meanwhile and waits before it adds to the counts.  With a memset in its place,
+// and the histogram after that, a call takes 2 to 3 us more: 2^20 keys 39.2 us instead of
+// 37.0, 50021 pairs 30.5 instead of 28.2.
 // ---------------------------------------------------------------------------
-static __global__ void __launch_bounds__(1024) k_clear_ctrl(uint4* __restrict__ ctrl, uint4* __restrict__ more, size_t vecs) {
+static __global__ void __launch_bounds__(1024)
+k_clear_ctrl(uint4* __restrict__ ctrl, uint4* __restrict__ more, size_t vecs) {
     static_assert(sizeof(Ctrl) % sizeof(uint4) == 0, "whole vectors");
     pdl_launch_next();
     if (blockIdx.x == 0)

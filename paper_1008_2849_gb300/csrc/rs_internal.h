@@ -89,9 +89,10 @@ constexpr uint32_t kMsdShortItems = 256u * 4600u;
 constexpr uint32_t kMsdMaxItems = 256u * 7400u;
 // Large arrays may take the top-digits order: two scatter passes, then chunks of the
 // keys' `bits` highest bits sorted on chip by a CTA of `capacity` items (rs_chunks.cu).
-// bits = 0: not tried.  32-bit keys from kTopMinItems on (where the saved passes outweigh
-// what keys that do not spread pay for the launches: 18 us, 3 % of 2^25 keys), 64-bit
-// keys, which save six passes of eight, from kTopMinItems64.
+// bits = 0: not tried.  32-bit keys from kTopMinItems on (tried below, it took 382 us
+// instead of 389 for 2^24 pairs, but 574 instead of 538 for 24 million), 64-bit keys, which
+// save six passes of eight, from kTopMinItems64.  Above 495,976,448 items (271,187,968 wide
+// ones) the chunks of 16 bits no longer fit a CTA.
 constexpr uint32_t kTopMinItems = 1u << 25;
 constexpr uint32_t kTopMinItems64 = 1u << 14;
 struct TopOrder {

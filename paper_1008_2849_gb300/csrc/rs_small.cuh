@@ -147,8 +147,9 @@ k_warp_sort(uint32_t* keys, uint32_t* vals, const uint32_t* __restrict__ off,
 // items in shared memory: 32 / BITS stable counting-sort passes between two
 // shared buffers.  Arrays are the segments listed from `list` on (every
 // `step`-th entry; count in *list_count), with list == nullptr the
-// segments 0, 1, ..., with step == 0 the ranges (first item, items) in `list`, or with off == nullptr the single
-// array [0, single_n).  The 4-bit form only; 8-bit digits take k_bin_sort.
+// segments 0, 1, ..., with step == 0 the ranges (first item, items) in `list`,
+// or with off == nullptr the single array [0, single_n).  4-bit digits, for
+// RS_TUNE_SMALL_BITS = 4; the default is k_bin_sort.
 // Per pass: per-warp digit counts, their prefix over (digit, warp), then every
 // warp ranks its items slot by slot (peers from one ballot per digit bit,
 // positions from the warp's counters) and moves them to the other buffer.  A
