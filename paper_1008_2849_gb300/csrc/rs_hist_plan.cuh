@@ -272,10 +272,11 @@ __host__ __device__ constexpr uint32_t top_hot_limit(bool key64, uint32_t sample
     return samples / 4096 * (key64 ? 8 : 3);
 }
 // The most pairs of samples in one of 2^bits cells: four standard deviations over those of
-// even keys.
-__device__ __forceinline__ uint32_t top_pair_limit(uint32_t samples, uint32_t bits) {
+// even keys, and those of cells whose sizes deviate by `spread` of their mean.
+__device__ __forceinline__ uint32_t top_pair_limit(uint32_t samples, uint32_t bits,
+                                                   float spread = 0.0f) {
     const uint32_t even = (uint32_t)((unsigned long long)samples * samples / 2 >> bits);
-    return even + (uint32_t)(4.0f * sqrtf((float)even));
+    return even + (uint32_t)(4.0f * sqrtf((float)even) + spread * spread * (float)even);
 }
 
 // What the plan works on; bucket_cap and msd_off for the MSD-first order
@@ -286,7 +287,18 @@ struct PlanArgs {
     uint32_t n, key_type, bucket_cap;
     uint32_t* msd_off;
     uint32_t top_bits, chunk_step;
+    uint32_t capacity;  // items of a chunk that a CTA takes
 };
+
+// Chunks are cut by prefix, so they grow longer where the keys are denser, and the top
+// digit's histogram shows that better than a sample: this is how many items one of its
+// values may have for its 2^(bits - 8) chunks to fit a CTA.  With over a sixteenth of the
+// items in fuller ones an array takes the passes.  2^27 pairs whose density rises by 1.2, 1.5
+// and 4 times from the least to the greatest key: 2497, 3843 and 5335 us by chunks, 2895 by
+// the passes; 2^25 64-bit keys 1.2 and 2.1 times: 1184 and 2770 by prefix, 1128 by position.
+__device__ __forceinline__ uint32_t top_digit_most(uint32_t bits, uint32_t capacity) {
+    return (capacity - capacity / 64) << (bits - RADIX_BITS);
+}
 
 // Dynamic shared memory of k_plan when top_bits is set: two bytes for each cell of the
 // 2^top_bits or 2^TOP_HASH_BITS, and where repeated keys are looked for at least a table of
@@ -308,7 +320,7 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     using K = std::conditional_t<NPASS == 8, unsigned long long, uint32_t>;
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_trivial[NPASS];
-    __shared__ uint32_t s_big, s_uneven;
+    __shared__ uint32_t s_big, s_uneven, s_long;
     __shared__ uint32_t s_part[32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t b = tid & (RADIX - 1);
@@ -317,7 +329,7 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
     pdl_launch_next();
     pdl_wait();  // the histograms are complete
     if (tid < NPASS) s_trivial[tid] = 0;
-    if (tid == 0) s_big = s_uneven = 0;
+    if (tid == 0) s_big = s_uneven = s_long = 0;
     // Thread (p, b): p = tid / 256 (+ 4 in the second round for 64-bit keys).
     uint32_t first3 = 0;  // digit 3, for the MSD-first order
     for (uint32_t round = 0; round < NPASS / 4; ++round) {
@@ -341,13 +353,15 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
             if (h > plan.bucket_cap) s_big = 1;
         }
         if (p >= NPASS - 2 && h > n / RADIX * 2) s_uneven = 1;
+        if (TOP && p == NPASS - 1 && top_bits != 0 && h > top_digit_most(top_bits, plan.capacity))
+            atomicAdd(&s_long, h);
         __syncthreads();  // s_warp is reused by the next round
     }
     const bool msd =
         NPASS == 4 && plan.msd_off != nullptr && !s_trivial[PASSES - 1] && !s_big;
     uint32_t executed = 0;
     for (uint32_t q = 0; q < NPASS; ++q) executed += s_trivial[q] ? 0 : 1;
-    bool top = !msd && top_bits != 0 && !s_uneven && executed >= 3;
+    bool top = !msd && top_bits != 0 && !s_uneven && s_long <= n / 16 && executed >= 3;
     const bool deep = NPASS == 8 && top_bits != 0 && executed >= 4;
     uint32_t low = 0;  // the lowest digit with a pass
     if constexpr (TOP) if (top || deep) {  // the same for every thread
@@ -441,8 +455,10 @@ __global__ void __launch_bounds__(1024) k_plan(const PlanArgs plan) {
         }
         if (top) {
             low = NPASS - 2;
+            // Chunks may deviate by half of what a CTA takes over their mean.
+            const float room = (float)plan.capacity / (float)(n >> top_bits) - 1.0f;
             top = !repeat && spread(top_bits, 2 * (samples >> top_bits) + 12,
-                                    top_pair_limit(samples, top_bits), [&](K x) {
+                                    top_pair_limit(samples, top_bits, 0.5f * room), [&](K x) {
                                         return (uint32_t)(x >> (8 * sizeof(K) - top_bits));
                                     });
         }

@@ -203,7 +203,7 @@ rs_status enqueue_sort(uint32_t* keys, uint32_t* vals, uint32_t n, cudaStream_t 
     const TopOrder top = ck.msd != 0 ? top_order(n) : TopOrder{0, 0};
     uint32_t* msd_off = reinterpret_cast<uint32_t*>(ws + L.msd_off);
     const PlanArgs plan{ctrl, keys, n, key_type, bucket_capacity(long_buckets),
-                        msd ? msd_off : nullptr, top.bits, 0u};
+                        msd ? msd_off : nullptr, top.bits, 0u, top.capacity};
 
     st = enqueue_clear(ctrl, stream);
     if (st != RS_OK) return st;

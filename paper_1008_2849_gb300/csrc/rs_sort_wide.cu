@@ -138,7 +138,8 @@ rs_status enqueue_sort_wide(void* keys, void* vals, uint32_t n, uint32_t key_typ
     // Keys that spread evenly: two passes, then chunks on chip (see enqueue_sort).
     const TopOrder top = knobs().cls[size_class(n)].msd != 0 ? top_order_wide(n, key64)
                                                              : TopOrder{0, 0};
-    const PlanArgs plan{ctrl, keys, n, key_type, 0u, nullptr, top.bits, top.capacity / 2};
+    const PlanArgs plan{ctrl, keys, n, key_type, 0u, nullptr, top.bits, top.capacity / 2,
+                        top.capacity};
     st = key64 ? enqueue_plan<PASSES64>(plan, stream) : enqueue_plan<PASSES>(plan, stream);
     if (st != RS_OK) return st;
 

@@ -56,6 +56,11 @@ def _keys(kind, n, bits, seed):
             k &= _words(rng, n, bits)
     if name == "hot":  # `count` in 1000 items have one key
         k[rng.random(n) < float(count) / 1000] = k[0]
+    if name == "slope":  # denser towards the greatest key, by 1 - c to 1 + c of the mean
+        c = float(count) / 100
+        x = (np.sqrt((1 - c) ** 2 + 4 * c * rng.random(n)) - (1 - c)) / (2 * c)
+        high = np.minimum(x, 1 - 2.0 ** -53) * 2.0 ** 32
+        k = high.astype(np.uint32) if bits == 32 else (high.astype(np.uint64) << 32) | (k >> 32)
     return k
 
 
@@ -189,3 +194,26 @@ def test_orders_of_crowded_segments(rs, kind, pairs):
         assert np.array_equal(to_host(vd), vo)
     c = _ctrl(ws)
     assert c[MSD_TILES] > 0 and (c[LSD_TILES] > 0) == pairs
+
+
+@pytest.mark.parametrize("slope, taken", [(0.05, True), (0.35, False), (0.7, False)])
+def test_density_of_32_bit_keys(rs, slope, taken):
+    """2^25 keys whose chunks grow too long for a CTA where they are denser take the
+    passes."""
+    n = 1 << 25
+    k = _keys("slope %g" % (100 * slope), n, 32, 12)
+    ws = _workspace(rs.workspace_bytes(n, False))
+    kd = to_dev(k)
+    rs.sort_keys_ex(kd, ws)
+    rs.check_stream()
+    assert np.array_equal(to_host(kd), np.sort(k))
+    assert (_ctrl(ws)[CHUNKS] > 0) == taken
+
+
+@pytest.mark.parametrize("n, slope, by_prefix", [(1 << 18, 0.35, True), (1 << 22, 0.6, True),
+                                                 ((1 << 23) + 5, 0.9, False)])
+def test_density_of_64_bit_keys(rs, n, slope, by_prefix):
+    """Where a CTA takes far more than an even chunk, denser chunks fit too; else the keys
+    go by position."""
+    c = _sort64(rs, _keys("slope %g" % (100 * slope), n, 64, 13))
+    assert c[CHUNKS] > 0 and (c[STEP] == 0) == by_prefix
