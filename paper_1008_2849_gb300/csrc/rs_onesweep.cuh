@@ -167,7 +167,7 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
     // for pairs, 54 instead of 83 for keys.  2^27 pairs of ANDs of three words, which launch
     // the on-chip sort in vain: 3188 us a call before, 3164 now, 3161 without that launch.
     constexpr bool LOOPS = ITEMS > 8;
-    constexpr int STORE_UNROLL = PAIRS && LOOPS ? 13 : 64;
+    constexpr int STORE_UNROLL = PAIRS ? 13 : 64;
     static_assert(L::BYTES + 4096 <= 232448, "shared memory plan exceeds one CTA's limit");
 
     extern __shared__ uint4 s_dyn[];
@@ -691,14 +691,31 @@ k_onesweep(K* __restrict__ ka, V* __restrict__ va,
                     }
                 }
             };
-            constexpr int UNROLL = FULL ? STORE_UNROLL : LOOPS ? 8 : 64;
+            // (The other shapes without a count in the pragma: with 64 there, which unrolls as
+            // much, 60000 to 900000 pairs of ANDs of two words took 2 us more in four passes.)
+            constexpr int UNROLL = FULL ? STORE_UNROLL : 8;
+            if constexpr (LOOPS) {
+                if constexpr (FREE > 0) {
+                    if (tid >= RADIX) {
+#pragma unroll UNROLL
+                        for (uint32_t k = 0; k < EARLY_PER; ++k)
+                            store_slot(k * FREE + (tid - RADIX));
+                    }
+                }
+#pragma unroll UNROLL
+                for (uint32_t k = 0; k < LATE_PER; ++k) {
+                    const uint32_t s = EARLY + k * THREADS + tid;
+                    if ((TILE - EARLY) % THREADS == 0 || s < TILE) store_slot(s);
+                }
+                return;
+            }
             if constexpr (FREE > 0) {
                 if (tid >= RADIX) {
-#pragma unroll UNROLL
+#pragma unroll
                     for (uint32_t k = 0; k < EARLY_PER; ++k) store_slot(k * FREE + (tid - RADIX));
                 }
             }
-#pragma unroll UNROLL
+#pragma unroll
             for (uint32_t k = 0; k < LATE_PER; ++k) {
                 const uint32_t s = EARLY + k * THREADS + tid;
                 if ((TILE - EARLY) % THREADS == 0 || s < TILE) store_slot(s);
